@@ -96,6 +96,10 @@ __device__ __forceinline__ void ring_boxes(const MarkerArgs& a, int m, int n, in
 // advance launch has `nblocks` blocks in all (the last of them to finish runs
 // the epilogue): the single-context kernel runs unit blockIdx.x of gridDim.x,
 // the batched kernel (ensembles) one unit of one member per block.
+//
+// Everything but the velocities is read before dep_wait(): the positions,
+// forces, weights and bonds were complete when the fused kernel (the
+// predecessor in a chained launch) let this one start.
 template <typename C, bool DYN>
 __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigned nblocks) {
     using E = typename Ext<C>::E;
@@ -125,9 +129,12 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigne
         E x, y, xp, yp, xn, yn;
         load_pos<C>(a, v, x, y);
         PosIO<C>::load(a.Xp, v, xp, yp);
+        const Shape<C> sh = load_shape<C>(a, v);
+        dep_wait();
+        dep_trigger();
         if (valid) {
             C Ux, Uy;
-            interp_vertex<C>(a, v, Ux, Uy);
+            interp_vertex<C>(a, sh, Ux, Uy);
             U[2 * v] = Ux;
             U[2 * v + 1] = Uy;
             if (DYN && kind == LBIB_MEMBRANE_DYNAMIC) {
@@ -164,11 +171,15 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigne
         const C* F = static_cast<const C*>(a.F);
         E x, y;
         C Ux = 0, Uy = 0, ax = 0, ay = 0, bx = 0, by = 0, fx = 0, fy = 0;
+        E xq, yq;
+        const int kv = valid ? k : 0;
+        load_pos<C>(a, off + kv, x, y);
+        load_pos<C>(a, off + (kv + 1 == n ? 0 : kv + 1), xq, yq);
+        const Shape<C> sh = load_shape<C>(a, off + kv);
+        dep_wait();
+        dep_trigger();
         if (valid) {
-            E xq, yq;
-            load_pos<C>(a, off + k, x, y);
-            load_pos<C>(a, off + (k + 1 == n ? 0 : k + 1), xq, yq);
-            interp_vertex<C>(a, off + k, Ux, Uy);
+            interp_vertex<C>(a, sh, Ux, Uy);
             ax = etoc(esub(x, xr));
             ay = etoc(esub(y, yr));
             bx = etoc(esub(xq, xr));
@@ -235,10 +246,14 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigne
         E x, y, xpv, ypv;
         C Ux = 0, Uy = 0;
         C sx = 0, sy = 0, su = 0, sv = 0;
+        const int kv = valid ? k : 0;
+        load_pos<C>(a, off + kv, x, y);
+        PosIO<C>::load(a.Xp, off + kv, xpv, ypv);
+        const Shape<C> sh = load_shape<C>(a, off + kv);
+        dep_wait();
+        dep_trigger();
         if (valid) {
-            load_pos<C>(a, off + k, x, y);
-            PosIO<C>::load(a.Xp, off + k, xpv, ypv);
-            interp_vertex<C>(a, off + k, Ux, Uy);
+            interp_vertex<C>(a, sh, Ux, Uy);
             sx = etoc(esub(x, xr));
             sy = etoc(esub(y, yr));
             su = Ux;
@@ -390,31 +405,29 @@ __global__ void __launch_bounds__(kAdvThreads) k_advance_batch(const __grid_cons
     advance_unit<C, DYN>(s_a, blockIdx.x - b.off[m], (unsigned)s_a.nau);
 }
 
-cudaError_t launch_advance(lbib_precision prec, const MarkerArgs& a, cudaStream_t s) {
-    if (a.adv_threads < kChunkV || a.adv_threads > kAdvThreads || a.adv_threads % 32) return cudaErrorInvalidValue;
-    if (prec == LBIB_F64) {
-        if (a.has_dyn) k_advance<double, true><<<a.nau, a.adv_threads, 0, s>>>(a);
-        else k_advance<double, false><<<a.nau, a.adv_threads, 0, s>>>(a);
-    } else {
-        if (a.has_dyn) k_advance<float, true><<<a.nau, a.adv_threads, 0, s>>>(a);
-        else k_advance<float, false><<<a.nau, a.adv_threads, 0, s>>>(a);
-    }
-    return cudaGetLastError();
+template <typename C>
+static auto advance_kernel(bool dyn) {
+    return dyn ? k_advance<C, true> : k_advance<C, false>;
+}
+template <typename C>
+static auto advance_batch_kernel(bool dyn) {
+    return dyn ? k_advance_batch<C, true> : k_advance_batch<C, false>;
 }
 
-cudaError_t launch_advance_batch(lbib_precision prec, bool dyn, const MarkerBatch& b, int threads, cudaStream_t s) {
+cudaError_t launch_advance(lbib_precision prec, const MarkerArgs& a, cudaStream_t s, bool chained) {
+    if (a.adv_threads < kChunkV || a.adv_threads > kAdvThreads || a.adv_threads % 32) return cudaErrorInvalidValue;
+    return launch_kernel(prec == LBIB_F64 ? advance_kernel<double>(a.has_dyn) : advance_kernel<float>(a.has_dyn), a.nau,
+                         a.adv_threads, 0, s, chained, a);
+}
+
+cudaError_t launch_advance_batch(lbib_precision prec, bool dyn, const MarkerBatch& b, int threads, cudaStream_t s,
+                                 bool chained) {
     if (b.n < 1 || b.n > kBatchMax) return cudaErrorInvalidValue;
     const int nunits = b.off[b.n];
     if (nunits <= 0) return cudaSuccess;
     if (threads < kChunkV || threads > kAdvThreads || threads % 32) return cudaErrorInvalidValue;
-    if (prec == LBIB_F64) {
-        if (dyn) k_advance_batch<double, true><<<nunits, threads, 0, s>>>(b);
-        else k_advance_batch<double, false><<<nunits, threads, 0, s>>>(b);
-    } else {
-        if (dyn) k_advance_batch<float, true><<<nunits, threads, 0, s>>>(b);
-        else k_advance_batch<float, false><<<nunits, threads, 0, s>>>(b);
-    }
-    return cudaGetLastError();
+    return launch_kernel(prec == LBIB_F64 ? advance_batch_kernel<double>(dyn) : advance_batch_kernel<float>(dyn), nunits,
+                         threads, 0, s, chained, b);
 }
 
 }  // namespace lbib

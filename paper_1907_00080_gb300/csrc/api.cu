@@ -785,25 +785,34 @@ static HydroArgs hydro_args(const lbib_ctx* c, int src) {
 }
 
 // the fused collide-stream kernel in the context's form
-static cudaError_t launch_fused(const lbib_ctx* c, const LbArgs& l, cudaStream_t s) {
+static cudaError_t launch_fused(const lbib_ctx* c, const LbArgs& l, cudaStream_t s, bool chained = false) {
     const bool walls = c->walls != LBIB_WALLS_NONE;
-    if (c->ty == 0) return launch_lb_stream(c->prec, c->vec, walls, c->nv > 0, c->stream_grid, l, s);
-    return launch_lb_step(c->prec, c->vec, c->ty, walls, c->nv > 0, l, s);
+    if (c->ty == 0) return launch_lb_stream(c->prec, c->vec, walls, c->nv > 0, c->stream_grid, l, s, chained);
+    return launch_lb_step(c->prec, c->vec, c->ty, walls, c->nv > 0, l, s, chained);
 }
 
+// Whether the advance kernel starts beside the fused kernel's tail.  Its
+// early blocks gather on the SMs that the fused kernel leaves first: with
+// thousands of blocks (64-member ensemble: 2720, FP16 step 174 -> 183 us) or
+// FP64 work (capillary step 56.7 -> 58.6 us) that costs more than the overlap
+// gives (capillary FP32 17.6 -> 17.0 us, 10-member ensemble 45.3 -> 43.3 us)
+static bool chain_advance(lbib_precision prec, int nunits) { return prec != LBIB_F64 && nunits <= 4 * 152; }
+
 // one time step from population buffer `src`: forces + weights + spreading,
-// fused collide-stream, interpolation + advance, bond kinetics
-static cudaError_t enqueue_step(lbib_ctx* c, int src, cudaStream_t s) {
+// fused collide-stream, interpolation + advance, bond kinetics.  The launches
+// of a step are chained (see dep_wait); `first` marks the first step of a
+// captured sequence, whose first kernel has no predecessor of the cycle
+static cudaError_t enqueue_step(lbib_ctx* c, int src, cudaStream_t s, bool first) {
     MarkerArgs a = c->ma;
     a.gsum = c->G[src];
     a.flags = c->flags[src];
     cudaError_t e;
     const bool has_ib = c->nv > 0;
-    if (c->ndyn > 0 && (e = launch_hydro(c->prec, a, hydro_args(c, src), s)) != cudaSuccess) return e;
-    if (has_ib && (e = launch_forces(c->prec, a, c->max_mem_n, s)) != cudaSuccess) return e;
+    if (c->ndyn > 0 && (e = launch_hydro(c->prec, a, hydro_args(c, src), s, !first)) != cudaSuccess) return e;
+    if (has_ib && (e = launch_forces(c->prec, a, s, !first || c->ndyn > 0)) != cudaSuccess) return e;
     const LbArgs l = lb_args(c, src, src, 1);
-    if ((e = launch_fused(c, l, s)) != cudaSuccess) return e;
-    if (has_ib && (e = launch_advance(c->prec, a, s)) != cudaSuccess) return e;
+    if ((e = launch_fused(c, l, s, !first || has_ib)) != cudaSuccess) return e;
+    if (has_ib && (e = launch_advance(c->prec, a, s, chain_advance(c->prec, a.nau))) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
@@ -835,7 +844,7 @@ static lbib_status build_graphs(lbib_ctx* c) {
             int src = start;
             cudaError_t le = cudaSuccess;
             for (int k = 0; k < nsteps && le == cudaSuccess; ++k) {
-                le = enqueue_step(c, src, cap);
+                le = enqueue_step(c, src, cap, k == 0);
                 src = 1 - src;
             }
             e = cudaStreamEndCapture(cap, &g);
@@ -1207,7 +1216,7 @@ extern "C" lbib_status lbib_profile_kernels(lbib_ctx* c, int32_t reps, double* m
     a.flags = c->flags[c->cur];
     // forces + spreading (accumulates into the field of the current parity)
     CK(cudaEventRecord(ev[0], c->stream));
-    for (int r = 0; r < reps && has_ib; ++r) CK(launch_forces(c->prec, a, c->max_mem_n, c->stream));
+    for (int r = 0; r < reps && has_ib; ++r) CK(launch_forces(c->prec, a, c->stream));
     CK(cudaEventRecord(ev[1], c->stream));
     // fused collide-stream, ping-pong between the buffers
     const int gpar = 1 - c->cur;
@@ -1420,14 +1429,16 @@ static lbib_status ensemble_batch_tables(lbib_ensemble* e, int ngroups) {
 }
 
 // one time step of every member of group g in the batched form, at phase p
-static cudaError_t ensemble_batch_step(const lbib_ensemble* e, int g, int p, cudaStream_t s) {
+// (first: of a captured sequence, see enqueue_step)
+static cudaError_t ensemble_batch_step(const lbib_ensemble* e, int g, int p, cudaStream_t s, bool first) {
     const lbib_ctx* c0 = e->m[0];
     const bool walls = c0->walls != LBIB_WALLS_NONE;
-    cudaError_t r = launch_forces_batch(c0->prec, e->fbb[p][g], s);
+    cudaError_t r = launch_forces_batch(c0->prec, e->fbb[p][g], s, !first);
     if (r == cudaSuccess)
-        r = c0->ty > 0 ? launch_lb_batch(c0->prec, c0->vec, c0->ty, walls, e->lbb[p][g], s)
-                       : launch_lb_stream_batch(c0->prec, c0->vec, walls, e->stream_grid, e->lbb[p][g], s);
-    if (r == cudaSuccess) r = launch_advance_batch(c0->prec, false, e->abb[p][g], e->adv_threads, s);
+        r = c0->ty > 0 ? launch_lb_batch(c0->prec, c0->vec, c0->ty, walls, e->lbb[p][g], s, true)
+                       : launch_lb_stream_batch(c0->prec, c0->vec, walls, e->stream_grid, e->lbb[p][g], s, true);
+    if (r == cudaSuccess) r = launch_advance_batch(c0->prec, false, e->abb[p][g], e->adv_threads, s,
+                                                       chain_advance(c0->prec, e->abb[p][g].off[e->abb[p][g].n]));
     return r;
 }
 
@@ -1453,7 +1464,7 @@ static lbib_status ensemble_build_batched(lbib_ensemble* e, int ngroups) {
             for (int g = 0; g < G && le == cudaSuccess; ++g) {
                 cudaStream_t s = G == 1 ? cap : gs[g];
                 if (G > 1) le = cudaStreamWaitEvent(s, ev[G], 0);
-                for (int k = 0; k < nsteps && le == cudaSuccess; ++k) le = ensemble_batch_step(e, g, flip ^ (k & 1), s);
+                for (int k = 0; k < nsteps && le == cudaSuccess; ++k) le = ensemble_batch_step(e, g, flip ^ (k & 1), s, k == 0);
                 if (G > 1 && le == cudaSuccess) le = cudaEventRecord(ev[g], s);
                 if (G > 1 && le == cudaSuccess) le = cudaStreamWaitEvent(cap, ev[g], 0);
             }

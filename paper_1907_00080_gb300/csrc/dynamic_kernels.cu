@@ -277,6 +277,8 @@ __global__ void __launch_bounds__(HydroShape<kHydroV>::threads) k_hydro(const Ma
     // the unit record carries the membrane's offset and size, so that no block
     // waits on a second table before its first position load
     const int4 u = h.units[blockIdx.x];
+    dep_wait();
+    dep_trigger();
     const int k0 = u.x, kv = u.y, off = u.z, n = u.w;
     const int nel = kv + 1, nfit = 2 * kv + 1;
     // the particle velocities of the chunk, fetched now for the last stage
@@ -360,24 +362,17 @@ __global__ void __launch_bounds__(HydroShape<kHydroV>::threads) k_hydro(const Ma
 
 int hydro_chunk(lbib_precision prec) { return prec == LBIB_F64 ? kHydroV64 : kHydroV32; }
 
-cudaError_t launch_hydro(lbib_precision prec, const MarkerArgs& a, const HydroArgs& h, cudaStream_t s) {
+cudaError_t launch_hydro(lbib_precision prec, const MarkerArgs& a, const HydroArgs& h, cudaStream_t s, bool chained) {
     if (h.nunits == 0) return cudaSuccess;
+    constexpr int t64 = HydroShape<kHydroV64>::threads, t32 = HydroShape<kHydroV32>::threads;
     switch (prec) {
-        case LBIB_F64:
-            k_hydro<double, kHydroV64><<<h.nunits, HydroShape<kHydroV64>::threads, 0, s>>>(a, h);
-            break;
-        case LBIB_F32:
-            k_hydro<float, kHydroV32><<<h.nunits, HydroShape<kHydroV32>::threads, 0, s>>>(a, h);
-            break;
-        case LBIB_F32_STORE_F16:
-            k_hydro<__half, kHydroV32><<<h.nunits, HydroShape<kHydroV32>::threads, 0, s>>>(a, h);
-            break;
+        case LBIB_F64: return launch_kernel(k_hydro<double, kHydroV64>, h.nunits, t64, 0, s, chained, a, h);
+        case LBIB_F32: return launch_kernel(k_hydro<float, kHydroV32>, h.nunits, t32, 0, s, chained, a, h);
+        case LBIB_F32_STORE_F16: return launch_kernel(k_hydro<__half, kHydroV32>, h.nunits, t32, 0, s, chained, a, h);
         case LBIB_F32_STORE_BF16:
-            k_hydro<__nv_bfloat16, kHydroV32><<<h.nunits, HydroShape<kHydroV32>::threads, 0, s>>>(a, h);
-            break;
-        default: return cudaErrorInvalidValue;
+            return launch_kernel(k_hydro<__nv_bfloat16, kHydroV32>, h.nunits, t32, 0, s, chained, a, h);
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace lbib

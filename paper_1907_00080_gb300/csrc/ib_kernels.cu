@@ -123,6 +123,10 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit) {
     __shared__ C s_cox[kStageSeg * kSegV], s_coy[kStageSeg * kSegV];
     __shared__ int s_cn[kStageSeg], s_cv0[kStageSeg];
     const Rest<C>* rest = static_cast<const Rest<C>*>(a.rest);
+    // (with dynamic particles the predecessor is the hydrodynamic kernel, which
+    // started after the positions were complete: its results are waited for
+    // where they are used)
+    if (!a.has_dyn) dep_wait();
 
     // ---- phase 0: positions of the chunk and two halo vertices on each side
     for (int p = tid; p < kn + 4; p += blockDim.x) {
@@ -467,6 +471,7 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit) {
             }
         }
     }
+    if (a.has_dyn) dep_wait();
     __syncthreads();
     if (wid < 2 && tid < kn) {
         const C mag = fix60_to_c<C>((long long)s_rep[tid]);
@@ -491,6 +496,10 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit) {
         s_F[tid][1] = Sy;
     }
     __syncthreads();
+    // (here rather than at the start: the fused kernel's early blocks would
+    // take SMs unevenly around the force blocks; FP64 capillary step 58.6 vs
+    // 63.4 us, FP32 17.0 vs 17.5 us)
+    dep_trigger();
 
     // ---- phase 3: spreading (Sec. 2.2, the transpose of the interpolation):
     // w_j F_v into the fixed-point force field; flag the fused-kernel tiles hit
@@ -590,19 +599,16 @@ cudaError_t launch_rest(lbib_precision prec, const MarkerArgs& a, void* rest, do
     return cudaGetLastError();
 }
 
-cudaError_t launch_forces(lbib_precision prec, const MarkerArgs& a, int, cudaStream_t s) {
-    if (is_f64(prec)) k_forces<double><<<a.nfu, kForceThreads, 0, s>>>(a);
-    else k_forces<float><<<a.nfu, kForceThreads, 0, s>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_forces(lbib_precision prec, const MarkerArgs& a, cudaStream_t s, bool chained) {
+    return launch_kernel(is_f64(prec) ? k_forces<double> : k_forces<float>, a.nfu, kForceThreads, 0, s, chained, a);
 }
 
-cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, cudaStream_t s) {
+cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, cudaStream_t s, bool chained) {
     if (b.n < 1 || b.n > kBatchMax) return cudaErrorInvalidValue;
     const int nunits = b.off[b.n];
     if (nunits <= 0) return cudaSuccess;
-    if (is_f64(prec)) k_forces_batch<double><<<nunits, kForceThreads, 0, s>>>(b);
-    else k_forces_batch<float><<<nunits, kForceThreads, 0, s>>>(b);
-    return cudaGetLastError();
+    return launch_kernel(is_f64(prec) ? k_forces_batch<double> : k_forces_batch<float>, nunits, kForceThreads, 0, s,
+                         chained, b);
 }
 
 cudaError_t launch_seg_boxes(lbib_precision prec, const MarkerArgs& a, cudaStream_t s) {

@@ -52,31 +52,16 @@ __device__ __forceinline__ void lb_tile(const LbArgs& a, int bx, int by) {
     const S* __restrict__ src = static_cast<const S*>(a.src);
     const float inv = a.inv_scale;
 
-    // ---- on lattices that stay in L2, the spread force of every node is read
-    // up front (the field is zero outside the tiles this step's spreading
-    // touched), so that its latency overlaps the population loads instead of
-    // following the tile flag
-    longlong2 gpre[VEC];
-    const bool pre_g = IB == 2 && a.g_prefetch && ok;
-    if (pre_g) {
-#pragma unroll
-        for (int k = 0; k < VEC; ++k) gpre[k] = a.gsum[(size_t)y * nx + x0 + k];
+    // ---- prologue: the pulled rows, as loaded (aligned vectors), and the single
+    // off-vector element at a warp's or row's edge.  With markers the
+    // predecessor of a chained launch is the force kernel, which leaves the
+    // populations alone: these loads run beside it.  (Nothing here consumes a
+    // loaded value, so the wait below does not wait for them.)
+    if (!HAS_IB) {
+        dep_wait();
+        dep_trigger();
     }
-    // this thread's force tile and its flags, read before the populations so
-    // that the flag (an L2 hit) is back while the population loads are still
-    // in flight and the force load that depends on it overlaps them: during a
-    // step the row-tile form flags segments of 32 nodes of one row (tile_w =
-    // 32, tile_h = 1), so the threads that share a flag are lanes of one warp;
-    // in the fields-only read-back the tiles may be those of the persistent form
-    int t = 0, flag = 0, flag_o = 0;
-    if (HAS_IB) {
-        t = (min(y, ny - 1) / a.tile_h) * a.tiles_x + min(x0, nx - 1) / a.tile_w;
-        flag = a.flags[t];
-        if (a.clear_other) flag_o = a.flags_other[t];
-    }
-
-    // ---- pull streaming (Eq. BGK left side) with half-way bounce-back
-    C f[9][VEC];
+    C f[9][VEC], edge[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         int sy = y - cy(i);
@@ -86,38 +71,66 @@ __device__ __forceinline__ void lb_tile(const LbArgs& a, int bx, int by) {
         } else {
             sy = sy < 0 ? sy + ny : (sy >= ny ? sy - ny : sy);
         }
-        if (bb) {
-            // the population that left this node toward the wall comes back
-            // reversed, plus the momentum of a moving wall (diagonals only)
-            const S* row = src + (size_t)opp(i) * N + (size_t)y * nx;
-            load_pack<S, VEC>(row, x0, ok, inv, f[i]);
-            if (cx(i) != 0) {
-                const C t = C(cx(i)) * wall_term<C>(a, cy(i) > 0);
-#pragma unroll
-                for (int k = 0; k < VEC; ++k) f[i][k] += t;
-            }
-            continue;
+        edge[i] = C(0);
+        // (bounce-back: the population that left this node toward the wall comes back reversed)
+        const S* row = bb ? src + (size_t)opp(i) * N + (size_t)y * nx : src + (size_t)i * N + (size_t)sy * nx;
+        load_pack<S, VEC>(row, x0, ok, inv, f[i]);
+        if (cx(i) == 1) {
+            if (lane == 0 && ok && !bb) edge[i] = Storage<S>::load(row[x0 == 0 ? nx - 1 : x0 - 1], inv);
+        } else if (cx(i) == -1) {
+            if (ok && !bb && (lane == 31 || x0 + VEC >= nx))
+                edge[i] = Storage<S>::load(row[x0 + VEC >= nx ? 0 : x0 + VEC], inv);
         }
-        const S* row = src + (size_t)i * N + (size_t)sy * nx;
-        C v[VEC];
-        load_pack<S, VEC>(row, x0, ok, inv, v);
-        if (cx(i) == 0) {
+    }
+    if (HAS_IB) {
+        dep_wait();
+        dep_trigger();
+    }
+
+    // ---- this thread's force tile and its flags: during a step the row-tile
+    // form flags segments of 32 nodes of one row (tile_w = 32, tile_h = 1), so
+    // the threads that share a flag are lanes of one warp; in the fields-only
+    // read-back the tiles may be those of the persistent form.  On lattices
+    // that stay in L2, the spread force of every node is read with the flags
+    // (the field is zero outside the tiles this step's spreading touched)
+    // instead of after them
+    longlong2 gpre[VEC];
+    const bool pre_g = IB == 2 && a.g_prefetch && ok;
+    if (pre_g) {
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) f[i][k] = v[k];
+        for (int k = 0; k < VEC; ++k) gpre[k] = a.gsum[(size_t)y * nx + x0 + k];
+    }
+    int t = 0, flag = 0, flag_o = 0;
+    if (HAS_IB) {
+        t = (min(y, ny - 1) / a.tile_h) * a.tiles_x + min(x0, nx - 1) / a.tile_w;
+        flag = a.flags[t];
+        if (a.clear_other) flag_o = a.flags_other[t];
+    }
+
+    // ---- pull streaming (Eq. BGK left side) with half-way bounce-back: the
+    // x-shifted directions take the off-vector element from the neighbouring lane
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        if (cx(i) == 0) continue;
+        const bool bb = WALLS && (y - cy(i) < 0 || y - cy(i) >= ny);
+        if (bb) {
+            // the momentum of a moving wall (diagonals only)
+            const C w = C(cx(i)) * wall_term<C>(a, cy(i) > 0);
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) f[i][k] += w;
         } else if (cx(i) == 1) {
             // needs x0-1 .. x0+VEC-2
-            C prev = __shfl_up_sync(FULL, v[VEC - 1], 1);
-            if (lane == 0 && ok) prev = Storage<S>::load(row[x0 == 0 ? nx - 1 : x0 - 1], inv);
-            f[i][0] = prev;
+            C prev = __shfl_up_sync(FULL, f[i][VEC - 1], 1);
+            if (lane == 0 && ok) prev = edge[i];
 #pragma unroll
-            for (int k = 1; k < VEC; ++k) f[i][k] = v[k - 1];
+            for (int k = VEC - 1; k > 0; --k) f[i][k] = f[i][k - 1];
+            f[i][0] = prev;
         } else {
             // needs x0+1 .. x0+VEC
-            C next = __shfl_down_sync(FULL, v[0], 1);
-            if (ok && (lane == 31 || x0 + VEC >= nx))
-                next = Storage<S>::load(row[x0 + VEC >= nx ? 0 : x0 + VEC], inv);
+            C next = __shfl_down_sync(FULL, f[i][0], 1);
+            if (ok && (lane == 31 || x0 + VEC >= nx)) next = edge[i];
 #pragma unroll
-            for (int k = 0; k < VEC - 1; ++k) f[i][k] = v[k + 1];
+            for (int k = 0; k < VEC - 1; ++k) f[i][k] = f[i][k + 1];
             f[i][VEC - 1] = next;
         }
     }
@@ -229,81 +242,74 @@ __global__ void __launch_bounds__(512) k_lb_step_batch(const __grid_constant__ L
 }
 
 template <typename S, int VEC>
-static cudaError_t launch_lb_t(int ty, bool walls, bool has_ib, const LbArgs& a, cudaStream_t s) {
+static cudaError_t launch_lb_t(int ty, bool walls, bool has_ib, const LbArgs& a, cudaStream_t s, bool chained) {
     dim3 block(32, ty);
     dim3 grid((a.nx + 32 * VEC - 1) / (32 * VEC), (a.ny + ty - 1) / ty);
     // the up-front force read is its own instantiation: its registers would
     // lower the occupancy of the plain form, which DRAM-bound runs need
     const int ib = has_ib ? (a.g_prefetch ? 2 : 1) : 0;
-    if (walls) {
-        if (ib == 2) k_lb_step<S, VEC, true, 2><<<grid, block, 0, s>>>(a);
-        else if (ib == 1) k_lb_step<S, VEC, true, 1><<<grid, block, 0, s>>>(a);
-        else k_lb_step<S, VEC, true, 0><<<grid, block, 0, s>>>(a);
-    } else {
-        if (ib == 2) k_lb_step<S, VEC, false, 2><<<grid, block, 0, s>>>(a);
-        else if (ib == 1) k_lb_step<S, VEC, false, 1><<<grid, block, 0, s>>>(a);
-        else k_lb_step<S, VEC, false, 0><<<grid, block, 0, s>>>(a);
-    }
-    return cudaGetLastError();
+    auto kern = walls ? (ib == 2 ? k_lb_step<S, VEC, true, 2> : (ib == 1 ? k_lb_step<S, VEC, true, 1> : k_lb_step<S, VEC, true, 0>))
+                      : (ib == 2 ? k_lb_step<S, VEC, false, 2> : (ib == 1 ? k_lb_step<S, VEC, false, 1> : k_lb_step<S, VEC, false, 0>));
+    return launch_kernel(kern, grid, block, 0, s, chained, a);
 }
 
 template <typename S, int VEC>
-static cudaError_t launch_lb_batch_t(int ty, bool walls, const LbBatch& b, cudaStream_t s) {
+static cudaError_t launch_lb_batch_t(int ty, bool walls, const LbBatch& b, cudaStream_t s, bool chained) {
     const int nblocks = b.off[b.n];
     if (nblocks <= 0) return cudaSuccess;
     dim3 block(32, ty);
-    if (walls) k_lb_step_batch<S, VEC, true><<<nblocks, block, 0, s>>>(b);
-    else k_lb_step_batch<S, VEC, false><<<nblocks, block, 0, s>>>(b);
-    return cudaGetLastError();
+    return launch_kernel(walls ? k_lb_step_batch<S, VEC, true> : k_lb_step_batch<S, VEC, false>, nblocks, block, 0, s,
+                         chained, b);
 }
 
-cudaError_t launch_lb_batch(lbib_precision prec, int vec, int ty, bool walls, const LbBatch& b, cudaStream_t s) {
+cudaError_t launch_lb_batch(lbib_precision prec, int vec, int ty, bool walls, const LbBatch& b, cudaStream_t s,
+                            bool chained) {
     if (b.n < 1 || b.n > kBatchMax) return cudaErrorInvalidValue;
     switch (prec) {
         case LBIB_F64:
-            if (vec == 1) return launch_lb_batch_t<double, 1>(ty, walls, b, s);
-            if (vec == 2) return launch_lb_batch_t<double, 2>(ty, walls, b, s);
+            if (vec == 1) return launch_lb_batch_t<double, 1>(ty, walls, b, s, chained);
+            if (vec == 2) return launch_lb_batch_t<double, 2>(ty, walls, b, s, chained);
             break;
         case LBIB_F32:
-            if (vec == 1) return launch_lb_batch_t<float, 1>(ty, walls, b, s);
-            if (vec == 2) return launch_lb_batch_t<float, 2>(ty, walls, b, s);
-            if (vec == 4) return launch_lb_batch_t<float, 4>(ty, walls, b, s);
+            if (vec == 1) return launch_lb_batch_t<float, 1>(ty, walls, b, s, chained);
+            if (vec == 2) return launch_lb_batch_t<float, 2>(ty, walls, b, s, chained);
+            if (vec == 4) return launch_lb_batch_t<float, 4>(ty, walls, b, s, chained);
             break;
         case LBIB_F32_STORE_F16:
-            if (vec == 2) return launch_lb_batch_t<__half, 2>(ty, walls, b, s);
-            if (vec == 4) return launch_lb_batch_t<__half, 4>(ty, walls, b, s);
-            if (vec == 8) return launch_lb_batch_t<__half, 8>(ty, walls, b, s);
+            if (vec == 2) return launch_lb_batch_t<__half, 2>(ty, walls, b, s, chained);
+            if (vec == 4) return launch_lb_batch_t<__half, 4>(ty, walls, b, s, chained);
+            if (vec == 8) return launch_lb_batch_t<__half, 8>(ty, walls, b, s, chained);
             break;
         case LBIB_F32_STORE_BF16:
-            if (vec == 2) return launch_lb_batch_t<__nv_bfloat16, 2>(ty, walls, b, s);
-            if (vec == 4) return launch_lb_batch_t<__nv_bfloat16, 4>(ty, walls, b, s);
-            if (vec == 8) return launch_lb_batch_t<__nv_bfloat16, 8>(ty, walls, b, s);
+            if (vec == 2) return launch_lb_batch_t<__nv_bfloat16, 2>(ty, walls, b, s, chained);
+            if (vec == 4) return launch_lb_batch_t<__nv_bfloat16, 4>(ty, walls, b, s, chained);
+            if (vec == 8) return launch_lb_batch_t<__nv_bfloat16, 8>(ty, walls, b, s, chained);
             break;
     }
     return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_lb_step(lbib_precision prec, int vec, int ty, bool walls, bool has_ib,
-                           const LbArgs& a, cudaStream_t s) {
+                           const LbArgs& a, cudaStream_t s, bool chained) {
     switch (prec) {
         case LBIB_F64:
-            if (vec == 1) return launch_lb_t<double, 1>(ty, walls, has_ib, a, s);
-            if (vec == 2) return launch_lb_t<double, 2>(ty, walls, has_ib, a, s);
+            if (vec == 1) return launch_lb_t<double, 1>(ty, walls, has_ib, a, s, chained);
+            if (vec == 2) return launch_lb_t<double, 2>(ty, walls, has_ib, a, s, chained);
             break;
         case LBIB_F32:
-            if (vec == 1) return launch_lb_t<float, 1>(ty, walls, has_ib, a, s);
-            if (vec == 2) return launch_lb_t<float, 2>(ty, walls, has_ib, a, s);
-            if (vec == 4) return launch_lb_t<float, 4>(ty, walls, has_ib, a, s);
+            if (vec == 1) return launch_lb_t<float, 1>(ty, walls, has_ib, a, s, chained);
+            if (vec == 2) return launch_lb_t<float, 2>(ty, walls, has_ib, a, s, chained);
+            if (vec == 4) return launch_lb_t<float, 4>(ty, walls, has_ib, a, s, chained);
             break;
         case LBIB_F32_STORE_F16:
-            if (vec == 2) return launch_lb_t<__half, 2>(ty, walls, has_ib, a, s);
-            if (vec == 4) return launch_lb_t<__half, 4>(ty, walls, has_ib, a, s);
-            if (vec == 8) return launch_lb_t<__half, 8>(ty, walls, has_ib, a, s);
+            if (vec == 2) return launch_lb_t<__half, 2>(ty, walls, has_ib, a, s, chained);
+            if (vec == 4) return launch_lb_t<__half, 4>(ty, walls, has_ib, a, s, chained);
+            if (vec == 8) return launch_lb_t<__half, 8>(ty, walls, has_ib, a, s, chained);
             break;
         case LBIB_F32_STORE_BF16:
-            if (vec == 2) return launch_lb_t<__nv_bfloat16, 2>(ty, walls, has_ib, a, s);
-            if (vec == 4) return launch_lb_t<__nv_bfloat16, 4>(ty, walls, has_ib, a, s);
-            if (vec == 8) return launch_lb_t<__nv_bfloat16, 8>(ty, walls, has_ib, a, s);
+            if (vec == 2) return launch_lb_t<__nv_bfloat16, 2>(ty, walls, has_ib, a, s, chained);
+            if (vec == 4) return launch_lb_t<__nv_bfloat16, 4>(ty, walls, has_ib, a, s, chained);
+            if (vec == 8) return launch_lb_t<__nv_bfloat16, 8>(ty, walls, has_ib, a, s, chained);
             break;
     }
     return cudaErrorInvalidValue;

@@ -75,6 +75,10 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, unsigned bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
+// adds to the bytes expected in the current phase, without an arrival
+__device__ __forceinline__ void mbar_expect_tx_only(uint32_t bar, unsigned bytes) {
+    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
 // bounded wait for the phase with the given parity; false if it never completed
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     for (int it = 0; it < kSpinLimit; ++it) {
@@ -163,6 +167,7 @@ struct OneLattice {
     __device__ void stage_args(ItemRef p, int, int st, int lane) const {
         if (lane == 0) s_pos[st] = p;
     }
+    __device__ bool lattice_only() const { return a.flags == nullptr; }
     __device__ const LbArgs& staged(int) const { return a; }
     __device__ ItemRef staged_pos(long long, int st) const { return s_pos[st]; }
 };
@@ -197,6 +202,7 @@ struct ManyLattices {
             reinterpret_cast<long long*>(&s_args[st])[w] = reinterpret_cast<const long long*>(&A)[w];
         if (lane == 0) s_pos[st] = p;
     }
+    __device__ bool lattice_only() const { return false; }  // batches have markers
     __device__ const LbArgs& staged(int st) const { return s_args[st]; }
     __device__ ItemRef staged_pos(long long, int st) const { return s_pos[st]; }
 };
@@ -513,8 +519,26 @@ __device__ __forceinline__ void stream_ws(const Items& it) {
         // ---- producer: stage segment k once the consumers have left the
         // segment k - kStages that used the same stage; its tile flags were
         // fetched three segments ahead (their latency stays off the producer's path)
+        // prologue: the rows of the first kStages items (populations alone, which
+        // the force kernel leaves alone), beside the tail of the predecessor;
+        // their bytes are expected now, the producer's arrivals on the full
+        // barriers follow with their flags
         FlagRegs r0, r1, r2;
         r0 = r1 = r2 = FlagRegs{{0, 0}, {0, 0}, {0, 0}, 0};
+        if (it.lattice_only()) dep_wait();  // the predecessor wrote the populations
+        {
+            ItemRef p{0, 0};
+            int m = 0;
+            for (int k = 0; k < kStages && k < my_n; ++k) {
+                const LbArgs& A = it.locate(first + (long long)k * stride, p, m);
+                const uint32_t bar = smem_addr(&bars[k]);
+                if (lane == 0) mbar_expect_tx_only(bar, stage_bytes<S, NPT>(A, p));
+                __syncwarp();
+                if (lane < 9) stage_rows<S, NPT, WALLS>(A, p, smem0 + k * Gm::STAGE_BYTES, bar, lane, 9);
+                if (lane == 0) s_last_issued[k] = k;
+            }
+        }
+        dep_wait();
         if (my_n > 0) fetch_flags<W>(it, first, lane, r0, 0);
         if (my_n > 1) fetch_flags<W>(it, first + stride, lane, r1, r0.m);
         if (my_n > 2) fetch_flags<W>(it, first + 2 * stride, lane, r2, r1.m);
@@ -536,18 +560,24 @@ __device__ __forceinline__ void stream_ws(const Items& it) {
             const LbArgs& A = it.staged(stage);
             const ItemRef p = it.staged_pos(item, stage);
             const uint32_t bar = smem_addr(&bars[stage]);
-            if (lane == 0) mbar_expect_tx(bar, stage_bytes<S, NPT>(A, p));
-            __syncwarp();
-            if (lane < 9) stage_rows<S, NPT, WALLS>(A, p, smem0 + stage * Gm::STAGE_BYTES, bar, lane, 9);
-            if (lane == 0) s_last_issued[stage] = k;
+            if (k < kStages) {
+                if (lane == 0) mbar_arrive(bar);
+            } else {
+                if (lane == 0) mbar_expect_tx(bar, stage_bytes<S, NPT>(A, p));
+                __syncwarp();
+                if (lane < 9) stage_rows<S, NPT, WALLS>(A, p, smem0 + stage * Gm::STAGE_BYTES, bar, lane, 9);
+                if (lane == 0) s_last_issued[stage] = k;
+            }
             r0 = r1;
             r1 = r2;
             if (k + 3 < my_n) fetch_flags<W>(it, first + (long long)(k + 3) * stride, lane, r2, r1.m);
         }
     } else {
         // ---- consumers
+        dep_wait();
         for (int k = 0; k < my_n; ++k) {
             const int stage = k % kStages;
+            if (k == my_n - 1) dep_trigger();
             const bool ok = mbar_wait_sleep(smem_addr(&bars[stage]), (uint32_t)((k / kStages) & 1));
             const long long item = first + (long long)k * stride;
             const LbArgs& A = it.staged(stage);
@@ -625,13 +655,29 @@ __device__ __forceinline__ void stream_bar(const Items& it) {
 
     // (the member hint stays 0: this schedule serves single lattices, whose
     // items have no member to search)
+    // (the rows before the wait: the force kernel, a chained launch's
+    // predecessor with markers, leaves the populations alone; the flags after
+    // it.  Without markers the predecessor wrote the populations.)
     if (warp == 0) {
-        for (int k = 0; k < kStages && k < my_n; ++k) {
-            FlagRegs r;
-            fetch_flags<W>(it, first + (long long)k * stride, lane, r, 0);
-            keep_flags(r, lane, &s_fm[k]);
-            issue(k, r);
+        FlagRegs r[kStages];
+        if (it.lattice_only()) dep_wait();
+#pragma unroll
+        for (int k = 0; k < kStages; ++k) {
+            r[k] = FlagRegs{{0, 0}, {0, 0}, {0, 0}, 0};
+            if (k < my_n) {
+                it.locate(first + (long long)k * stride, r[k].p, r[k].m);
+                issue(k, r[k]);
+            }
         }
+        dep_wait();
+#pragma unroll
+        for (int k = 0; k < kStages; ++k)
+            if (k < my_n) fetch_flags<W>(it, first + (long long)k * stride, lane, r[k], 0);
+#pragma unroll
+        for (int k = 0; k < kStages; ++k)
+            if (k < my_n) keep_flags(r[k], lane, &s_fm[k]);
+    } else {
+        dep_wait();
     }
     __syncthreads();
 
@@ -639,6 +685,7 @@ __device__ __forceinline__ void stream_bar(const Items& it) {
     int k = 0;
     for (; k < my_n; ++k) {
         const int stage = k % kStages;
+        if (k == my_n - 1) dep_trigger();
         // warp 0 fetches the flags of the item it stages at the end of this one
         FlagRegs nf{{0, 0}, {0, 0}, {0, 0}, 0};
         if (warp == 0 && k + kStages < my_n) fetch_flags<W>(it, first + (long long)(k + kStages) * stride, lane, nf, 0);
@@ -746,7 +793,7 @@ cudaError_t prepare_t(int* grid) {
 // or a batch (b)
 template <typename S, int NPT>
 cudaError_t dispatch(bool prepare, bool walls, int grid, int* grid_out, const LbArgs* a, const LbBatch* b,
-                     cudaStream_t s) {
+                     cudaStream_t s, bool chained) {
     const bool batch = b != nullptr;
     if (prepare) {
         if (batch) return walls ? prepare_t<S, NPT, true, true>(grid_out) : prepare_t<S, NPT, false, true>(grid_out);
@@ -764,37 +811,34 @@ cudaError_t dispatch(bool prepare, bool walls, int grid, int* grid_out, const Lb
     const int g = (int)(items < grid ? items : grid);
     if (g <= 0) return cudaSuccess;
     constexpr int SM = Geom<S, NPT>::SMEM;
-    if (batch) {
-        if (walls) stream_kernel<S, NPT, true, true>()<<<g, threads, SM, s>>>(*b);
-        else stream_kernel<S, NPT, false, true>()<<<g, threads, SM, s>>>(*b);
-    } else {
-        if (walls) stream_kernel<S, NPT, true, false>()<<<g, threads, SM, s>>>(*a);
-        else stream_kernel<S, NPT, false, false>()<<<g, threads, SM, s>>>(*a);
-    }
-    return cudaGetLastError();
+    if (batch)
+        return launch_kernel(walls ? stream_kernel<S, NPT, true, true>() : stream_kernel<S, NPT, false, true>(), g, threads,
+                             SM, s, chained, *b);
+    return launch_kernel(walls ? stream_kernel<S, NPT, true, false>() : stream_kernel<S, NPT, false, false>(), g, threads, SM,
+                         s, chained, *a);
 }
 
 cudaError_t dispatch_all(lbib_precision prec, int npt, bool prepare, bool walls, int grid, int* grid_out,
-                         const LbArgs* a, const LbBatch* b, cudaStream_t s) {
+                         const LbArgs* a, const LbBatch* b, cudaStream_t s, bool chained = false) {
     switch (prec) {
         case LBIB_F64:
-            if (npt == 1) return dispatch<double, 1>(prepare, walls, grid, grid_out, a, b, s);
-            if (npt == 2) return dispatch<double, 2>(prepare, walls, grid, grid_out, a, b, s);
+            if (npt == 1) return dispatch<double, 1>(prepare, walls, grid, grid_out, a, b, s, chained);
+            if (npt == 2) return dispatch<double, 2>(prepare, walls, grid, grid_out, a, b, s, chained);
             break;
         case LBIB_F32:
-            if (npt == 1) return dispatch<float, 1>(prepare, walls, grid, grid_out, a, b, s);
-            if (npt == 2) return dispatch<float, 2>(prepare, walls, grid, grid_out, a, b, s);
-            if (npt == 4) return dispatch<float, 4>(prepare, walls, grid, grid_out, a, b, s);
+            if (npt == 1) return dispatch<float, 1>(prepare, walls, grid, grid_out, a, b, s, chained);
+            if (npt == 2) return dispatch<float, 2>(prepare, walls, grid, grid_out, a, b, s, chained);
+            if (npt == 4) return dispatch<float, 4>(prepare, walls, grid, grid_out, a, b, s, chained);
             break;
         case LBIB_F32_STORE_F16:
-            if (npt == 2) return dispatch<__half, 2>(prepare, walls, grid, grid_out, a, b, s);
-            if (npt == 4) return dispatch<__half, 4>(prepare, walls, grid, grid_out, a, b, s);
-            if (npt == 8) return dispatch<__half, 8>(prepare, walls, grid, grid_out, a, b, s);
+            if (npt == 2) return dispatch<__half, 2>(prepare, walls, grid, grid_out, a, b, s, chained);
+            if (npt == 4) return dispatch<__half, 4>(prepare, walls, grid, grid_out, a, b, s, chained);
+            if (npt == 8) return dispatch<__half, 8>(prepare, walls, grid, grid_out, a, b, s, chained);
             break;
         case LBIB_F32_STORE_BF16:
-            if (npt == 2) return dispatch<__nv_bfloat16, 2>(prepare, walls, grid, grid_out, a, b, s);
-            if (npt == 4) return dispatch<__nv_bfloat16, 4>(prepare, walls, grid, grid_out, a, b, s);
-            if (npt == 8) return dispatch<__nv_bfloat16, 8>(prepare, walls, grid, grid_out, a, b, s);
+            if (npt == 2) return dispatch<__nv_bfloat16, 2>(prepare, walls, grid, grid_out, a, b, s, chained);
+            if (npt == 4) return dispatch<__nv_bfloat16, 4>(prepare, walls, grid, grid_out, a, b, s, chained);
+            if (npt == 8) return dispatch<__nv_bfloat16, 8>(prepare, walls, grid, grid_out, a, b, s, chained);
             break;
     }
     return cudaErrorInvalidValue;
@@ -811,8 +855,8 @@ cudaError_t prepare_lb_stream(lbib_precision prec, int npt, bool walls, bool, in
 }
 
 cudaError_t launch_lb_stream(lbib_precision prec, int npt, bool walls, bool, int grid, const LbArgs& a,
-                             cudaStream_t s) {
-    return dispatch_all(prec, npt, false, walls, grid, nullptr, &a, nullptr, s);
+                             cudaStream_t s, bool chained) {
+    return dispatch_all(prec, npt, false, walls, grid, nullptr, &a, nullptr, s, chained);
 }
 
 cudaError_t prepare_lb_stream_batch(lbib_precision prec, int npt, bool walls, int* grid) {
@@ -822,8 +866,8 @@ cudaError_t prepare_lb_stream_batch(lbib_precision prec, int npt, bool walls, in
 }
 
 cudaError_t launch_lb_stream_batch(lbib_precision prec, int npt, bool walls, int grid, const LbBatch& b,
-                                   cudaStream_t s) {
-    return dispatch_all(prec, npt, false, walls, grid, nullptr, nullptr, &b, s);
+                                   cudaStream_t s, bool chained) {
+    return dispatch_all(prec, npt, false, walls, grid, nullptr, nullptr, &b, s, chained);
 }
 
 }  // namespace lbib

@@ -20,6 +20,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "lbib.h"
@@ -288,13 +289,49 @@ __device__ __forceinline__ int marker_member(const MarkerBatch& b, int blk) {
     return blk < kBlockTable ? (int)b.member[blk] : batch_member(b.off, b.n, blk);
 }
 
+// ---------------------------------------------------------------- chained launches
+// The kernels of a captured time step are chained by programmatic dependent
+// launch (`chained` = true at the launch): a kernel may start while its
+// predecessor still runs and overlaps its prologue with it.  The rules that
+// make this safe, for the cycle (hydro ->) forces -> fused -> advance -> ...:
+//  - dep_wait() returns when the predecessor's grid is complete and its
+//    writes are visible; every thread calls it before it writes anything to
+//    global memory that another kernel of the cycle touches and before it
+//    reads what the predecessor writes;
+//  - dep_trigger() lets the successor start; every kernel calls it after its
+//    own dep_wait().  So when a block starts, all kernels before its
+//    predecessor are complete, and its prologue may read whatever the
+//    predecessor does not write (with dynamic particles the force kernel's
+//    predecessor is the hydrodynamic kernel, so all of it but the
+//    hydrodynamic force and the spreading runs beside that one).
+// Outside a chain both are no-ops and launches are ordinary.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool chained,
+                                 A&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, std::forward<A>(args)...);
+}
+
 // ---------------------------------------------------------------- launchers
 // lb_kernels.cu
 cudaError_t launch_lb_step(lbib_precision prec, int vec, int ty, bool walls, bool has_ib,
-                           const LbArgs& a, cudaStream_t s);
+                           const LbArgs& a, cudaStream_t s, bool chained = false);
 // batched row tiles of up to kBatchMax lattices with markers, all with the
 // tile shape (vec, ty); b.off[b.n] blocks
-cudaError_t launch_lb_batch(lbib_precision prec, int vec, int ty, bool walls, const LbBatch& b, cudaStream_t s);
+cudaError_t launch_lb_batch(lbib_precision prec, int vec, int ty, bool walls, const LbBatch& b, cudaStream_t s,
+                            bool chained = false);
 // lb_stream_kernel.cu: the persistent bulk-copy form of the fused kernel (one
 // CTA per SM slot streams row segments of 256 * npt nodes through a 4-stage
 // shared-memory pipeline); prepare_ sets its shared-memory limit and returns
@@ -302,12 +339,12 @@ cudaError_t launch_lb_batch(lbib_precision prec, int vec, int ty, bool walls, co
 int lb_stream_halo(lbib_precision prec);  // elements per 16-byte halo chunk
 cudaError_t prepare_lb_stream(lbib_precision prec, int npt, bool walls, bool has_ib, int* grid);
 cudaError_t launch_lb_stream(lbib_precision prec, int npt, bool walls, bool has_ib, int grid,
-                             const LbArgs& a, cudaStream_t s);
+                             const LbArgs& a, cudaStream_t s, bool chained = false);
 // the persistent form over the segments of up to kBatchMax lattices (b.off:
 // first segment of each member, b.tiles_x: its segments per row)
 cudaError_t prepare_lb_stream_batch(lbib_precision prec, int npt, bool walls, int* grid);
 cudaError_t launch_lb_stream_batch(lbib_precision prec, int npt, bool walls, int grid, const LbBatch& b,
-                                   cudaStream_t s);
+                                   cudaStream_t s, bool chained = false);
 // walls: 0 periodic, 1 bounce-back (bb_* the moving-wall terms), 2 Zou-He (uw_* the wall
 // velocities; the unknown populations of the wall rows rebuilt without a force)
 cudaError_t launch_stream_out(lbib_precision prec, const void* src, double* out, int nx, int ny,
@@ -326,17 +363,19 @@ cudaError_t launch_mass(lbib_precision prec, const void* src, long long n_elems,
 // ib_kernels.cu
 cudaError_t launch_rest(lbib_precision prec, const MarkerArgs& a, void* rest, double* A0, double* qa,
                         cudaStream_t s);
-cudaError_t launch_forces(lbib_precision prec, const MarkerArgs& a, int max_n, cudaStream_t s);
-cudaError_t launch_advance(lbib_precision prec, const MarkerArgs& a, cudaStream_t s);
+cudaError_t launch_forces(lbib_precision prec, const MarkerArgs& a, cudaStream_t s, bool chained = false);
+cudaError_t launch_advance(lbib_precision prec, const MarkerArgs& a, cudaStream_t s, bool chained = false);
 // batched marker kernels of up to kBatchMax contexts (b.off[b.n] blocks); the
 // advance blocks have `threads` threads (the widest member's)
-cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, cudaStream_t s);
-cudaError_t launch_advance_batch(lbib_precision prec, bool dyn, const MarkerBatch& b, int threads, cudaStream_t s);
+cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, cudaStream_t s, bool chained = false);
+cudaError_t launch_advance_batch(lbib_precision prec, bool dyn, const MarkerBatch& b, int threads, cudaStream_t s,
+                                 bool chained = false);
 cudaError_t launch_seg_boxes(lbib_precision prec, const MarkerArgs& a, cudaStream_t s);
 cudaError_t launch_areas(lbib_precision prec, const MarkerArgs& a, double* areas, cudaStream_t s);
 // dynamic_kernels.cu: hydrodynamic stresses and forcing terms of the dynamic
 // particles at the start of a step (before launch_forces)
-cudaError_t launch_hydro(lbib_precision prec, const MarkerArgs& a, const HydroArgs& h, cudaStream_t s);
+cudaError_t launch_hydro(lbib_precision prec, const MarkerArgs& a, const HydroArgs& h, cudaStream_t s,
+                         bool chained = false);
 int hydro_chunk(lbib_precision prec);  // vertices per block of the hydrodynamic kernel
 // observables.cu: 8 doubles per membrane (see lbib_membrane_observables)
 cudaError_t launch_observables(lbib_precision prec, const MarkerArgs& a, double* out, cudaStream_t s);

@@ -248,17 +248,33 @@ __device__ __forceinline__ void seg_box_regs(const MarkerArgs& a, int sg, int la
     }
 }
 
-// interpolation U_v = sum_j phi_v(x_j) u(x_j) with the weights of this step
+// interpolation U_v = sum_j phi_v(x_j) u(x_j) with the weights of this step:
+// the weights and the stencil origin, read ahead of the velocities (in the
+// advance kernel's prologue, beside the fused kernel that writes those)
 template <typename C>
-__device__ __forceinline__ void interp_vertex(const MarkerArgs& a, int v, C& Ux, C& Uy) {
+struct Shape {
+    C w[9];
+    int i0, j0;
+};
+template <typename C>
+__device__ __forceinline__ Shape<C> load_shape(const MarkerArgs& a, int v) {
+    const C* W = static_cast<const C*>(a.W);
+    Shape<C> s;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) s.w[q] = W[9 * (size_t)v + q];
+    const int2 o = reinterpret_cast<const int2*>(a.stencil)[v];
+    s.i0 = o.x;
+    s.j0 = o.y;
+    return s;
+}
+template <typename C>
+__device__ __forceinline__ void interp_vertex(const MarkerArgs& a, const Shape<C>& s, C& Ux, C& Uy) {
     const C* ux = static_cast<const C*>(a.ux);
     const C* uy = static_cast<const C*>(a.uy);
-    const C* W = static_cast<const C*>(a.W);
-    const int i0 = a.stencil[2 * v], j0 = a.stencil[2 * v + 1];
     C sx = C(0), sy = C(0);
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-        int j = j0 + b - 1;
+        int j = s.j0 + b - 1;
         if (a.walls) {
             if (j < 0 || j >= a.ny) continue;
         } else {
@@ -266,9 +282,9 @@ __device__ __forceinline__ void interp_vertex(const MarkerArgs& a, int v, C& Ux,
         }
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            int i = i0 + q - 1;
+            int i = s.i0 + q - 1;
             i = i < 0 ? i + a.nx : (i >= a.nx ? i - a.nx : i);
-            const C w = W[9 * (size_t)v + b * 3 + q];
+            const C w = s.w[b * 3 + q];
             const size_t node = (size_t)j * a.nx + i;
             sx += w * ux[node];
             sy += w * uy[node];
