@@ -575,7 +575,9 @@ lbib_status lbib_profile_kernels(lbib_ctx* ctx, int32_t reps, double* ms_per_lau
  * Errors: LBIB_E_STATE before the first step. */
 lbib_status lbib_profile_hydro(lbib_ctx* ctx, int32_t reps, double* ms_per_launch);
 
-/* Number of kernels one time step launches (for launch accounting). */
+/* Number of kernels one time step launches (for launch accounting; with
+ * membranes, every captured sequence of 1 or 16 steps ends with one small
+ * launch more, which settles the last step's bonds). */
 int32_t lbib_kernels_per_step(const lbib_ctx* ctx);
 
 /* Scale exponent k of the 16-bit storage (d_i * 2^k); 0 for F32/F64. */

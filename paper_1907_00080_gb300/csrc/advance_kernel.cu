@@ -7,10 +7,14 @@
 // rigid motion, the latter follows Newton-Euler).  Per vertex: interpolate
 // u^n (Sec. 2.3), advance with Eq. kinematicPos (BDF2; forward Euler on the
 // first step), refresh the repulsion boxes.  Then the ligands whose element
-// lies inside the unit are decided at X^{n+1} (bond_logic.cuh); the last
-// block to finish decides the few ligands whose element straddles two units,
-// applies ruptures and formations for all ligands and advances the step
-// counter.
+// starts in the unit are decided at X^{n+1} (bond_logic.cuh); a chunk whose
+// last element ends in the ring's next chunk advances that one vertex too.
+//
+// The decisions are applied by the next force kernel (settle_bonds).  A last
+// block that decided the elements across chunks and applied everything, as
+// this kernel had before, was a third of its time: 6100 of 18000 cycles on the
+// 640 x 160 capillary (a device-wide fence and an arrival counter, then two
+// more rounds to L2).
 #include "marker_common.cuh"
 
 namespace lbib {
@@ -32,22 +36,6 @@ __device__ __forceinline__ typename Ext<C>::E ehi_pos_y(const MarkerArgs& a, int
     return y;
 }
 
-template <typename C>
-__device__ __forceinline__ void load_pos_cg(const void* X, int v, typename Ext<C>::E& x,
-                                            typename Ext<C>::E& y);
-template <>
-__device__ __forceinline__ void load_pos_cg<double>(const void* X, int v, double& x, double& y) {
-    const double* p = static_cast<const double*>(X);
-    x = __ldcg(p + 2 * v);
-    y = __ldcg(p + 2 * v + 1);
-}
-template <>
-__device__ __forceinline__ void load_pos_cg<float>(const void* X, int v, ff& x, ff& y) {
-    const float4 q = __ldcg(static_cast<const float4*>(X) + v);
-    x = ff{q.x, q.z};
-    y = ff{q.y, q.w};
-}
-
 // Eqs. verletPos / verletVel of a deformable dynamic particle: the vertex moves
 // by the interpolated velocity (the first tentative velocity) plus F / (2 m_v)
 // (F the total force of this step, m_v = rho_P A_0 / n); its velocity is the
@@ -56,13 +44,14 @@ __device__ __forceinline__ void load_pos_cg<float>(const void* X, int v, ff& x, 
 template <typename C>
 __device__ __forceinline__ void verlet(const MarkerArgs& a, int m, int v, typename Ext<C>::E x,
                                        typename Ext<C>::E y, typename Ext<C>::E xp, typename Ext<C>::E yp,
-                                       C Ux, C Uy, long long step, typename Ext<C>::E& xn,
+                                       C Ux, C Uy, long long step, bool store_v, typename Ext<C>::E& xn,
                                        typename Ext<C>::E& yn) {
     const C* F = static_cast<const C*>(a.F);
     C* V = static_cast<C*>(a.V);
     const C mv = C(a.mem_dyn[3 * m + 2]);
     xn = eaddc(x, Ux + (C(0.5) * F[2 * (size_t)v]) / mv);
     yn = eaddc(y, Uy + (C(0.5) * F[2 * (size_t)v + 1]) / mv);
+    if (!store_v) return;
     if (step == 0) {
         V[2 * (size_t)v] = etoc(esub(xn, x));
         V[2 * (size_t)v + 1] = etoc(esub(yn, y));
@@ -92,23 +81,23 @@ __device__ __forceinline__ void ring_boxes(const MarkerArgs& a, int m, int n, in
 // DYN: the context holds dynamic particles (without them their paths are not
 // compiled into the kernel, which keeps its code small)
 //
-// advance_unit is the body for advance unit `u` of the context `a`, whose
-// advance launch has `nblocks` blocks in all (the last of them to finish runs
-// the epilogue): the single-context kernel runs unit blockIdx.x of gridDim.x,
-// the batched kernel (ensembles) one unit of one member per block.
+// advance_unit is the body for advance unit `u` of the context `a`: the
+// single-context kernel runs unit blockIdx.x, the batched kernel (ensembles)
+// one unit of one member per block.
 //
 // Everything but the velocities is read before dep_wait(): the positions,
 // forces, weights and bonds were complete when the fused kernel (the
 // predecessor in a chained launch) let this one start.
 template <typename C, bool DYN>
-__device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigned nblocks) {
+__device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u) {
     using E = typename Ext<C>::E;
     const int4 u0 = a.au[2 * u], u1 = a.au[2 * u + 1];
     const int m = u0.x, k0 = u0.y, kn = u0.z, off = u0.w, n = u1.x, kind = u1.y;
     const int tid = threadIdx.x, lane = tid & 31;
     __shared__ E s_x[kAdvThreads], s_y[kAdvThreads];
-    __shared__ C cred[4 * 33];
-    __shared__ bool s_last;
+    __shared__ C cred[2][4][8];
+    __shared__ int s_np;  // formation candidates listed
+    if (tid == 0) s_np = 0;
     const long long step = *a.d_step;
     C* U = static_cast<C*>(a.U);
     // the unit's ligand records and current bonds, fetched now so that their
@@ -124,28 +113,40 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigne
 
     if (kind == LBIB_MEMBRANE_KINEMATIC || (DYN && kind == LBIB_MEMBRANE_DYNAMIC)) {
         // ---- kinematic or deformable dynamic chunk: one vertex per thread
-        const bool valid = tid < kn;
-        const int v = off + k0 + (valid ? tid : 0);
+        // (and one thread for the next chunk's first vertex, where this unit's
+        // ligands may need it: read from the halo records, nothing stored)
+        const bool mine = tid < kn;
+        const bool next = tid == kn && nlq > 0 && kn < n;
+        const bool wraps = k0 + kn == n;
+        const int v = off + (mine ? k0 + tid : (next && !wraps ? k0 + kn : (next ? 0 : k0)));
         E x, y, xp, yp, xn, yn;
-        load_pos<C>(a, v, x, y);
-        PosIO<C>::load(a.Xp, v, xp, yp);
+        if (next) {
+            const int un = wraps ? u - k0 / kChunkV : u + 1;
+            PosIO<C>::load(a.halo, 2 * un, x, y);
+            PosIO<C>::load(a.halo, 2 * un + 1, xp, yp);
+        } else {
+            load_pos<C>(a, v, x, y);
+            PosIO<C>::load(a.Xp, v, xp, yp);
+        }
         const Shape<C> sh = load_shape<C>(a, v);
         dep_wait();
         dep_trigger();
-        if (valid) {
+        if (mine || next) {
             C Ux, Uy;
             interp_vertex<C>(a, sh, Ux, Uy);
-            U[2 * v] = Ux;
-            U[2 * v + 1] = Uy;
             if (DYN && kind == LBIB_MEMBRANE_DYNAMIC) {
-                verlet<C>(a, m, v, x, y, xp, yp, Ux, Uy, step, xn, yn);
+                verlet<C>(a, m, v, x, y, xp, yp, Ux, Uy, step, mine, xn, yn);
             } else {
                 bdf2<C>(x, xp, Ux, step, xn);
                 bdf2<C>(y, yp, Uy, step, yn);
             }
-            if (!isfinite(ehi(xn)) || !isfinite(ehi(yn))) atomicOr(a.status, ST_NONFINITE);
-            PosIO<C>::store(a.Xp, v, x, y);
-            PosIO<C>::store(a.X, v, xn, yn);
+            if (mine) {
+                U[2 * v] = Ux;
+                U[2 * v + 1] = Uy;
+                if (!isfinite(ehi(xn)) || !isfinite(ehi(yn))) atomicOr(a.status, ST_NONFINITE);
+                PosIO<C>::store(a.Xp, v, x, y);
+                PosIO<C>::store(a.X, v, xn, yn);
+            }
             s_x[tid] = xn;
             s_y[tid] = yn;
         } else {
@@ -158,7 +159,7 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigne
         E gx, gy;
         shfl_e(gx, xn, lane & ~(kSegV - 1));
         shfl_e(gy, yn, lane & ~(kSegV - 1));
-        seg_box_regs<C>(a, sg, lane, valid ? xn : gx, valid ? yn : gy);
+        seg_box_regs<C>(a, sg, lane, mine ? xn : gx, mine ? yn : gy);
     } else if (DYN && kind == LBIB_MEMBRANE_DYNAMIC_RIGID) {
         // ---- rigid dynamic particle, the whole ring in this block: Eqs.
         // linearVelRig / angularVelRig.  F and its moment M about the area
@@ -190,14 +191,14 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigne
         // area centroid relative to vertex 0 from the triangles (vertex 0, k, k+1)
         const C cr = ax * by - ay * bx;
         C s2 = cr, gsx = cr * (ax + bx), gsy = cr * (ay + by), z0 = 0;
-        block_sum4_c<C>(s2, gsx, gsy, z0, cred);
+        block_sum4_c<C>(s2, gsx, gsy, z0, cred[0]);
         const C gx = gsx / (C(3) * s2), gy = gsy / (C(3) * s2);
         const C rx = ax - gx, ry = ay - gy;
         // the rigid state is read by every thread before thread 0 rewrites it
         double* rb = a.rb + 6 * m;
         const double u0 = rb[0], v0 = rb[1], up = rb[2], vp = rb[3], w0 = rb[4], wp = rb[5];
         C Fx = fx, Fy = fy, Mz = valid ? rx * fy - ry * fx : C(0), z1 = 0;
-        block_sum4_c<C>(Fx, Fy, Mz, z1, cred);
+        block_sum4_c<C>(Fx, Fy, Mz, z1, cred[1]);
         const double mass = a.mem_dyn[3 * m], inertia = a.mem_dyn[3 * m + 1];
         const double axd = double(Fx) / mass, ayd = double(Fy) / mass, ald = double(Mz) / inertia;
         double un, vn, wn;
@@ -261,7 +262,7 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigne
         }
         // least-squares rigid motion U_c + omega x (x - x_c), positions about vertex 0
         const C inv_n = C(1) / C(n);
-        block_sum4_c<C>(sx, sy, su, sv, cred);
+        block_sum4_c<C>(sx, sy, su, sv, cred[0]);
         const C mx = sx * inv_n, my = sy * inv_n, mu = su * inv_n, mv = sv * inv_n;
         C num = 0, den = 0;
         if (valid) {
@@ -270,7 +271,7 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigne
             den = rx * rx + ry * ry;
         }
         C z0 = 0, z1 = 0;
-        block_sum4_c<C>(num, den, z0, z1, cred);
+        block_sum4_c<C>(num, den, z0, z1, cred[1]);
         const C om = num / den;
         if (valid) {
             const int v = off + k;
@@ -292,7 +293,7 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigne
     }
     __syncthreads();
 
-    // ---- bond decisions for the ligands whose element lies inside this unit.
+    // ---- bond decisions for the ligands whose element starts in this unit.
     // (a) per ligand: rupture test of its bond, and the receptors of the 3x3
     //     cells around it that were free at the start of the step, as
     //     (ligand, receptor) pairs;
@@ -304,9 +305,6 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigne
         __shared__ int s_best[kAdvThreads];
         __shared__ int s_look[kAdvThreads];
         __shared__ int s_lig[kAdvThreads], s_ka[kAdvThreads], s_kb[kAdvThreads];
-        __shared__ int s_np;
-        if (tid == 0) s_np = 0;
-        __syncthreads();
         for (int q = tid; q < nlq; q += blockDim.x) {
             const int4 rec = my_rec;  // q == tid: a unit has no more ligands than threads
             const int l = rec.x, ka = rec.y, kb = rec.z;
@@ -345,6 +343,7 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigne
             }
         }
         __syncthreads();
+        if (s_np == 0) return;  // no receptor near any of the unit's ligands
         const int np = s_np < kMaxPairs ? s_np : kMaxPairs;
         for (int t = tid; t < np; t += blockDim.x) {
             const int q = s_pl[t], p = s_pr[t];
@@ -367,42 +366,22 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u, unsigne
             }
         }
     }
-
-    // ---- epilogue of the last block: straddling ligands, apply, next step
-    if (!arrive_last(&a.tickets[0], &s_last, nblocks)) return;
-    for (int q = tid; q < (a.nrec > 0 ? a.nstrad : 0); q += blockDim.x) {
-        const int l = a.strad_ligs[q];
-        E xa, ya, xb, yb;
-        load_pos_cg<C>(a.X, a.lig_a[l], xa, ya);
-        load_pos_cg<C>(a.X, a.lig_b[l], xb, yb);
-        LigandPoint<C> lp;
-        lp.init(xa, ya, xb, yb);
-        bond_decide<C>(a, l, lp, step);
-    }
-    __syncthreads();
-    if (a.nlig > 0 && a.nrec > 0) bond_apply_all(a);
-    __syncthreads();
-    if (tid == 0) {
-        *a.d_step += 1;
-        a.tickets[0] = 0;
-    }
 }
 
 template <typename C, bool DYN>
 __global__ void __launch_bounds__(kAdvThreads) k_advance(const MarkerArgs a) {
-    advance_unit<C, DYN>(a, blockIdx.x, gridDim.x);
+    advance_unit<C, DYN>(a, blockIdx.x);
 }
 
 // Batched form: the advance units of up to kBatchMax contexts (ensemble
-// members) in one launch, one block per (member, unit); each member's last
-// block runs its epilogue.  Blocks have the threads of the widest member (idle
+// members) in one launch, one block per (member, unit).  Blocks have the threads of the widest member (idle
 // threads beyond a unit's vertices, as in the single-context kernel).
 template <typename C, bool DYN>
 __global__ void __launch_bounds__(kAdvThreads) k_advance_batch(const __grid_constant__ MarkerBatch b) {
     __shared__ MarkerArgs s_a;
     const int m = marker_member(b, blockIdx.x);
     stage_args(&s_a, b.args + m);
-    advance_unit<C, DYN>(s_a, blockIdx.x - b.off[m], (unsigned)s_a.nau);
+    advance_unit<C, DYN>(s_a, blockIdx.x - b.off[m]);
 }
 
 template <typename C>

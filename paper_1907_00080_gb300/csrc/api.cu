@@ -238,7 +238,7 @@ extern "C" lbib_status lbib_create(const lbib_lattice* lat, double tau, const do
     c->n_partials = 1024;
     if (e == cudaSuccess) e = cudaMalloc(&c->partials, sizeof(double) * c->n_partials);
     if (e == cudaSuccess) e = cudaMalloc(&c->dscalar, sizeof(double) * 8);
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_step, sizeof(long long));
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_step, 2 * sizeof(long long));
     if (e == cudaSuccess) e = cudaMalloc(&c->d_status, sizeof(int));
     if (e != cudaSuccess) {
         lbib_destroy(c);
@@ -246,7 +246,7 @@ extern "C" lbib_status lbib_create(const lbib_lattice* lat, double tau, const do
     }
     e = cudaMemsetAsync(c->ux, 0, N * c->cmp_elem, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->uy, 0, N * c->cmp_elem, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_step, 0, sizeof(long long), c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_step, 0, 2 * sizeof(long long), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = init_populations(c);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -448,22 +448,26 @@ static lbib_status finalize(lbib_ctx* c) {
     }
     // work units, kUnitInts ints each (one 32-byte read per block):
     // {membrane, first local vertex, vertex count, membrane offset, membrane size,
-    //  kind, then for force units the membrane's first segment, for advance
-    //  units the first ligand record and the number of ligand records}
+    //  kind, then for force units the membrane's first segment and the advance
+    //  unit of the same chunk (-1: whole ring), for advance units the first
+    //  ligand record and the number of ligand records}
     std::vector<int> fu, au;
     for (int m = 0; m < nm; ++m) {
         const int n = c->h_mem_n[m], off = c->h_mem_off[m], kind = c->h_mem_kind[m];
         for (int k0 = 0; k0 < n; k0 += kChunkV) {
-            fu.insert(fu.end(), {m, k0, std::min(kChunkV, n - k0), off, n, kind, mem_seg_off[m], 0});
+            const int u = whole_ring(kind) ? -1 : (int)(au.size() / kUnitInts);
+            fu.insert(fu.end(), {m, k0, std::min(kChunkV, n - k0), off, n, kind, mem_seg_off[m], u});
             if (!whole_ring(kind)) au.insert(au.end(), {m, k0, std::min(kChunkV, n - k0), off, n, kind, 0, 0});
         }
         if (whole_ring(kind)) au.insert(au.end(), {m, 0, n, off, n, kind, 0, 0});
     }
-    // ligands decided inside each advance unit (both element vertices in it),
-    // as records {ligand, local index of its element's two vertices, 0}, and
-    // the straddling rest, decided by the kernel's last block
+    // ligands of each advance unit (that of their element's first vertex), as
+    // records {ligand, local index of its element's two vertices, 0}; an
+    // element that ends in the ring's next unit has the local index after the
+    // unit's last vertex there, which takes one thread more
     const int nau = (int)(au.size() / kUnitInts);
-    std::vector<int> au_ligs, strad;
+    std::vector<int> au_ligs;
+    int adv_threads = kChunkV;
     {
         std::vector<std::vector<int>> per(nau);
         std::vector<int> unit_of(std::max(nv, 1), -1);
@@ -471,16 +475,16 @@ static lbib_status finalize(lbib_ctx* c) {
             const int* u = &au[kUnitInts * q];
             for (int k = 0; k < u[2]; ++k) unit_of[u[3] + u[1] + k] = q;
         }
-        for (int l = 0; l < nl; ++l) {
-            const int ua = unit_of[lig_a[l]], ub = unit_of[lig_b[l]];
-            if (ua == ub) per[ua].push_back(l);
-            else strad.push_back(l);
-        }
+        for (int l = 0; l < nl; ++l) per[unit_of[lig_a[l]]].push_back(l);
         for (int q = 0; q < nau; ++q) {
             int* u = &au[kUnitInts * q];
             u[6] = (int)(au_ligs.size() / 4);
             u[7] = (int)per[q].size();  // <= vertices of the unit <= 4 kChunkV (one per advance thread)
-            for (int l : per[q]) au_ligs.insert(au_ligs.end(), {l, lig_a[l] - u[3] - u[1], lig_b[l] - u[3] - u[1], 0});
+            adv_threads = std::max(adv_threads, u[2] + (u[7] > 0 && u[2] < u[4] ? 1 : 0));
+            for (int l : per[q]) {
+                const int second = unit_of[lig_b[l]] == q ? lig_b[l] - u[3] - u[1] : u[2];
+                au_ligs.insert(au_ligs.end(), {l, lig_a[l] - u[3] - u[1], second, 0});
+            }
         }
     }
 
@@ -515,12 +519,12 @@ static lbib_status finalize(lbib_ctx* c) {
         add(16 * nv); add(16 * nv); add(2 * cs * nv); add(2 * cs * nv); add(9 * cs * nv); add(8 * nv);
         add(32 * nv); add(4 * nv); add(16 * nv + 16 * nr);
         add(4 * c->nseg); add(4 * c->nseg); add(4 * c->nseg); add(16 * c->nseg); add(4 * (nm + 1));
-        add(4 * nl); add(4 * nl); add(4 * nl); add(4 * nl); add(4 * nl);
+        for (int k = 0; k < 8; ++k) add(4 * nl);
         add(16 * nr); add(16 * nr); add(4 * nr); add(4 * nr); add(4 * rcell_start.size()); add(4 * rcell_ids.size()); add(16 * nr);
-        add(4 * nr); add(4 * nr);
-        add(4 * c->ntiles); add(4 * c->ntiles); add(8 * (nm + 1)); add(16);
+        add(4 * nr); add(4 * nr); add(4 * nr);
+        add(4 * c->ntiles); add(4 * c->ntiles); add(8 * (nm + 1));
         add(4 * fu.size()); add(4 * au.size());
-        add(4 * au_ligs.size()); add(4 * strad.size());
+        add(4 * au_ligs.size()); add(32 * (size_t)nau);
         add(2 * cs * nv); add(2 * cs * nv); add(2 * cs * nv); add(48 * (nm + 1)); add(24 * (nm + 1));
         add(4 * hydro_units.size());
         bytes = probe.used + 256;
@@ -561,26 +565,27 @@ static lbib_status finalize(lbib_ctx* c) {
     int* d_mem_seg_off = ar.take<int>(nm + 1);
     int* d_lig_a = ar.take<int>(nl);
     int* d_lig_b = ar.take<int>(nl);
-    a.bond_of_lig = ar.take<int>(nl);
-    a.cand = ar.take<int>(nl);
-    a.rupt = ar.take<int>(nl);
+    for (int q = 0; q < 2; ++q) {
+        c->bond[q] = ar.take<int>(nl);
+        c->cand[q] = ar.take<int>(nl);
+        c->rupt[q] = ar.take<int>(nl);
+    }
     double* rec_xy = ar.take<double>(2 * (size_t)nr);
     void* rec_e = ar.take<double>(2 * (size_t)nr);
     a.owner = ar.take<int>(nr);
     a.owner_cell = ar.take<int>(nr);
     int* d_rcell_of_rec = ar.take<int>(nr);
-    a.claim = ar.take<int>(nr);
+    for (int q = 0; q < 2; ++q) c->claim[q] = ar.take<int>(nr);
     int* d_rcs = ar.take<int>(rcell_start.size());
     int* d_rci = ar.take<int>(rcell_ids.size());
     void* d_rcpos = ar.take<double>(2 * (size_t)nr);
     c->flags[0] = ar.take<int>(c->ntiles);
     c->flags[1] = ar.take<int>(c->ntiles);
     c->d_areas = ar.take<double>(nm + 1);
-    c->tickets = ar.take<unsigned int>(4);
     int* d_fu = ar.take<int>(fu.size());
     int* d_au = ar.take<int>(au.size());
     int* d_au_ligs = ar.take<int>(au_ligs.size());
-    int* d_strad = ar.take<int>(strad.size());
+    a.halo = ar.take<double>(4 * (size_t)nau);
     void* V = ar.take<char>(2 * cs * nv);
     void* Hf = ar.take<char>(2 * cs * nv);
     void* Dib = ar.take<char>(2 * cs * nv);
@@ -615,7 +620,6 @@ static lbib_status finalize(lbib_ctx* c) {
         CK(H2D(d_fu, fu.data(), 4 * fu.size()));
         CK(H2D(d_au, au.data(), 4 * au.size()));
         if (!au_ligs.empty()) CK(H2D(d_au_ligs, au_ligs.data(), 4 * au_ligs.size()));
-        if (!strad.empty()) CK(H2D(d_strad, strad.data(), 4 * strad.size()));
         CK(cudaMemsetAsync(V, 0, 2 * cs * nv, c->stream));
         CK(cudaMemsetAsync(Hf, 0, 2 * cs * nv, c->stream));
         CK(cudaMemsetAsync(Dib, 0, 2 * cs * nv, c->stream));
@@ -627,16 +631,15 @@ static lbib_status finalize(lbib_ctx* c) {
     if (nl > 0) {
         CK(H2D(d_lig_a, lig_a.data(), 4 * nl));
         CK(H2D(d_lig_b, lig_b.data(), 4 * nl));
-        CK(cudaMemsetAsync(a.bond_of_lig, 0xFF, 4 * nl, c->stream));
-        CK(cudaMemsetAsync(a.cand, 0xFF, 4 * nl, c->stream));
-        CK(cudaMemsetAsync(a.rupt, 0xFF, 4 * nl, c->stream));
+        for (int q = 0; q < 2; ++q)
+            for (int* p : {c->bond[q], c->cand[q], c->rupt[q]}) CK(cudaMemsetAsync(p, 0xFF, 4 * nl, c->stream));
     }
     if (nr > 0) {
         CK(H2D(rec_xy, c->h_rec.data(), 16 * (size_t)nr));
         CK(launch_pos_in(c->prec, rec_xy, rec_e, nr, c->stream));
         CK(cudaMemsetAsync(a.owner, 0xFF, 4 * nr, c->stream));
         CK(cudaMemsetAsync(a.owner_cell, 0xFF, 4 * nr, c->stream));
-        CK(cudaMemsetAsync(a.claim, 0x7F, 4 * nr, c->stream));  // 0x7F7F7F7F: no claim
+        for (int q = 0; q < 2; ++q) CK(cudaMemsetAsync(c->claim[q], 0x7F, 4 * nr, c->stream));  // 0x7F7F7F7F: no claim
     }
     CK(H2D(d_rcs, rcell_start.data(), 4 * rcell_start.size()));
     if (!rcell_ids.empty()) {
@@ -656,7 +659,6 @@ static lbib_status finalize(lbib_ctx* c) {
     }
     CK(cudaMemsetAsync(c->flags[0], 0, 4 * c->ntiles, c->stream));
     CK(cudaMemsetAsync(c->flags[1], 0, 4 * c->ntiles, c->stream));
-    CK(cudaMemsetAsync(c->tickets, 0, 16, c->stream));
     if (nv > 0) {
         const size_t gb = sizeof(longlong2) * (size_t)c->nx * c->ny;
         for (int p = 0; p < 2; ++p) {
@@ -671,14 +673,10 @@ static lbib_status finalize(lbib_ctx* c) {
     a.d_rep = c->d_rep; a.nseg = c->nseg;
     a.seg_mem = d_seg_mem; a.seg_v0 = d_seg_v0; a.seg_n = d_seg_n; a.mem_seg_off = d_mem_seg_off;
     a.nfu = (int)(fu.size() / kUnitInts); a.nau = nau;
-    // advance blocks: one thread per vertex of the longest rigid ring, at least
-    // a chunk; small blocks leave room for other work (ensembles) on the SMs
-    {
-        int longest = kChunkV;
-        for (int m = 0; m < nm; ++m)
-            if (whole_ring(c->h_mem_kind[m])) longest = std::max(longest, c->h_mem_n[m]);
-        a.adv_threads = (longest + 31) / 32 * 32;
-    }
+    // advance blocks: one thread per vertex of the largest unit (a chunk, with
+    // its ligands' one vertex more, or a rigid ring); small blocks leave room
+    // for other work (ensembles) on the SMs
+    a.adv_threads = (adv_threads + 31) / 32 * 32;
     // dynamic particles: states at rest, the ids for the hydrodynamic kernel
     a.V = V; a.Hf = Hf; a.Dib = Dib; a.rb = rb; a.mem_dyn = mem_dyn; a.has_dyn = c->ndyn > 0 ? 1 : 0;
     c->d_hydro_units = reinterpret_cast<int4*>(d_hydro_units);
@@ -686,7 +684,6 @@ static lbib_status finalize(lbib_ctx* c) {
     a.fu = reinterpret_cast<const int4*>(d_fu);
     a.au = reinterpret_cast<const int4*>(d_au);
     a.au_ligs = reinterpret_cast<const int4*>(d_au_ligs);
-    a.nstrad = (int)strad.size(); a.strad_ligs = d_strad;
     a.nlig = nl; a.nrec = nr; a.lig_a = d_lig_a; a.lig_b = d_lig_b;
     a.rec_xy = rec_xy; a.rec_e = rec_e; a.rcell_start = d_rcs; a.rcell_ids = d_rci; a.rcell_pos = d_rcpos;
     a.rcell_of_rec = d_rcell_of_rec;
@@ -698,7 +695,7 @@ static lbib_status finalize(lbib_ctx* c) {
     a.kf_dt = c->bp.kf_dt; a.kr0_dt = c->bp.kr0_dt; a.beta_f = c->bp.beta_f; a.beta_r = c->bp.beta_r;
     a.seed = c->bp.seed; a.instance = c->bp.instance;
     a.tile_w = c->tile_w; a.tile_h = c->tile_h; a.tiles_x = c->tiles_x; a.tiles_y = c->tiles_y;
-    a.d_step = c->d_step; a.status = c->d_status; a.tickets = c->tickets;
+    a.status = c->d_status;
     a.f.nx = (float)c->nx; a.f.ny = (float)c->ny; a.f.inv_nx = (float)a.inv_nx; a.f.inv_ny = (float)a.inv_ny;
     a.f.sigma = (float)a.sigma; a.f.y_eq = (float)a.y_eq; a.f.inv_y_eq = (float)a.inv_y_eq;
     a.f.d_rep = (float)a.d_rep; a.f.d_cut = (float)a.d_cut; a.f.d_break = (float)a.d_break;
@@ -791,6 +788,24 @@ static cudaError_t launch_fused(const lbib_ctx* c, const LbArgs& l, cudaStream_t
     return launch_lb_step(c->prec, c->vec, c->ty, walls, c->nv > 0, l, s, chained);
 }
 
+// the marker arguments of a step that starts from population buffer `src`
+static MarkerArgs marker_args(const lbib_ctx* c, int src) {
+    MarkerArgs a = c->ma;
+    a.gsum = c->G[src];
+    a.flags = c->flags[src];
+    a.bond_of_lig = c->bond[src];
+    a.cand = c->cand[src];
+    a.rupt = c->rupt[src];
+    a.claim = c->claim[src];
+    a.bond_prev = c->bond[1 - src];
+    a.cand_prev = c->cand[1 - src];
+    a.rupt_prev = c->rupt[1 - src];
+    a.claim_prev = c->claim[1 - src];
+    a.d_step = c->d_step + src;
+    a.step_prev = c->d_step + (1 - src);
+    return a;
+}
+
 // Whether the advance kernel starts beside the fused kernel's tail.  Its
 // early blocks gather on the SMs that the fused kernel leaves first: with
 // thousands of blocks (64-member ensemble: 2720, FP16 step 174 -> 183 us) or
@@ -801,18 +816,18 @@ static bool chain_advance(lbib_precision prec, int nunits) { return prec != LBIB
 // one time step from population buffer `src`: forces + weights + spreading,
 // fused collide-stream, interpolation + advance, bond kinetics.  The launches
 // of a step are chained (see dep_wait); `first` marks the first step of a
-// captured sequence, whose first kernel has no predecessor of the cycle
-static cudaError_t enqueue_step(lbib_ctx* c, int src, cudaStream_t s, bool first) {
-    MarkerArgs a = c->ma;
-    a.gsum = c->G[src];
-    a.flags = c->flags[src];
+// captured sequence, whose first kernel has no predecessor of the cycle (the
+// sequence before it settled its bond decisions), `last` the last one
+static cudaError_t enqueue_step(lbib_ctx* c, int src, cudaStream_t s, bool first, bool last) {
+    const MarkerArgs a = marker_args(c, src);
     cudaError_t e;
     const bool has_ib = c->nv > 0;
     if (c->ndyn > 0 && (e = launch_hydro(c->prec, a, hydro_args(c, src), s, !first)) != cudaSuccess) return e;
-    if (has_ib && (e = launch_forces(c->prec, a, s, !first || c->ndyn > 0)) != cudaSuccess) return e;
+    if (has_ib && (e = launch_forces(c->prec, a, !first, s, !first || c->ndyn > 0)) != cudaSuccess) return e;
     const LbArgs l = lb_args(c, src, src, 1);
     if ((e = launch_fused(c, l, s, !first || has_ib)) != cudaSuccess) return e;
     if (has_ib && (e = launch_advance(c->prec, a, s, chain_advance(c->prec, a.nau))) != cudaSuccess) return e;
+    if (has_ib && last && (e = launch_settle(marker_args(c, 1 - src), s)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
@@ -844,7 +859,7 @@ static lbib_status build_graphs(lbib_ctx* c) {
             int src = start;
             cudaError_t le = cudaSuccess;
             for (int k = 0; k < nsteps && le == cudaSuccess; ++k) {
-                le = enqueue_step(c, src, cap, k == 0);
+                le = enqueue_step(c, src, cap, k == 0, k == nsteps - 1);
                 src = 1 - src;
             }
             e = cudaStreamEndCapture(cap, &g);
@@ -1112,7 +1127,7 @@ extern "C" lbib_status lbib_read_bonds(lbib_ctx* c, int32_t* lig, int32_t* rec, 
     if (st != LBIB_OK) return st;
     std::vector<int> b(c->nlig);
     if (c->nlig > 0) {
-        CK(cudaMemcpyAsync(b.data(), c->ma.bond_of_lig, 4 * (size_t)c->nlig, cudaMemcpyDeviceToHost, c->stream));
+        CK(cudaMemcpyAsync(b.data(), c->bond[c->cur], 4 * (size_t)c->nlig, cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
     }
     int cnt = 0;
@@ -1152,7 +1167,7 @@ extern "C" lbib_status lbib_membrane_observables(lbib_ctx* c, double* out) {
     if (st != LBIB_OK) return st;
     if (c->nmem == 0) return LBIB_OK;
     if (!c->d_obs) CK(cudaMalloc(&c->d_obs, 8 * sizeof(double) * (size_t)c->nmem));
-    CK(launch_observables(c->prec, c->ma, c->d_obs, c->stream));
+    CK(launch_observables(c->prec, marker_args(c, c->cur), c->d_obs, c->stream));
     CK(cudaMemcpyAsync(out, c->d_obs, 8 * sizeof(double) * (size_t)c->nmem, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     return LBIB_OK;
@@ -1211,12 +1226,10 @@ extern "C" lbib_status lbib_profile_kernels(lbib_ctx* c, int32_t reps, double* m
     cudaEvent_t ev[6];
     for (int k = 0; k < 6; ++k) CK(cudaEventCreate(&ev[k]));
     const bool has_ib = c->nv > 0;
-    MarkerArgs a = c->ma;
-    a.gsum = c->G[c->cur];
-    a.flags = c->flags[c->cur];
+    const MarkerArgs a = marker_args(c, c->cur);
     // forces + spreading (accumulates into the field of the current parity)
     CK(cudaEventRecord(ev[0], c->stream));
-    for (int r = 0; r < reps && has_ib; ++r) CK(launch_forces(c->prec, a, c->stream));
+    for (int r = 0; r < reps && has_ib; ++r) CK(launch_forces(c->prec, a, false, c->stream));
     CK(cudaEventRecord(ev[1], c->stream));
     // fused collide-stream, ping-pong between the buffers
     const int gpar = 1 - c->cur;
@@ -1372,10 +1385,7 @@ static lbib_status ensemble_batch_tables(lbib_ensemble* e, int ngroups) {
             lbib_ctx* c = e->m[i];
             for (int p = 0; p < 2; ++p) {
                 const int src = e->cur0[i] ^ p;
-                MarkerArgs a = c->ma;
-                a.gsum = c->G[src];
-                a.flags = c->flags[src];
-                ma[p * n + i] = a;
+                ma[p * n + i] = marker_args(c, src);
             }
         }
         ECK(cudaMalloc(&e->margs, sizeof(MarkerArgs) * 2 * n));
@@ -1409,7 +1419,7 @@ static lbib_status ensemble_batch_tables(lbib_ensemble* e, int ngroups) {
                 fb.off[k] = fu;
                 ab.off[k] = au;
                 kb += gx * gy;
-                fu += c->ma.nfu;
+                fu += c->ma.nfu + 1;  // and the block that settles the member's bonds
                 au += c->ma.nau;
                 e->adv_threads = std::max(e->adv_threads, c->ma.adv_threads);
             }
@@ -1430,15 +1440,17 @@ static lbib_status ensemble_batch_tables(lbib_ensemble* e, int ngroups) {
 
 // one time step of every member of group g in the batched form, at phase p
 // (first: of a captured sequence, see enqueue_step)
-static cudaError_t ensemble_batch_step(const lbib_ensemble* e, int g, int p, cudaStream_t s, bool first) {
+static cudaError_t ensemble_batch_step(lbib_ensemble* e, int g, int p, cudaStream_t s, bool first, bool last) {
     const lbib_ctx* c0 = e->m[0];
     const bool walls = c0->walls != LBIB_WALLS_NONE;
+    e->fbb[p][g].settle = first ? 0 : 1;
     cudaError_t r = launch_forces_batch(c0->prec, e->fbb[p][g], s, !first);
     if (r == cudaSuccess)
         r = c0->ty > 0 ? launch_lb_batch(c0->prec, c0->vec, c0->ty, walls, e->lbb[p][g], s, true)
                        : launch_lb_stream_batch(c0->prec, c0->vec, walls, e->stream_grid, e->lbb[p][g], s, true);
     if (r == cudaSuccess) r = launch_advance_batch(c0->prec, false, e->abb[p][g], e->adv_threads, s,
                                                        chain_advance(c0->prec, e->abb[p][g].off[e->abb[p][g].n]));
+    if (r == cudaSuccess && last) r = launch_settle_batch(e->fbb[1 - p][g].args, e->fbb[1 - p][g].n, s);
     return r;
 }
 
@@ -1464,7 +1476,7 @@ static lbib_status ensemble_build_batched(lbib_ensemble* e, int ngroups) {
             for (int g = 0; g < G && le == cudaSuccess; ++g) {
                 cudaStream_t s = G == 1 ? cap : gs[g];
                 if (G > 1) le = cudaStreamWaitEvent(s, ev[G], 0);
-                for (int k = 0; k < nsteps && le == cudaSuccess; ++k) le = ensemble_batch_step(e, g, flip ^ (k & 1), s, k == 0);
+                for (int k = 0; k < nsteps && le == cudaSuccess; ++k) le = ensemble_batch_step(e, g, flip ^ (k & 1), s, k == 0, k == nsteps - 1);
                 if (G > 1 && le == cudaSuccess) le = cudaEventRecord(ev[g], s);
                 if (G > 1 && le == cudaSuccess) le = cudaStreamWaitEvent(cap, ev[g], 0);
             }
@@ -1828,7 +1840,7 @@ extern "C" lbib_status lbib_tangent_step(lbib_tangent* t, int64_t n) {
     if (c->poisoned) return fail(c, LBIB_E_STATE, "context poisoned by an earlier device-side failure");
     for (int64_t k = 0; k < n; ++k) {
         TangentArgs a{};
-        a.m = c->ma;
+        a.m = marker_args(c, c->cur);
         a.f = static_cast<const double*>(c->f[c->cur]);
         a.fd_src = t->fd[t->cf];
         a.fd_dst = t->fd[1 - t->cf];
@@ -1927,11 +1939,11 @@ cudaError_t snap_copy(lbib_ctx* c, Snap& s, bool to_snap) {
     if ((e = cp(s.f, c->f[c->cur], 9 * N * c->pop_elem)) != cudaSuccess) return e;
     if ((e = cp(s.X, c->ma.X, 16 * nv)) != cudaSuccess) return e;
     if ((e = cp(s.Xp, c->ma.Xp, 16 * nv)) != cudaSuccess) return e;
-    if ((e = cp(s.bond, c->ma.bond_of_lig, 4 * nlig)) != cudaSuccess) return e;
+    if ((e = cp(s.bond, c->bond[c->cur], 4 * nlig)) != cudaSuccess) return e;
     if ((e = cp(s.owner, c->ma.owner, 4 * nrec)) != cudaSuccess) return e;
     if ((e = cp(s.owner_cell, c->ma.owner_cell, 4 * nrec)) != cudaSuccess) return e;
     if ((e = cp(s.seg_box, c->ma.seg_box, sizeof(float4) * c->nseg)) != cudaSuccess) return e;
-    if ((e = cp(s.d_step, c->d_step, 8)) != cudaSuccess) return e;
+    if ((e = cp(s.d_step, c->d_step + c->cur, 8)) != cudaSuccess) return e;
     if (to_snap) s.step = c->steps;
     else c->steps = s.step;
     return cudaSuccess;
@@ -2141,14 +2153,14 @@ extern "C" lbib_status lbib_adjoint_reverse(lbib_adjoint* a) {
                 CopyList l{};
                 l.src[0] = c->f[c->cur]; l.dst[0] = a->tape_f + (size_t)k * 9 * N; l.words[0] = 18 * N;
                 l.src[1] = c->ma.X; l.dst[1] = a->tape_X + (size_t)k * 2 * nv; l.words[1] = 4 * nvr;
-                l.src[2] = c->ma.bond_of_lig; l.dst[2] = a->tape_bond + (size_t)k * nl; l.words[2] = (size_t)c->nlig;
+                l.src[2] = c->bond[c->cur]; l.dst[2] = a->tape_bond + (size_t)k * nl; l.words[2] = (size_t)c->nlig;
                 l.n = 3;
                 CK(launch_copy_words(l, c->stream));
             } else {
                 CK(launch_widen_storage(c->prec, c->f[c->cur], a->tape_f + (size_t)k * 9 * N, 9 * N, c->inv_scale,
                                         c->stream));
                 if (nvr) CK(launch_pos_out(c->prec, c->ma.X, a->tape_X + (size_t)k * 2 * nv, c->nv, c->stream));
-                if (c->nlig) CK(d2d(a->tape_bond + (size_t)k * nl, c->ma.bond_of_lig, 4 * (size_t)c->nlig));
+                if (c->nlig) CK(d2d(a->tape_bond + (size_t)k * nl, c->bond[c->cur], 4 * (size_t)c->nlig));
             }
             const int src = c->cur;
             CK(cudaGraphLaunch(c->graph[c->cur][0], c->stream));
@@ -2313,8 +2325,8 @@ struct StatePart {
 std::vector<StatePart> state_parts(lbib_ctx* c) {
     const size_t N = (size_t)c->nx * c->ny, nv = c->nv, nlig = c->nlig, nrec = c->ma.nrec;
     return {{c->f[c->cur], 9 * N * c->pop_elem}, {c->ma.X, 16 * nv},          {c->ma.Xp, 16 * nv},
-            {c->ma.bond_of_lig, 4 * nlig},       {c->ma.owner, 4 * nrec},     {c->ma.owner_cell, 4 * nrec},
-            {c->ma.seg_box, sizeof(float4) * (size_t)c->nseg},              {c->d_step, 8},
+            {c->bond[c->cur], 4 * nlig},       {c->ma.owner, 4 * nrec},     {c->ma.owner_cell, 4 * nrec},
+            {c->ma.seg_box, sizeof(float4) * (size_t)c->nseg},              {c->d_step + c->cur, 8},
             // dynamic particles: vertex velocities and rigid states
             {c->ma.V, c->ndyn > 0 ? 2 * c->cmp_elem * nv : 0},
             {c->ma.rb, c->ndyn > 0 ? 6 * sizeof(double) * (size_t)c->nmem : 0}};
@@ -2395,13 +2407,13 @@ extern "C" lbib_status lbib_load(lbib_ctx* c, const char* path) {
         if (c->G[p]) CK(cudaMemsetAsync(c->G[p], 0, sizeof(longlong2) * N, c->stream));
         if (c->flags[p]) CK(cudaMemsetAsync(c->flags[p], 0, 4 * (size_t)c->ntiles, c->stream));
     }
-    CK(cudaMemsetAsync(c->tickets, 0, 16, c->stream));
     CK(cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream));
     if (c->nlig > 0) {
-        CK(cudaMemsetAsync(c->ma.cand, 0xFF, 4 * (size_t)c->nlig, c->stream));
-        CK(cudaMemsetAsync(c->ma.rupt, 0xFF, 4 * (size_t)c->nlig, c->stream));
+        for (int q = 0; q < 2; ++q)
+            for (int* p : {c->cand[q], c->rupt[q]}) CK(cudaMemsetAsync(p, 0xFF, 4 * (size_t)c->nlig, c->stream));
     }
-    if (c->ma.nrec > 0) CK(cudaMemsetAsync(c->ma.claim, 0x7F, 4 * (size_t)c->ma.nrec, c->stream));
+    if (c->ma.nrec > 0)
+        for (int q = 0; q < 2; ++q) CK(cudaMemsetAsync(c->claim[q], 0x7F, 4 * (size_t)c->ma.nrec, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     c->steps = h.steps;
     c->poisoned = false;

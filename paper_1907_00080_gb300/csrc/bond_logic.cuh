@@ -180,52 +180,6 @@ __device__ __forceinline__ bool ruptures(const MarkerArgs& a, LigandPoint<C>& lp
     return u < p_rupture(a, d);
 }
 
-// One ligand, one thread: rupture test of its bond, then (if free) the lowest
-// receptor id that passes the formation test among the receptors of the 3x3
-// grid cells around the ligand point (cells are at least d_cut wide), claimed
-// with atomicMin so that the lowest ligand id wins.
-template <typename C>
-__device__ __forceinline__ void bond_decide(const MarkerArgs& a, int l, LigandPoint<C>& lp, long long step) {
-    if (!lp.finite()) return;  // reported by the advance
-    const int r = a.bond_of_lig[l];
-    if (r >= 0) {
-        if (!ruptures<C>(a, lp, step, l, r)) return;
-        a.rupt[l] = r;
-    }
-    const float cxh = float(ehi(lp.cx)), cyh = float(ehi(lp.cy));
-    const float xw = cxh - a.f.nx * floorf(cxh * a.f.inv_nx);
-    int gx = (int)floorf(xw * a.f.inv_rc_w);
-    gx = gx >= a.rc_nx ? a.rc_nx - 1 : (gx < 0 ? 0 : gx);
-    const int gy = (int)fminf(fmaxf(floorf((cyh - a.f.rc_y0) * a.f.inv_rc_h), -4.f), float(a.rc_ny) + 4.f);
-    // the three cell rows' ranges first (independent loads), then their receptors
-    int p0[9], p1[9];
-#pragma unroll
-    for (int c = 0; c < 9; ++c) {
-        const int qy = gy - 1 + c / 3, qx = gx - 1 + c % 3;
-        p0[c] = p1[c] = 0;
-        if (qy >= 0 && qy < a.rc_ny) {
-            const int cell = qy * a.rc_nx + ((qx % a.rc_nx) + a.rc_nx) % a.rc_nx;
-            p0[c] = a.rcell_start[cell];
-            p1[c] = a.rcell_start[cell + 1];
-        }
-    }
-    int best = INT_MAX;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) {
-        for (int p = p0[c]; p < p1[c]; ++p) {
-            const int rr = a.rcell_ids[p];
-            typename Ext<C>::E rx, ry;
-            PosIO<C>::load(a.rcell_pos, p, rx, ry);
-            if (rr >= best || a.owner_cell[p] >= 0) continue;  // bound at the start of the step
-            if (forms<C>(a, lp, step, l, rr, rx, ry)) best = rr;
-        }
-    }
-    if (best != INT_MAX) {
-        a.cand[l] = best;
-        atomicMin(&a.claim[best], l);
-    }
-}
-
 // 3x3 receptor-grid cells around a ligand point: the nine [p0, p1) ranges of
 // the cell-ordered receptor arrays (empty outside the grid's rows)
 template <typename C>
@@ -240,71 +194,50 @@ __device__ __forceinline__ void ligand_cells(const MarkerArgs& a, const LigandPo
         const int qy = gy - 1 + c / 3, qx = gx - 1 + c % 3;
         p0[c] = p1[c] = 0;
         if (qy >= 0 && qy < a.rc_ny) {
-            const int cell = qy * a.rc_nx + ((qx % a.rc_nx) + a.rc_nx) % a.rc_nx;
+            // (qx lies in -1 .. rc_nx)
+            const int cell = qy * a.rc_nx + (qx < 0 ? qx + a.rc_nx : (qx >= a.rc_nx ? qx - a.rc_nx : qx));
             p0[c] = a.rcell_start[cell];
             p1[c] = a.rcell_start[cell + 1];
         }
     }
 }
 
-// Epilogue run by one block after every ligand has been decided: apply the
-// ruptures and the winning claims, clear the claims, advance the step counter.
-// Data written by other blocks is read past L1.
-static __device__ __forceinline__ void bond_apply_all(const MarkerArgs& a) {
-    // ruptures free their receptor, won claims bind it; owner is kept both by
-    // receptor id and in cell order (owner_cell, read by the formation tests)
-    constexpr int kPer = 4;  // ligands per thread per pass, loads issued together
-    const bool one_pass = a.nlig <= kPer * (int)blockDim.x;
-    int keep_c[kPer];
-    for (int base = 0; base < a.nlig; base += kPer * blockDim.x) {
-        int q[kPer], r_old[kPer], c[kPer], cl[kPer], pr[kPer], pc[kPer];
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            q[i] = base + threadIdx.x + i * blockDim.x;
-            r_old[i] = q[i] < a.nlig ? __ldcg(&a.rupt[q[i]]) : -1;
-            c[i] = q[i] < a.nlig ? __ldcg(&a.cand[q[i]]) : -1;
-            keep_c[i] = c[i];
-        }
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            cl[i] = c[i] >= 0 ? __ldcg(&a.claim[c[i]]) : -1;
-            pc[i] = c[i] >= 0 ? a.rcell_of_rec[c[i]] : -1;
-            pr[i] = r_old[i] >= 0 ? a.rcell_of_rec[r_old[i]] : -1;
-        }
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            if (r_old[i] >= 0) {
-                a.owner[r_old[i]] = -1;
-                a.owner_cell[pr[i]] = -1;
-                a.bond_of_lig[q[i]] = -1;
-                a.rupt[q[i]] = -1;
+// The bond of ligand l at the start of this step: the settled one, or (the
+// previous step's decisions not yet settled) the previous one changed by them:
+// a won claim binds, else a rupture frees.
+__device__ __forceinline__ int bond_now(const MarkerArgs& a, int l, bool settled) {
+    if (settled) return a.bond_of_lig[l];
+    const int b = a.bond_prev[l], c = a.cand_prev[l], r = a.rupt_prev[l];
+    if (c >= 0 && a.claim_prev[c] == l) return c;
+    return r >= 0 ? -1 : b;
+}
+
+// Settle the decisions of the previous step, all threads of one block: the
+// bonds and the step counter of this parity, the receptors' owners (by receptor
+// id and in cell order), and this parity's own decisions of two steps ago
+// cleared for the coming advance kernel.  A receptor that a rupture frees was
+// bound at the start of that step and one that is won was free, so no receptor
+// is written twice.
+static __device__ __forceinline__ void settle_bonds(const MarkerArgs& a) {
+    if (a.nrec > 0) {
+        for (int l = threadIdx.x; l < a.nlig; l += blockDim.x) {
+            const int b = a.bond_prev[l], c = a.cand_prev[l], r = a.rupt_prev[l], old = a.cand[l];
+            const bool won = c >= 0 && a.claim_prev[c] == l;
+            if (r >= 0) {
+                a.owner[r] = -1;
+                a.owner_cell[a.rcell_of_rec[r]] = -1;
             }
-            if (c[i] >= 0 && cl[i] == q[i]) {
-                a.bond_of_lig[q[i]] = c[i];
-                a.owner[c[i]] = q[i];
-                a.owner_cell[pc[i]] = q[i];
+            if (won) {
+                a.owner[c] = l;
+                a.owner_cell[a.rcell_of_rec[c]] = l;
             }
+            a.bond_of_lig[l] = won ? c : (r >= 0 ? -1 : b);
+            if (old >= 0) a.claim[old] = INT_MAX;
+            a.cand[l] = -1;
+            a.rupt[l] = -1;
         }
     }
-    __syncthreads();  // every claim has been read before any is cleared
-    if (one_pass) {
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            const int q = threadIdx.x + i * blockDim.x;
-            if (keep_c[i] >= 0) {
-                a.claim[keep_c[i]] = INT_MAX;
-                a.cand[q] = -1;
-            }
-        }
-    } else {
-        for (int q = threadIdx.x; q < a.nlig; q += blockDim.x) {
-            const int c = __ldcg(&a.cand[q]);
-            if (c >= 0) {
-                a.claim[c] = INT_MAX;
-                a.cand[q] = -1;
-            }
-        }
-    }
+    if (threadIdx.x == 0) *a.d_step = *a.step_prev + 1;
 }
 
 }  // namespace lbib

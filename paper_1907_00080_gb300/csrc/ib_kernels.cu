@@ -53,11 +53,11 @@ __global__ void k_rest(const MarkerArgs a, void* rest_v, double* A0, double* qa)
 // Eq. adhFor on element e (if its ligand is bonded), half to the vertex;
 // positions of the element's two vertices are given
 template <typename C, typename E>
-__device__ __forceinline__ void bond_on_element(const MarkerArgs& a, int e, E xa, E ya, E xb, E yb, C& Fx,
-                                                C& Fy) {
+__device__ __forceinline__ void bond_on_element(const MarkerArgs& a, int e, bool settled, E xa, E ya, E xb, E yb,
+                                                C& Fx, C& Fy) {
     const int l = a.elem_lig[e];
     if (l < 0) return;
-    const int r = a.bond_of_lig[l];
+    const int r = bond_now(a, l, settled);
     if (r < 0) return;
     E rx, ry;
     PosIO<C>::load(a.rec_e, r, rx, ry);
@@ -97,8 +97,14 @@ constexpr int kScreenIter = 8;                    // segment boxes per lane load
 // single-context kernel runs unit blockIdx.x, the batched kernel (ensembles)
 // one unit of one member per block.
 template <typename C>
-__device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit) {
+__device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool settle) {
     using E = typename Ext<C>::E;
+    if (unit == a.nfu) {  // one block more than units: the previous step's bond decisions
+        dep_wait();
+        dep_trigger();
+        if (settle) settle_bonds(a);
+        return;
+    }
     const int4 u0 = a.fu[2 * unit], u1 = a.fu[2 * unit + 1];
     const int m = u0.x, k0 = u0.y, kn = u0.z, off = u0.w, n = u1.x;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -135,6 +141,14 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit) {
         load_pos<C>(a, off + k, s_x[p], s_y[p]);
     }
     if (tid < kChunkV) s_rep[tid] = 0ull;
+    if (tid == 32 * 9 && u1.w >= 0 && a.nlig > 0) {
+        // this chunk's first vertex for the advance of the chunk before it
+        E xh, yh;
+        load_pos<C>(a, off + k0, xh, yh);
+        PosIO<C>::store(a.halo, 2 * u1.w, xh, yh);
+        PosIO<C>::load(a.Xp, off + k0, xh, yh);
+        PosIO<C>::store(a.halo, 2 * u1.w + 1, xh, yh);
+    }
     // the screening warps fetch this chunk's own segment boxes now (the unit
     // record carries the membrane's first segment), behind the position loads
     const int sown0 = u1.z + k0 / kSegV;
@@ -370,8 +384,8 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit) {
             const int sj = j + 1;  // geometry slot of vertex k
             // Eq. adhFor on the two elements sharing v, half each
             if (a.nlig > 0) {
-                bond_on_element<C, E>(a, L, xl, yl, xv, yv, Fx, Fy);
-                bond_on_element<C, E>(a, v, xv, yv, xR, yR, Fx, Fy);
+                bond_on_element<C, E>(a, L, !settle, xl, yl, xv, yv, Fx, Fy);
+                bond_on_element<C, E>(a, v, !settle, xv, yv, xR, yR, Fx, Fy);
             }
             // Eq. strainFor on elements (v, R) and (L, v); l - l_0 is formed as
             // (l^2 - l_0^2) / (l + l_0) with the squares in the extended type
@@ -528,8 +542,8 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit) {
 }
 
 template <typename C>
-__global__ void __launch_bounds__(kForceThreads) k_forces(const MarkerArgs a) {
-    forces_unit<C>(a, blockIdx.x);
+__global__ void __launch_bounds__(kForceThreads) k_forces(const MarkerArgs a, const bool settle) {
+    forces_unit<C>(a, blockIdx.x, settle);
 }
 
 // Batched form: the force units of up to kBatchMax contexts (ensemble
@@ -542,7 +556,20 @@ __global__ void __launch_bounds__(kForceThreads, 3) k_forces_batch(const __grid_
     __shared__ MarkerArgs s_a;
     const int m = marker_member(b, blockIdx.x);
     stage_args(&s_a, b.args + m);
-    forces_unit<C>(s_a, blockIdx.x - b.off[m]);
+    forces_unit<C>(s_a, blockIdx.x - b.off[m], b.settle != 0);
+}
+
+// the end of a launch sequence: the last step's bond decisions, one block per
+// context
+__global__ void __launch_bounds__(256) k_settle(const MarkerArgs a) {
+    dep_wait();
+    settle_bonds(a);
+}
+__global__ void __launch_bounds__(256) k_settle_batch(const MarkerArgs* __restrict__ args) {
+    __shared__ MarkerArgs s_a;
+    stage_args(&s_a, args + blockIdx.x);
+    dep_wait();
+    settle_bonds(s_a);
 }
 
 // ---------------------------------------------------------------- segments
@@ -599,8 +626,9 @@ cudaError_t launch_rest(lbib_precision prec, const MarkerArgs& a, void* rest, do
     return cudaGetLastError();
 }
 
-cudaError_t launch_forces(lbib_precision prec, const MarkerArgs& a, cudaStream_t s, bool chained) {
-    return launch_kernel(is_f64(prec) ? k_forces<double> : k_forces<float>, a.nfu, kForceThreads, 0, s, chained, a);
+cudaError_t launch_forces(lbib_precision prec, const MarkerArgs& a, bool settle, cudaStream_t s, bool chained) {
+    return launch_kernel(is_f64(prec) ? k_forces<double> : k_forces<float>, a.nfu + (settle ? 1 : 0), kForceThreads, 0, s,
+                         chained, a, settle);
 }
 
 cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, cudaStream_t s, bool chained) {
@@ -609,6 +637,14 @@ cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, cudaS
     if (nunits <= 0) return cudaSuccess;
     return launch_kernel(is_f64(prec) ? k_forces_batch<double> : k_forces_batch<float>, nunits, kForceThreads, 0, s,
                          chained, b);
+}
+
+cudaError_t launch_settle(const MarkerArgs& a, cudaStream_t s) {
+    return launch_kernel(k_settle, 1, 256, 0, s, true, a);
+}
+
+cudaError_t launch_settle_batch(const MarkerArgs* args, int n, cudaStream_t s) {
+    return launch_kernel(k_settle_batch, n, 256, 0, s, true, args);
 }
 
 cudaError_t launch_seg_boxes(lbib_precision prec, const MarkerArgs& a, cudaStream_t s) {

@@ -161,16 +161,28 @@ struct MarkerArgs {
     // cuts every membrane into chunks of kChunkV vertices, the advance kernel
     // cuts kinematic membranes the same way and keeps rigid-projected ones whole
     int nfu, nau;
-    int adv_threads;          // threads per advance block: 64, or the longest rigid ring rounded up to a warp
+    int adv_threads;          // threads per advance block (the largest unit, rounded up to a warp)
     const int4* fu;           // [nfu][2]: {m, k0, kn, off} {n, kind, lig0, nlig} (see kUnitInts)
     const int4* au;           // [nau][2], same records
     // bonds
     int nlig, nrec;
     const int* lig_a;         // [nlig] first vertex of the ligand element
     const int* lig_b;         // [nlig] second vertex
-    int* bond_of_lig;         // [nlig]
+    // Bonds.  The advance kernel of step n decides (cand, rupt, claim) but
+    // changes nothing; the decisions become the bonds of step n + 1 when they
+    // are settled: by a block of its own in the force kernel of step n + 1, or
+    // by k_settle behind the last step of a launch sequence.  Bonds, decisions
+    // and step counter are kept twice, by the parity of the step that starts
+    // from them (the parity of its population buffer): settling reads the
+    // previous parity and writes this one, so the force kernel's other blocks
+    // can look their bonds up in the previous parity meanwhile.
+    int* bond_of_lig;         // [nlig] bonds of this step
     int* cand;                // [nlig]
     int* rupt;                // [nlig]
+    const int* bond_prev;     // the previous parity's bonds and decisions
+    const int* cand_prev;
+    const int* rupt_prev;
+    const int* claim_prev;
     const double* rec_xy;     // [nrec][2] receptor positions (FP64 decisions)
     const void* rec_e;        // [nrec] the same in the marker position layout
     int* owner;               // [nrec]
@@ -190,10 +202,10 @@ struct MarkerArgs {
     int tile_w, tile_h, tiles_x, tiles_y;
     longlong2* gsum;
     int* flags;
-    // step counter, status and the arrival counters of the last-block epilogues
+    // step counter (this and the previous parity) and status
     long long* d_step;
+    const long long* step_prev;
     int* status;
-    unsigned int* tickets;    // arrival counter of the advance kernel's last-block epilogue
     // u field (compute type)
     const void* ux;
     const void* uy;
@@ -202,11 +214,12 @@ struct MarkerArgs {
         float nx, ny, inv_nx, inv_ny, sigma, y_eq, inv_y_eq, d_rep, d_cut, d_break;
         float kf_dt, kr0_dt, beta_f, beta_r, inv_rc_w, inv_rc_h, rc_y0;
     } f;
-    // ligands decided by each advance unit (element inside the unit, CSR), and
-    // the ligands whose element straddles two units (decided by the last block)
+    // ligands decided by each advance unit (the unit of their element's first
+    // vertex, CSR); the second vertex of a unit's last element is the first of
+    // the ring's next unit, local index = the unit's vertex count
     const int4* au_ligs;      // {ligand, local vertex a, local vertex b, 0} per unit ligand
-    int nstrad;
-    const int* strad_ligs;
+    void* halo;               // [nau][2] X^n and X^{n-1} of each chunk's first vertex, written by the force
+                              // kernel for the chunk before it in the ring (advance overwrites X, Xp)
     // dynamic particles (Sec. 2.4): compute-type [nv][2] arrays, meaningful on
     // the vertices of dynamic membranes only
     void* V;                  // particle velocity u_p^n
@@ -283,6 +296,7 @@ struct MarkerBatch {
     int n;
     int off[kBatchMax + 1];     // first block of each member's units
     const MarkerArgs* args;     // [n]
+    int settle;                 // force kernel: settle the previous step's bond decisions
     unsigned char member[kBlockTable];  // member of block b < min(off[n], kBlockTable)
 };
 __device__ __forceinline__ int marker_member(const MarkerBatch& b, int blk) {
@@ -363,7 +377,13 @@ cudaError_t launch_mass(lbib_precision prec, const void* src, long long n_elems,
 // ib_kernels.cu
 cudaError_t launch_rest(lbib_precision prec, const MarkerArgs& a, void* rest, double* A0, double* qa,
                         cudaStream_t s);
-cudaError_t launch_forces(lbib_precision prec, const MarkerArgs& a, cudaStream_t s, bool chained = false);
+// (settle: an extra block settles the previous step's bond decisions, and the
+// others look their bonds up through them; else a.bond_of_lig is settled)
+cudaError_t launch_forces(lbib_precision prec, const MarkerArgs& a, bool settle, cudaStream_t s,
+                          bool chained = false);
+// settle the last step's decisions into the parity of `a` (a launch sequence's end)
+cudaError_t launch_settle(const MarkerArgs& a, cudaStream_t s);
+cudaError_t launch_settle_batch(const MarkerArgs* args, int n, cudaStream_t s);
 cudaError_t launch_advance(lbib_precision prec, const MarkerArgs& a, cudaStream_t s, bool chained = false);
 // batched marker kernels of up to kBatchMax contexts (b.off[b.n] blocks); the
 // advance blocks have `threads` threads (the widest member's)
@@ -440,9 +460,11 @@ struct lbib_ctx {
     double* d_areas = nullptr;
     double* xy_stage = nullptr;             // 2*nv doubles for marker read/write
     double* d_obs = nullptr;                // 8*nmem doubles of membrane observables (lazy)
-    unsigned int* tickets = nullptr;
+    // by parity (see MarkerArgs)
+    int *bond[2] = {nullptr, nullptr}, *cand[2] = {nullptr, nullptr}, *rupt[2] = {nullptr, nullptr};
+    int* claim[2] = {nullptr, nullptr};
 
-    long long* d_step = nullptr;
+    long long* d_step = nullptr;            // [2], by parity
     int* d_status = nullptr;
     long long steps = 0;
     bool fields_valid = false;

@@ -174,49 +174,33 @@ __device__ typename Ext<C>::E ring_area_group(const MarkerArgs& a, int off, int 
 }
 
 // four block-wide sums in the compute type at once (every thread gets all four
-// in its arguments); each by a fixed shuffle tree per warp, then over the warps
+// in its arguments); each by a fixed shuffle tree per warp, then every thread
+// adds the warps' partials in a fixed tree of eight (blocks have at most eight
+// warps).  One barrier: `red` (4 x 8) is the call's own.
 template <typename C>
-__device__ void block_sum4_c(C& v0, C& v1, C& v2, C& v3, C* red) {
+__device__ void block_sum4_c(C& v0, C& v1, C& v2, C& v3, C (*red)[8]) {
     C v[4] = {v0, v1, v2, v3};
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(kFull, v[q], o);
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] += __shfl_down_sync(kFull, v[q], o);
     const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    __syncthreads();
     if ((threadIdx.x & 31) == 0) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) red[33 * q + w] = v[q];
+        for (int q = 0; q < 4; ++q) red[q][w] = v[q];
     }
     __syncthreads();
-    if (threadIdx.x < 32) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            C t = threadIdx.x < nw ? red[33 * q + threadIdx.x] : C(0);
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(kFull, t, o);
-            if (threadIdx.x == 0) red[33 * q + 32] = t;
-        }
+    for (int q = 0; q < 4; ++q) {
+        C t[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t[k] = k < nw ? red[q][k] : C(0);
+        v[q] = ((t[0] + t[4]) + (t[2] + t[6])) + ((t[1] + t[5]) + (t[3] + t[7]));
     }
-    __syncthreads();
-    v0 = red[32];
-    v1 = red[33 + 32];
-    v2 = red[66 + 32];
-    v3 = red[99 + 32];
-}
-
-// Last-block epilogue: every block of a context's launch counts itself in once
-// it is done; the block that arrives last (it sees all other blocks' writes
-// after the fences) runs the epilogue and resets the counter.  No block ever
-// waits for another.  nblocks: the context's blocks in the launch.
-__device__ __forceinline__ bool arrive_last(unsigned int* counter, bool* flag, unsigned nblocks) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        *flag = atomicAdd(counter, 1u) == nblocks - 1;
-    }
-    __syncthreads();
-    const bool last = *flag;
-    if (last) __threadfence();
-    return last;
+    v0 = v[0];
+    v1 = v[1];
+    v2 = v[2];
+    v3 = v[3];
 }
 
 // Box of one segment from positions held by a group of kSegV consecutive lanes
