@@ -61,23 +61,6 @@ __device__ __forceinline__ void verlet(const MarkerArgs& a, int m, int v, typena
     }
 }
 
-// repulsion boxes of a whole ring whose new positions are in shared memory:
-// kSegV lanes per segment
-template <typename C>
-__device__ __forceinline__ void ring_boxes(const MarkerArgs& a, int m, int n, int tid, int lane,
-                                           const typename Ext<C>::E* s_x, const typename Ext<C>::E* s_y) {
-    const int per_pass = blockDim.x / kSegV;
-    const int s0 = a.mem_seg_off[m], s1 = a.mem_seg_off[m + 1];
-    for (int base = 0; base < s1 - s0; base += per_pass) {
-        const int si = base + tid / kSegV;
-        const int kfirst = si * kSegV;
-        const int g = tid & (kSegV - 1);
-        const bool ok = si < s1 - s0;
-        const int kk = ok ? (kfirst + g < n ? kfirst + g : kfirst) : 0;
-        seg_box_regs<C>(a, ok ? s0 + si : -1, lane, s_x[kk], s_y[kk]);
-    }
-}
-
 // DYN: the context holds dynamic particles (without them their paths are not
 // compiled into the kernel, which keeps its code small)
 //
@@ -87,15 +70,20 @@ __device__ __forceinline__ void ring_boxes(const MarkerArgs& a, int m, int n, in
 //
 // Everything but the velocities is read before dep_wait(): the positions,
 // forces, weights and bonds were complete when the fused kernel (the
-// predecessor in a chained launch) let this one start.
+// predecessor in a chained launch) let this one start.  What needs no velocity
+// is also done before it: the rigid projection's position sums, and all of a
+// rigid dynamic particle, bond decisions included (the fused kernel touches
+// nothing that is written here).  The kinds share one path but for what is
+// their own, which keeps the instructions that a step has to fetch anew few.
 template <typename C, bool DYN>
 __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u) {
     using E = typename Ext<C>::E;
-    const int4 u0 = a.au[2 * u], u1 = a.au[2 * u + 1];
+    const int4 u0 = a.au[3 * u], u1 = a.au[3 * u + 1], u2 = a.au[3 * u + 2];
     const int m = u0.x, k0 = u0.y, kn = u0.z, off = u0.w, n = u1.x, kind = u1.y;
     const int tid = threadIdx.x, lane = tid & 31;
+    const bool body = DYN && kind == LBIB_MEMBRANE_DYNAMIC_RIGID;
     __shared__ E s_x[kAdvThreads], s_y[kAdvThreads];
-    __shared__ C cred[2][4][8];
+    __shared__ C cred[3][4][8];
     __shared__ int s_np;  // formation candidates listed
     if (tid == 0) s_np = 0;
     const long long step = *a.d_step;
@@ -111,239 +99,189 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u) {
         my_bond = a.bond_of_lig[my_rec.x];
     }
 
-    if (kind == LBIB_MEMBRANE_KINEMATIC || (DYN && kind == LBIB_MEMBRANE_DYNAMIC)) {
-        // ---- kinematic or deformable dynamic chunk: one vertex per thread
-        // (and one thread for the next chunk's first vertex, where this unit's
-        // ligands may need it: read from the halo records, nothing stored)
-        const bool mine = tid < kn;
-        const bool next = tid == kn && nlq > 0 && kn < n;
-        const bool wraps = k0 + kn == n;
-        const int v = off + (mine ? k0 + tid : (next && !wraps ? k0 + kn : (next ? 0 : k0)));
-        E x, y, xp, yp, xn, yn;
-        if (next) {
-            const int un = wraps ? u - k0 / kChunkV : u + 1;
-            PosIO<C>::load(a.halo, 2 * un, x, y);
-            PosIO<C>::load(a.halo, 2 * un + 1, xp, yp);
-        } else {
-            load_pos<C>(a, v, x, y);
-            PosIO<C>::load(a.Xp, v, xp, yp);
-        }
-        const Shape<C> sh = load_shape<C>(a, v);
-        dep_wait();
-        dep_trigger();
-        if (mine || next) {
-            C Ux, Uy;
-            interp_vertex<C>(a, sh, Ux, Uy);
-            if (DYN && kind == LBIB_MEMBRANE_DYNAMIC) {
-                verlet<C>(a, m, v, x, y, xp, yp, Ux, Uy, step, mine, xn, yn);
-            } else {
-                bdf2<C>(x, xp, Ux, step, xn);
-                bdf2<C>(y, yp, Uy, step, yn);
-            }
-            if (mine) {
-                U[2 * v] = Ux;
-                U[2 * v + 1] = Uy;
-                if (!isfinite(ehi(xn)) || !isfinite(ehi(yn))) atomicOr(a.status, ST_NONFINITE);
-                PosIO<C>::store(a.Xp, v, x, y);
-                PosIO<C>::store(a.X, v, xn, yn);
-            }
-            s_x[tid] = xn;
-            s_y[tid] = yn;
-        } else {
-            xn = x;
-            yn = y;
-        }
-        // boxes of the repulsion segments of this chunk (chunks are segment-aligned)
-        const int gfirst = tid & ~(kSegV - 1);
-        const int sg = gfirst < kn ? a.mem_seg_off[m] + (k0 + gfirst) / kSegV : -1;
-        E gx, gy;
-        shfl_e(gx, xn, lane & ~(kSegV - 1));
-        shfl_e(gy, yn, lane & ~(kSegV - 1));
-        seg_box_regs<C>(a, sg, lane, mine ? xn : gx, mine ? yn : gy);
-    } else if (DYN && kind == LBIB_MEMBRANE_DYNAMIC_RIGID) {
-        // ---- rigid dynamic particle, the whole ring in this block: Eqs.
+    // ---- one vertex per thread, and one thread for the next chunk's first
+    // vertex, where this unit's ligands may need it: read from the halo records,
+    // nothing stored
+    const bool mine = tid < kn;
+    const bool next = tid == kn && nlq > 0 && kn < n;
+    const bool wraps = k0 + kn == n;
+    const int v = off + (mine ? k0 + tid : (next && !wraps ? k0 + kn : (next ? 0 : k0)));
+    E x, y, xp, yp, xn, yn, cax, cay;
+    if (n > kDirectArea) PosIO<C>::load(a.halo, 2 * (u - k0 / kChunkV), cax, cay);  // X^n of vertex 0
+    if (next) {
+        const int un = wraps ? u - k0 / kChunkV : u + 1;
+        PosIO<C>::load(a.halo, 2 * un, x, y);
+        PosIO<C>::load(a.halo, 2 * un + 1, xp, yp);
+    } else {
+        load_pos<C>(a, v, x, y);
+        PosIO<C>::load(a.Xp, v, xp, yp);
+    }
+    const Shape<C> sh = load_shape<C>(a, v);
+    C Ux = 0, Uy = 0;
+    if (body) {
+        // a rigid dynamic particle, the whole ring in this block: Eqs.
         // linearVelRig / angularVelRig.  F and its moment M about the area
         // centroid give du/dt = F/m, domega/dt = M/I; the body translates by u
         // and turns by omega about its centroid (cos omega - 1 = -2 sin^2(omega/2))
-        E xr, yr;
+        E xr, yr, xq, yq;
         load_pos<C>(a, off, xr, yr);
-        const int k = tid;
-        const bool valid = k < n;
+        load_pos<C>(a, v + 1 == off + n ? off : v + 1, xq, yq);
         const C* F = static_cast<const C*>(a.F);
-        E x, y;
-        C Ux = 0, Uy = 0, ax = 0, ay = 0, bx = 0, by = 0, fx = 0, fy = 0;
-        E xq, yq;
-        const int kv = valid ? k : 0;
-        load_pos<C>(a, off + kv, x, y);
-        load_pos<C>(a, off + (kv + 1 == n ? 0 : kv + 1), xq, yq);
-        const Shape<C> sh = load_shape<C>(a, off + kv);
-        dep_wait();
-        dep_trigger();
-        if (valid) {
-            interp_vertex<C>(a, sh, Ux, Uy);
-            ax = etoc(esub(x, xr));
-            ay = etoc(esub(y, yr));
-            bx = etoc(esub(xq, xr));
-            by = etoc(esub(yq, yr));
-            fx = F[2 * (size_t)(off + k)];
-            fy = F[2 * (size_t)(off + k) + 1];
-        }
+        const C fx = mine ? F[2 * (size_t)v] : C(0), fy = mine ? F[2 * (size_t)v + 1] : C(0);
+        const C ax = mine ? etoc(esub(x, xr)) : C(0), ay = mine ? etoc(esub(y, yr)) : C(0);
+        const C bx = mine ? etoc(esub(xq, xr)) : C(0), by = mine ? etoc(esub(yq, yr)) : C(0);
         // area centroid relative to vertex 0 from the triangles (vertex 0, k, k+1)
         const C cr = ax * by - ay * bx;
-        C s2 = cr, gsx = cr * (ax + bx), gsy = cr * (ay + by), z0 = 0;
-        block_sum4_c<C>(s2, gsx, gsy, z0, cred[0]);
-        const C gx = gsx / (C(3) * s2), gy = gsy / (C(3) * s2);
+        C s3[3] = {cr, cr * (ax + bx), cr * (ay + by)};
+        block_sum_c<C, 3>(s3, cred[0]);
+        const C gx = s3[1] / (C(3) * s3[0]), gy = s3[2] / (C(3) * s3[0]);
         const C rx = ax - gx, ry = ay - gy;
-        // the rigid state is read by every thread before thread 0 rewrites it
-        double* rb = a.rb + 6 * m;
-        const double u0 = rb[0], v0 = rb[1], up = rb[2], vp = rb[3], w0 = rb[4], wp = rb[5];
-        C Fx = fx, Fy = fy, Mz = valid ? rx * fy - ry * fx : C(0), z1 = 0;
-        block_sum4_c<C>(Fx, Fy, Mz, z1, cred[1]);
-        const double mass = a.mem_dyn[3 * m], inertia = a.mem_dyn[3 * m + 1];
-        const double axd = double(Fx) / mass, ayd = double(Fy) / mass, ald = double(Mz) / inertia;
-        double un, vn, wn;
-        if (step == 0) {
-            un = u0 + axd;
-            vn = v0 + ayd;
-            wn = w0 + ald;
-        } else {
-            un = (2.0 / 3.0) * (2.0 * u0 - 0.5 * up + axd);
-            vn = (2.0 / 3.0) * (2.0 * v0 - 0.5 * vp + ayd);
-            wn = (2.0 / 3.0) * (2.0 * w0 - 0.5 * wp + ald);
-        }
-        if (tid == 0) {
-            rb[2] = u0;
-            rb[3] = v0;
-            rb[5] = w0;
-            rb[0] = un;
-            rb[1] = vn;
-            rb[4] = wn;
-        }
-        const C hs = sin(C(0.5) * C(wn));
-        const C c1 = C(-2) * hs * hs, sn = sin(C(wn));
-        if (valid) {
-            const int v = off + k;
-            const C drx = c1 * rx - sn * ry, dry = sn * rx + c1 * ry;
-            C* V = static_cast<C*>(a.V);
-            V[2 * (size_t)v] = C(un) - C(wn) * (ry + dry);
-            V[2 * (size_t)v + 1] = C(vn) + C(wn) * (rx + drx);
-            U[2 * v] = Ux;
-            U[2 * v + 1] = Uy;
-            const E xn = eaddc(x, C(un) + drx), yn = eaddc(y, C(vn) + dry);
-            if (!isfinite(ehi(xn)) || !isfinite(ehi(yn))) atomicOr(a.status, ST_NONFINITE);
-            PosIO<C>::store(a.Xp, v, x, y);
-            PosIO<C>::store(a.X, v, xn, yn);
-            s_x[k] = xn;
-            s_y[k] = yn;
+        C f3[3] = {fx, fy, mine ? rx * fy - ry * fx : C(0)};
+        block_sum_c<C, 3>(f3, cred[1]);
+        // the rigid state in FP64, one component a lane of the first warp (done
+        // by every warp, these operations took most of the kernel: 9000 of 20000
+        // cycles for a 210-vertex carrier)
+        __shared__ C s_rb[5];
+        if (tid < 3) {
+            double* rb = a.rb + 6 * m;
+            const int now = tid < 2 ? tid : 4, before = tid < 2 ? tid + 2 : 5;
+            const double s0 = rb[now], sp = rb[before];
+            const double acc = double(tid == 0 ? f3[0] : (tid == 1 ? f3[1] : f3[2])) / a.mem_dyn[3 * m + (tid < 2 ? 0 : 1)];
+            const double sn = step == 0 ? s0 + acc : (2.0 / 3.0) * (2.0 * s0 - 0.5 * sp + acc);
+            rb[before] = s0;
+            rb[now] = sn;
+            s_rb[tid] = C(sn);
+            if (tid == 2) {
+                const C hs = sin(C(0.5) * C(sn));
+                s_rb[3] = C(-2) * hs * hs;
+                s_rb[4] = sin(C(sn));
+            }
         }
         __syncthreads();
-        ring_boxes<C>(a, m, n, tid, lane, s_x, s_y);
+        const C un = s_rb[0], vn = s_rb[1], wn = s_rb[2], c1 = s_rb[3], sn = s_rb[4];
+        const C drx = c1 * rx - sn * ry, dry = sn * rx + c1 * ry;
+        xn = eaddc(x, un + drx);
+        yn = eaddc(y, vn + dry);
+        if (mine) {
+            C* V = static_cast<C*>(a.V);
+            V[2 * (size_t)v] = un - wn * (ry + dry);
+            V[2 * (size_t)v + 1] = vn + wn * (rx + drx);
+        }
     } else {
-        // ---- rigid-projected membrane: the whole ring in this block
-        E xr, yr;
-        load_pos<C>(a, off, xr, yr);
-        const int k = tid;
-        const bool valid = k < n;
-        E x, y, xpv, ypv;
-        C Ux = 0, Uy = 0;
-        C sx = 0, sy = 0, su = 0, sv = 0;
-        const int kv = valid ? k : 0;
-        load_pos<C>(a, off + kv, x, y);
-        PosIO<C>::load(a.Xp, off + kv, xpv, ypv);
-        const Shape<C> sh = load_shape<C>(a, off + kv);
+        // rigid projection (the whole ring in this block): positions about their
+        // mean, from vertex 0
+        const bool project = kind == LBIB_MEMBRANE_RIGID_PROJECTED;
+        const C inv_n = C(1) / C(n);
+        C rx = 0, ry = 0, den = 0;
+        if (project) {
+            E xr, yr;
+            load_pos<C>(a, off, xr, yr);
+            const C dx = etoc(esub(x, xr)), dy = etoc(esub(y, yr));
+            C p2[2] = {mine ? dx : C(0), mine ? dy : C(0)};
+            block_sum_c<C, 2>(p2, cred[0]);
+            rx = dx - p2[0] * inv_n;
+            ry = dy - p2[1] * inv_n;
+        }
         dep_wait();
         dep_trigger();
-        if (valid) {
-            interp_vertex<C>(a, sh, Ux, Uy);
-            sx = etoc(esub(x, xr));
-            sy = etoc(esub(y, yr));
-            su = Ux;
-            sv = Uy;
+        interp_vertex<C>(a, sh, Ux, Uy);
+        if (project) {
+            // least-squares rigid motion U_c + omega x (x - x_c)
+            C u2s[2] = {mine ? Ux : C(0), mine ? Uy : C(0)};
+            block_sum_c<C, 2>(u2s, cred[1]);
+            const C mu = u2s[0] * inv_n, mv = u2s[1] * inv_n;
+            C q2[2] = {mine ? rx * (Uy - mv) - ry * (Ux - mu) : C(0), mine ? rx * rx + ry * ry : C(0)};
+            block_sum_c<C, 2>(q2, cred[2]);
+            const C om = q2[0] / q2[1];
+            Ux = mu - om * ry;
+            Uy = mv + om * rx;
         }
-        // least-squares rigid motion U_c + omega x (x - x_c), positions about vertex 0
-        const C inv_n = C(1) / C(n);
-        block_sum4_c<C>(sx, sy, su, sv, cred[0]);
-        const C mx = sx * inv_n, my = sy * inv_n, mu = su * inv_n, mv = sv * inv_n;
-        C num = 0, den = 0;
-        if (valid) {
-            const C rx = etoc(esub(x, xr)) - mx, ry = etoc(esub(y, yr)) - my;
-            num = rx * (Uy - mv) - ry * (Ux - mu);
-            den = rx * rx + ry * ry;
+        if (DYN && kind == LBIB_MEMBRANE_DYNAMIC) {
+            verlet<C>(a, m, v, x, y, xp, yp, Ux, Uy, step, mine, xn, yn);
+        } else {
+            bdf2<C>(x, xp, Ux, step, xn);
+            bdf2<C>(y, yp, Uy, step, yn);
         }
-        C z0 = 0, z1 = 0;
-        block_sum4_c<C>(num, den, z0, z1, cred[1]);
-        const C om = num / den;
-        if (valid) {
-            const int v = off + k;
-            const C rx = etoc(esub(x, xr)) - mx, ry = etoc(esub(y, yr)) - my;
-            const C px = mu - om * ry, py = mv + om * rx;
-            U[2 * v] = px;
-            U[2 * v + 1] = py;
-            E xn, yn;
-            bdf2<C>(x, xpv, px, step, xn);
-            bdf2<C>(y, ypv, py, step, yn);
-            if (!isfinite(ehi(xn)) || !isfinite(ehi(yn))) atomicOr(a.status, ST_NONFINITE);
-            PosIO<C>::store(a.Xp, v, x, y);
-            PosIO<C>::store(a.X, v, xn, yn);
-            s_x[k] = xn;
-            s_y[k] = yn;
+        if (mine) {
+            U[2 * v] = Ux;
+            U[2 * v + 1] = Uy;
         }
-        __syncthreads();
-        ring_boxes<C>(a, m, n, tid, lane, s_x, s_y);
+    }
+    if (mine) {
+        if (!isfinite(ehi(xn)) || !isfinite(ehi(yn))) atomicOr(a.status, ST_NONFINITE);
+        PosIO<C>::store(a.Xp, v, x, y);
+        PosIO<C>::store(a.X, v, xn, yn);
+    }
+    s_x[tid] = xn;
+    s_y[tid] = yn;
+    {
+        // boxes of the unit's repulsion segments (units are segment-aligned); lanes
+        // past a segment's end take its first vertex
+        const int gfirst = tid & ~(kSegV - 1);
+        const int sg = gfirst < kn ? u2.x + (k0 + gfirst) / kSegV : -1;
+        const int gr = (tid & ~(kGroupV - 1)) < kn ? u2.y + (k0 + tid) / kGroupV : -1;
+        E gx, gy;
+        shfl_e(gx, xn, lane & ~(kSegV - 1));
+        shfl_e(gy, yn, lane & ~(kSegV - 1));
+        seg_box_regs<C>(a, sg, gr, lane, mine ? xn : gx, mine ? yn : gy);
     }
     __syncthreads();
+    if (n > kDirectArea && tid < 32) {
+        // the chunk's share of the ring's area at the new positions, by the first warp
+        const E part = chunk_area<C>(kn, lane, cax, cay, [&](int k, E& px, E& py) {
+            px = s_x[k];
+            py = s_y[k];
+        });
+        if (lane == 0) PosIO<C>::store(a.area_part, u, part, part);
+    }
 
     // ---- bond decisions for the ligands whose element starts in this unit.
-    // (a) per ligand: rupture test of its bond, and the receptors of the 3x3
-    //     cells around it that were free at the start of the step, as
-    //     (ligand, receptor) pairs;
+    // (a) per ligand: rupture test of its bond; a free ligand lists the
+    //     receptors of the 3x3 cells around it as (ligand, receptor) pairs;
     // (b) per pair: the formation test; each ligand keeps the lowest passing
     //     receptor id (a minimum: independent of evaluation order);
     // (c) per ligand that is free after (a): claim its receptor.
+    // Receptors have to be free at the start of the step.
     if (nlq > 0) {
         __shared__ int s_pl[kMaxPairs], s_pr[kMaxPairs];
         __shared__ int s_best[kAdvThreads];
-        __shared__ int s_look[kAdvThreads];
-        __shared__ int s_lig[kAdvThreads], s_ka[kAdvThreads], s_kb[kAdvThreads];
-        for (int q = tid; q < nlq; q += blockDim.x) {
-            const int4 rec = my_rec;  // q == tid: a unit has no more ligands than threads
-            const int l = rec.x, ka = rec.y, kb = rec.z;
-            s_lig[q] = l;
-            s_ka[q] = ka;
-            s_kb[q] = kb;
+        __shared__ int4 s_lig[kAdvThreads];
+        const int l = my_rec.x;  // a unit has no more ligands than threads
+        bool look = false;
+        if (tid < nlq) {
             LigandPoint<C> lp;
-            lp.init(s_x[ka], s_y[ka], s_x[kb], s_y[kb]);
-            s_best[q] = INT_MAX;
-            bool look = lp.finite();  // non-finite positions: reported above
-            const int r = my_bond;
-            if (look && r >= 0) {
-                look = ruptures<C>(a, lp, step, l, r);
-                if (look) a.rupt[l] = r;
+            lp.init(s_x[my_rec.y], s_y[my_rec.y], s_x[my_rec.z], s_y[my_rec.z]);
+            s_lig[tid] = my_rec;
+            s_best[tid] = INT_MAX;
+            look = lp.finite();  // non-finite positions: reported above
+            if (look && my_bond >= 0) {
+                look = ruptures<C>(a, lp, step, l, my_bond);
+                if (look) a.rupt[l] = my_bond;
             }
-            s_look[q] = look;
-            if (!look) continue;
-            int p0[9], p1[9];
-            ligand_cells<C>(a, lp, p0, p1);
-            // every receptor of the cells becomes a pair; whether it was free at
-            // the start of the step is checked per pair, in parallel
+            if (look && receptors_in_reach<C>(a, lp)) {
+                int p0[9], p1[9];
+                ligand_cells<C>(a, lp, p0, p1);
+                // every receptor of the cells becomes a pair; whether it was free at
+                // the start of the step is checked per pair, in parallel
 #pragma unroll
-            for (int c = 0; c < 9; ++c) {
-                for (int p = p0[c]; p < p1[c]; ++p) {
-                    const int slot = atomicAdd(&s_np, 1);
-                    if (slot < kMaxPairs) {
-                        s_pl[slot] = q;
-                        s_pr[slot] = p;
-                    } else {
-                        // list full: decide in place
-                        const int rr = a.rcell_ids[p];
-                        if (a.owner_cell[p] < 0 && forms<C>(a, lp, step, l, rr, ehi_pos_x<C>(a, p), ehi_pos_y<C>(a, p)))
-                            atomicMin(&s_best[q], rr);
+                for (int c = 0; c < 9; ++c) {
+                    for (int p = p0[c]; p < p1[c]; ++p) {
+                        const int slot = atomicAdd(&s_np, 1);
+                        if (slot < kMaxPairs) {
+                            s_pl[slot] = tid;
+                            s_pr[slot] = p;
+                        } else {
+                            // list full: decide in place
+                            const int rr = a.rcell_ids[p];
+                            if (a.owner_cell[p] < 0 && forms<C>(a, lp, step, l, rr, ehi_pos_x<C>(a, p), ehi_pos_y<C>(a, p)))
+                                atomicMin(&s_best[tid], rr);
+                        }
                     }
                 }
             }
         }
         __syncthreads();
-        if (s_np == 0) return;  // no receptor near any of the unit's ligands
+        // (often none: no receptor near any of the unit's free ligands)
         const int np = s_np < kMaxPairs ? s_np : kMaxPairs;
         for (int t = tid; t < np; t += blockDim.x) {
             const int q = s_pl[t], p = s_pr[t];
@@ -351,19 +289,25 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u) {
             typename Ext<C>::E rx, ry;
             PosIO<C>::load(a.rcell_pos, p, rx, ry);
             if (a.owner_cell[p] >= 0) continue;  // bound at the start of the step
-            const int l = s_lig[q], ka = s_ka[q], kb = s_kb[q];
+            const int4 rec = s_lig[q];
             LigandPoint<C> lp;
-            lp.init(s_x[ka], s_y[ka], s_x[kb], s_y[kb]);
-            if (forms<C>(a, lp, step, l, rr, rx, ry)) atomicMin(&s_best[q], rr);
+            lp.init(s_x[rec.y], s_y[rec.y], s_x[rec.z], s_y[rec.z]);
+            if (forms<C>(a, lp, step, rec.x, rr, rx, ry)) atomicMin(&s_best[q], rr);
         }
-        __syncthreads();
-        for (int q = tid; q < nlq; q += blockDim.x) {
-            const int best = s_best[q];
-            if (s_look[q] && best != INT_MAX) {
-                const int l = s_lig[q];
-                a.cand[l] = best;
-                atomicMin(&a.claim[best], l);
-            }
+        if (np > 0) __syncthreads();
+        if (look && s_best[tid] != INT_MAX) {
+            a.cand[l] = s_best[tid];
+            atomicMin(&a.claim[s_best[tid]], l);
+        }
+    }
+    if (body) {
+        // the flow's velocity at the vertices, for the read-back
+        dep_wait();
+        dep_trigger();
+        if (mine) {
+            interp_vertex<C>(a, sh, Ux, Uy);
+            U[2 * v] = Ux;
+            U[2 * v + 1] = Uy;
         }
     }
 }

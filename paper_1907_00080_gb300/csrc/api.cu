@@ -400,6 +400,14 @@ static lbib_status finalize(lbib_ctx* c) {
         }
     }
     mem_seg_off[nm] = (int)seg_mem.size();
+    // and groups of kGroupV of them, {membrane, first segment, first vertex, vertices}
+    std::vector<int> group, mem_group_off(nm + 1, 0);
+    for (int m = 0; m < nm; ++m) {
+        mem_group_off[m] = (int)(group.size() / 4);
+        for (int k = 0; k < c->h_mem_n[m]; k += kGroupV)
+            group.insert(group.end(), {m, mem_seg_off[m] + k / kSegV, c->h_mem_off[m] + k,
+                                       std::min(kGroupV, c->h_mem_n[m] - k)});
+    }
     c->nseg = (int)seg_mem.size();
     // ligand element vertices and element -> ligand map
     std::vector<int> lig_a(nl), lig_b(nl), elem_lig(std::max(nv, 1), -1), vmem(std::max(nv, 1));
@@ -415,6 +423,30 @@ static lbib_status finalize(lbib_ctx* c) {
     std::vector<int> mem_lig_off = c->h_mem_lig_off;
     if (mem_lig_off.empty()) mem_lig_off.assign(nm + 1, 0);
     // receptor grid: cells at least d_cut wide so a 3x3 block covers the cut-off disc
+    // heights no receptor is in reach of (see y_reach): below, in the largest
+    // gap, above; a little inside the exact bounds
+    float y_reach[4] = {-INFINITY, INFINITY, -INFINITY, INFINITY};
+    if (nr > 0) {
+        std::vector<double> ys(nr);
+        for (int r = 0; r < nr; ++r) ys[r] = c->h_rec[2 * r + 1];
+        std::sort(ys.begin(), ys.end());
+        const double dc = c->bp.d_cut * 1.001 + 1e-3;
+        double g0 = ys[0], g1 = ys[0];
+        for (int r = 0; r + 1 < nr; ++r)
+            if (ys[r + 1] - ys[r] > g1 - g0) {
+                g0 = ys[r];
+                g1 = ys[r + 1];
+            }
+        // (1e-3 covers FP32 rounding of the heights up to 8192 lattice units;
+        // beyond, the relative part)
+        const double eps = 1e-6 * (std::fabs(ys[0]) + std::fabs(ys[nr - 1]));
+        y_reach[0] = (float)(ys[0] - dc - eps);
+        y_reach[3] = (float)(ys[nr - 1] + dc + eps);
+        if (g1 - g0 > 2.0 * (dc + eps)) {
+            y_reach[1] = (float)(g0 + dc + eps);
+            y_reach[2] = (float)(g1 - dc - eps);
+        }
+    }
     int rc_nx = 1, rc_ny = 1;
     double rc_w = c->nx, rc_h = 1.0, rc_y0 = 0.0;
     std::vector<int> rcell_start(2, 0), rcell_ids;
@@ -446,20 +478,19 @@ static lbib_status finalize(lbib_ctx* c) {
         std::vector<int> cur(cnt.begin(), cnt.end() - 1);
         for (int r = 0; r < nr; ++r) rcell_ids[cur[cell[r]]++] = r;  // ascending id within a cell
     }
-    // work units, kUnitInts ints each (one 32-byte read per block):
-    // {membrane, first local vertex, vertex count, membrane offset, membrane size,
-    //  kind, then for force units the membrane's first segment and the advance
-    //  unit of the same chunk (-1: whole ring), for advance units the first
-    //  ligand record and the number of ligand records}
-    std::vector<int> fu, au;
+    // work units, kUnitInts ints each (read by a block before its first data load)
+    std::vector<int> fu, au, mem_au(nm + 1, 0);
     for (int m = 0; m < nm; ++m) {
         const int n = c->h_mem_n[m], off = c->h_mem_off[m], kind = c->h_mem_kind[m];
+        const int s0 = mem_seg_off[m], g0 = mem_group_off[m], ns = mem_seg_off[m + 1] - s0;
+        mem_au[m] = (int)(au.size() / kUnitInts);
         for (int k0 = 0; k0 < n; k0 += kChunkV) {
             const int u = whole_ring(kind) ? -1 : (int)(au.size() / kUnitInts);
-            fu.insert(fu.end(), {m, k0, std::min(kChunkV, n - k0), off, n, kind, mem_seg_off[m], u});
-            if (!whole_ring(kind)) au.insert(au.end(), {m, k0, std::min(kChunkV, n - k0), off, n, kind, 0, 0});
+            fu.insert(fu.end(), {m, k0, std::min(kChunkV, n - k0), off, n, kind, 0, u, s0, g0, ns, 0});
+            if (!whole_ring(kind))
+                au.insert(au.end(), {m, k0, std::min(kChunkV, n - k0), off, n, kind, 0, 0, s0, g0, ns, 0});
         }
-        if (whole_ring(kind)) au.insert(au.end(), {m, 0, n, off, n, kind, 0, 0});
+        if (whole_ring(kind)) au.insert(au.end(), {m, 0, n, off, n, kind, 0, 0, s0, g0, ns, 0});
     }
     // ligands of each advance unit (that of their element's first vertex), as
     // records {ligand, local index of its element's two vertices, 0}; an
@@ -518,13 +549,13 @@ static lbib_status finalize(lbib_ctx* c) {
         add(8 * (nm + 1)); add(8 * (nm + 1)); add(8 * (nm + 1)); add(4 * (nm + 2));
         add(16 * nv); add(16 * nv); add(2 * cs * nv); add(2 * cs * nv); add(9 * cs * nv); add(8 * nv);
         add(32 * nv); add(4 * nv); add(16 * nv + 16 * nr);
-        add(4 * c->nseg); add(4 * c->nseg); add(4 * c->nseg); add(16 * c->nseg); add(4 * (nm + 1));
+        add(4 * c->nseg); add(4 * c->nseg); add(4 * c->nseg); add(16 * c->nseg); add(4 * group.size()); add(4 * group.size());
         for (int k = 0; k < 8; ++k) add(4 * nl);
         add(16 * nr); add(16 * nr); add(4 * nr); add(4 * nr); add(4 * rcell_start.size()); add(4 * rcell_ids.size()); add(16 * nr);
         add(4 * nr); add(4 * nr); add(4 * nr);
         add(4 * c->ntiles); add(4 * c->ntiles); add(8 * (nm + 1));
         add(4 * fu.size()); add(4 * au.size());
-        add(4 * au_ligs.size()); add(32 * (size_t)nau);
+        add(4 * au_ligs.size()); add(32 * (size_t)nau); add(16 * (size_t)nau); add(4 * (nm + 1));
         add(2 * cs * nv); add(2 * cs * nv); add(2 * cs * nv); add(48 * (nm + 1)); add(24 * (nm + 1));
         add(4 * hydro_units.size());
         bytes = probe.used + 256;
@@ -562,7 +593,8 @@ static lbib_status finalize(lbib_ctx* c) {
     int* d_seg_v0 = ar.take<int>(c->nseg);
     int* d_seg_n = ar.take<int>(c->nseg);
     a.seg_box = ar.take<float4>(c->nseg);
-    int* d_mem_seg_off = ar.take<int>(nm + 1);
+    int* d_group = ar.take<int>(group.size());
+    a.group_box = ar.take<float4>(group.size() / 4);
     int* d_lig_a = ar.take<int>(nl);
     int* d_lig_b = ar.take<int>(nl);
     for (int q = 0; q < 2; ++q) {
@@ -586,6 +618,8 @@ static lbib_status finalize(lbib_ctx* c) {
     int* d_au = ar.take<int>(au.size());
     int* d_au_ligs = ar.take<int>(au_ligs.size());
     a.halo = ar.take<double>(4 * (size_t)nau);
+    a.area_part = ar.take<double>(2 * (size_t)nau);
+    int* d_mem_au = ar.take<int>(nm + 1);
     void* V = ar.take<char>(2 * cs * nv);
     void* Hf = ar.take<char>(2 * cs * nv);
     void* Dib = ar.take<char>(2 * cs * nv);
@@ -616,9 +650,10 @@ static lbib_status finalize(lbib_ctx* c) {
         CK(H2D(d_seg_mem, seg_mem.data(), 4 * seg_mem.size()));
         CK(H2D(d_seg_v0, seg_v0.data(), 4 * seg_v0.size()));
         CK(H2D(d_seg_n, seg_n.data(), 4 * seg_n.size()));
-        CK(H2D(d_mem_seg_off, mem_seg_off.data(), 4 * (nm + 1)));
+        CK(H2D(d_group, group.data(), 4 * group.size()));
         CK(H2D(d_fu, fu.data(), 4 * fu.size()));
         CK(H2D(d_au, au.data(), 4 * au.size()));
+        CK(H2D(d_mem_au, mem_au.data(), 4 * nm));
         if (!au_ligs.empty()) CK(H2D(d_au_ligs, au_ligs.data(), 4 * au_ligs.size()));
         CK(cudaMemsetAsync(V, 0, 2 * cs * nv, c->stream));
         CK(cudaMemsetAsync(Hf, 0, 2 * cs * nv, c->stream));
@@ -671,7 +706,8 @@ static lbib_status finalize(lbib_ctx* c) {
     a.mem_ks = ks; a.mem_kb = kb; a.mem_ka = ka; a.mem_A0 = A0; a.mem_qa = qa; a.mem_lig_off = lig_off;
     a.rest = rest; a.elem_lig = elig;
     a.d_rep = c->d_rep; a.nseg = c->nseg;
-    a.seg_mem = d_seg_mem; a.seg_v0 = d_seg_v0; a.seg_n = d_seg_n; a.mem_seg_off = d_mem_seg_off;
+    a.seg_mem = d_seg_mem; a.seg_v0 = d_seg_v0; a.seg_n = d_seg_n;
+    a.ngroup = (int)(group.size() / 4); a.group = reinterpret_cast<const int4*>(d_group);
     a.nfu = (int)(fu.size() / kUnitInts); a.nau = nau;
     // advance blocks: one thread per vertex of the largest unit (a chunk, with
     // its ligands' one vertex more, or a rigid ring); small blocks leave room
@@ -681,6 +717,7 @@ static lbib_status finalize(lbib_ctx* c) {
     a.V = V; a.Hf = Hf; a.Dib = Dib; a.rb = rb; a.mem_dyn = mem_dyn; a.has_dyn = c->ndyn > 0 ? 1 : 0;
     c->d_hydro_units = reinterpret_cast<int4*>(d_hydro_units);
     c->n_hydro_units = (int)(hydro_units.size() / 4);
+    a.mem_au = d_mem_au;
     a.fu = reinterpret_cast<const int4*>(d_fu);
     a.au = reinterpret_cast<const int4*>(d_au);
     a.au_ligs = reinterpret_cast<const int4*>(d_au_ligs);
@@ -702,9 +739,11 @@ static lbib_status finalize(lbib_ctx* c) {
     a.f.kf_dt = (float)a.kf_dt; a.f.kr0_dt = (float)a.kr0_dt; a.f.beta_f = (float)a.beta_f;
     a.f.beta_r = (float)a.beta_r; a.f.inv_rc_w = (float)a.inv_rc_w; a.f.inv_rc_h = (float)a.inv_rc_h;
     a.f.rc_y0 = (float)a.rc_y0;
+    for (int q = 0; q < 4; ++q) a.f.y_reach[q] = y_reach[q];
     a.ux = c->ux; a.uy = c->uy;
 
     if (nm > 0) {
+        CK(launch_area_parts(c->prec, a, c->stream));
         CK(launch_rest(c->prec, a, rest, A0, qa, c->stream));
         CK(launch_seg_boxes(c->prec, a, c->stream));
     }
@@ -1042,6 +1081,13 @@ extern "C" lbib_status lbib_read_markers(lbib_ctx* c, int32_t m, double* xy) {
     return LBIB_OK;
 }
 
+// what the advance kernel keeps beside the positions, after they were set
+// otherwise: the screening boxes and the long rings' area sums
+static cudaError_t refresh_markers(lbib_ctx* c, cudaStream_t s) {
+    const cudaError_t e = launch_seg_boxes(c->prec, c->ma, s);
+    return e != cudaSuccess ? e : launch_area_parts(c->prec, c->ma, s);
+}
+
 // the upload of marker positions X^n and X^{n-1}, enqueued on stream s (no wait)
 static lbib_status write_markers_on(lbib_ctx* c, const double* xy, const double* xy_prev, cudaStream_t s) {
     lbib_status st = finalize(c);
@@ -1053,7 +1099,7 @@ static lbib_status write_markers_on(lbib_ctx* c, const double* xy, const double*
     // X^{n-1} = X^n: the staged copy serves both
     if (xy_prev && xy_prev != xy) CK(cudaMemcpyAsync(c->xy_stage, xy_prev, b, cudaMemcpyHostToDevice, s));
     CK(launch_pos_in(c->prec, c->xy_stage, c->ma.Xp, c->nv, s));
-    CK(launch_seg_boxes(c->prec, c->ma, s));
+    CK(refresh_markers(c, s));
     return LBIB_OK;
 }
 
@@ -1944,6 +1990,7 @@ cudaError_t snap_copy(lbib_ctx* c, Snap& s, bool to_snap) {
     if ((e = cp(s.owner_cell, c->ma.owner_cell, 4 * nrec)) != cudaSuccess) return e;
     if ((e = cp(s.seg_box, c->ma.seg_box, sizeof(float4) * c->nseg)) != cudaSuccess) return e;
     if ((e = cp(s.d_step, c->d_step + c->cur, 8)) != cudaSuccess) return e;
+    if (!to_snap && (e = refresh_markers(c, c->stream)) != cudaSuccess) return e;
     if (to_snap) s.step = c->steps;
     else c->steps = s.step;
     return cudaSuccess;
@@ -2408,6 +2455,7 @@ extern "C" lbib_status lbib_load(lbib_ctx* c, const char* path) {
         if (c->flags[p]) CK(cudaMemsetAsync(c->flags[p], 0, 4 * (size_t)c->ntiles, c->stream));
     }
     CK(cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream));
+    CK(refresh_markers(c, c->stream));
     if (c->nlig > 0) {
         for (int q = 0; q < 2; ++q)
             for (int* p : {c->cand[q], c->rupt[q]}) CK(cudaMemsetAsync(p, 0xFF, 4 * (size_t)c->nlig, c->stream));

@@ -45,13 +45,23 @@ __device__ __forceinline__ void philox4x64_10(unsigned long long c[4], unsigned 
     }
 }
 
-// uniform in [0,1) from the top 53 bits of the first output word
-__device__ __forceinline__ double bond_uniform(const MarkerArgs& a, long long step, int lig, int rec,
-                                               int tag) {
+// the draw of a decision: the top 53 bits k of the first output word; the
+// uniform in [0, 1) is k 2^-53
+__device__ __forceinline__ unsigned long long bond_draw(const MarkerArgs& a, long long step, int lig, int rec,
+                                                        int tag) {
     unsigned long long c[4] = {(unsigned long long)step, (unsigned long long)lig,
                                (unsigned long long)rec, (unsigned long long)tag};
     philox4x64_10(c, a.seed, a.instance);
-    return (double)(c[0] >> 11) * 0x1.0p-53;
+    return c[0] >> 11;
+}
+__device__ __forceinline__ double uniform_of(unsigned long long k) { return (double)k * 0x1.0p-53; }
+// k 2^-53 < t and k 2^-53 > t for an FP32 threshold t < 2: exact (t 2^53 is a
+// scaling by a power of two), without the slow FP64 pipe
+__device__ __forceinline__ bool draw_below(unsigned long long k, float t) {
+    return t > 0.f && k < __float2ull_ru(t * 0x1.0p53f);
+}
+__device__ __forceinline__ bool draw_above(unsigned long long k, float t) {
+    return !(t >= 0.f) || k > __float2ull_rd(t * 0x1.0p53f);
 }
 
 // forward (formation) and reverse (rupture) probabilities per step, FP64
@@ -138,7 +148,7 @@ __device__ __forceinline__ bool forms(const MarkerArgs& a, LigandPoint<C>& lp, l
     if (sizeof(C) == 8) {
         const double d = lp.dist(a, r);
         if (!(d < a.d_cut)) return false;
-        return bond_uniform(a, step, l, r, 0) < p_form(a, d);
+        return uniform_of(bond_draw(a, step, l, r, 0)) < p_form(a, d);
     }
     const float df = float(lp.dist_est_at(a, rx, ry));
     const float dc = a.f.d_cut;
@@ -148,12 +158,12 @@ __device__ __forceinline__ bool forms(const MarkerArgs& a, LigandPoint<C>& lp, l
         d = lp.dist(a, r);
         if (!(d < a.d_cut)) return false;
     }
-    const double u = bond_uniform(a, step, l, r, 0);
+    const unsigned long long k = bond_draw(a, step, l, r, 0);
     const float pf = p_form_f(a, df);
-    if (u < (double)(pf - kMargin)) return true;
-    if (u > (double)(pf + kMargin)) return false;
+    if (draw_below(k, pf - kMargin)) return true;
+    if (draw_above(k, pf + kMargin)) return false;
     if (d < 0.0) d = lp.dist(a, r);
-    return u < p_form(a, d);
+    return uniform_of(k) < p_form(a, d);
 }
 
 // rupture test of the bond (l, r) (tag 1): d >= d_break or u < P_r(d)
@@ -162,7 +172,7 @@ __device__ __forceinline__ bool ruptures(const MarkerArgs& a, LigandPoint<C>& lp
     if (sizeof(C) == 8) {
         const double d = lp.dist(a, r);
         if (d >= a.d_break) return true;
-        return bond_uniform(a, step, l, r, 1) < p_rupture(a, d);
+        return uniform_of(bond_draw(a, step, l, r, 1)) < p_rupture(a, d);
     }
     const float df = float(lp.dist_est(a, r));
     const float db = a.f.d_break;
@@ -172,12 +182,20 @@ __device__ __forceinline__ bool ruptures(const MarkerArgs& a, LigandPoint<C>& lp
         d = lp.dist(a, r);
         if (d >= a.d_break) return true;
     }
-    const double u = bond_uniform(a, step, l, r, 1);
+    const unsigned long long k = bond_draw(a, step, l, r, 1);
     const float pr = p_rupture_f(a, df);
-    if (u < (double)(pr - kMargin)) return true;
-    if (u > (double)(pr + kMargin)) return false;
+    if (draw_below(k, pr - kMargin)) return true;
+    if (draw_above(k, pr + kMargin)) return false;
     if (d < 0.0) d = lp.dist(a, r);
-    return u < p_rupture(a, d);
+    return uniform_of(k) < p_rupture(a, d);
+}
+
+// false where no receptor can be within the cut-off of the ligand point by its
+// height alone
+template <typename C>
+__device__ __forceinline__ bool receptors_in_reach(const MarkerArgs& a, const LigandPoint<C>& lp) {
+    const float y = float(ehi(lp.cy));
+    return !(y < a.f.y_reach[0] || (y > a.f.y_reach[1] && y < a.f.y_reach[2]) || y > a.f.y_reach[3]);
 }
 
 // 3x3 receptor-grid cells around a ligand point: the nine [p0, p1) ranges of
@@ -202,14 +220,26 @@ __device__ __forceinline__ void ligand_cells(const MarkerArgs& a, const LigandPo
     }
 }
 
-// The bond of ligand l at the start of this step: the settled one, or (the
-// previous step's decisions not yet settled) the previous one changed by them:
-// a won claim binds, else a rupture frees.
-__device__ __forceinline__ int bond_now(const MarkerArgs& a, int l, bool settled) {
-    if (settled) return a.bond_of_lig[l];
-    const int b = a.bond_prev[l], c = a.cand_prev[l], r = a.rupt_prev[l];
-    if (c >= 0 && a.claim_prev[c] == l) return c;
-    return r >= 0 ? -1 : b;
+// The bonds at the start of this step of the ligands la, lb (-1: none): the
+// settled ones, or (the previous step's decisions not yet settled) the previous
+// ones changed by them: a won claim binds, else a rupture frees.  Both are
+// looked up at once.
+__device__ __forceinline__ void bonds_now(const MarkerArgs& a, int la, int lb, bool settled, int& ra, int& rb) {
+    const int ia = la < 0 ? 0 : la, ib = lb < 0 ? 0 : lb;
+    if (settled) {
+        ra = a.bond_of_lig[ia];
+        rb = a.bond_of_lig[ib];
+    } else {
+        ra = a.bond_prev[ia];
+        rb = a.bond_prev[ib];
+        const int ca = a.cand_prev[ia], cb = a.cand_prev[ib], xa = a.rupt_prev[ia], xb = a.rupt_prev[ib];
+        if (xa >= 0) ra = -1;
+        if (xb >= 0) rb = -1;
+        if (ca >= 0 && a.claim_prev[ca] == ia) ra = ca;
+        if (cb >= 0 && a.claim_prev[cb] == ib) rb = cb;
+    }
+    if (la < 0) ra = -1;
+    if (lb < 0) rb = -1;
 }
 
 // Settle the decisions of the previous step, all threads of one block: the

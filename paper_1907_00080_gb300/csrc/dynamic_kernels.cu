@@ -67,19 +67,23 @@ __device__ __forceinline__ void node_flow(const MarkerArgs& a, const HydroArgs& 
     const int nx = a.nx, ny = a.ny;
     const size_t N = (size_t)nx * ny;
     const size_t node = (size_t)j * nx + i;
-    C d[9];
+    // (the nine addresses first, then all the loads: one round trip)
+    size_t at[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-        int sy = j - cy(q);
-        if (a.walls && (sy < 0 || sy >= ny)) {
-            d[q] = Storage<S>::load(src[(size_t)opp(q) * N + node], h.inv_scale);
-            if (cx(q) != 0) d[q] += C(cx(q)) * hydro_wall<C>(h, cy(q) > 0);
-        } else {
-            sy = sy < 0 ? sy + ny : (sy >= ny ? sy - ny : sy);
-            int sx = i - cx(q);
-            sx = sx < 0 ? sx + nx : (sx >= nx ? sx - nx : sx);
-            d[q] = Storage<S>::load(src[(size_t)q * N + (size_t)sy * nx + sx], h.inv_scale);
-        }
+        int sy = j - cy(q), sx = i - cx(q);
+        const bool bb = a.walls && (sy < 0 || sy >= ny);
+        sy = sy < 0 ? sy + ny : (sy >= ny ? sy - ny : sy);
+        sx = sx < 0 ? sx + nx : (sx >= nx ? sx - nx : sx);
+        at[q] = bb ? (size_t)opp(q) * N + node : (size_t)q * N + (size_t)sy * nx + sx;
+    }
+    C d[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) d[q] = Storage<S>::load(src[at[q]], h.inv_scale);
+    if (a.walls && (j == 0 || j == ny - 1)) {
+#pragma unroll
+        for (int q = 0; q < 9; ++q)
+            if (cx(q) != 0 && (j - cy(q) < 0 || j - cy(q) >= ny)) d[q] += C(cx(q)) * hydro_wall<C>(h, cy(q) > 0);
     }
     const C drho = ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7])) + d[8];
     const C jx = (d[1] - d[3]) + ((d[5] - d[7]) + (d[8] - d[6]));
@@ -148,12 +152,21 @@ __device__ __forceinline__ NodeOf<C> node_of(const Stencil<C>& st, int b, int q)
     return o;
 }
 
-template <typename C>
-__device__ __forceinline__ void stencil_node(const MarkerArgs& a, const Stencil<C>& st, int b, int q, int& i,
-                                             int& j) {
-    j = st.j0 + b - 1;
-    if (!a.walls) j = ((j % a.ny) + a.ny) % a.ny;
-    i = ((st.i0 + q - 1) % a.nx + a.nx) % a.nx;
+// node (b, q) of the nine nearest to a point, wrapped into the lattice; false
+// (and the nearest fluid row) where it lies outside the walls
+template <typename C, typename E>
+__device__ __forceinline__ bool fit_node(const MarkerArgs& a, E px, E py, int b, int q, int& i, int& j) {
+    const C fi0 = fmin(fmax(C(efloor(eaddc(px, C(0.5)))), C(-1.0e7)), C(1.0e7));
+    const C fj0 = fmin(fmax(C(efloor(eaddc(py, C(0.5)))), C(-1.0e6)), C(1.0e6));
+    i = (((int)fi0 + q - 1) % a.nx + a.nx) % a.nx;
+    j = (int)fj0 + b - 1;
+    if (!a.walls) {
+        j = ((j % a.ny) + a.ny) % a.ny;
+        return true;
+    }
+    const bool fluid = j >= 0 && j < a.ny;
+    j = min(max(j, 0), a.ny - 1);
+    return fluid;
 }
 
 // The work of a block: a chunk of up to V consecutive vertices of one
@@ -179,6 +192,11 @@ template <typename S, typename E>
 __device__ __forceinline__ void probe_part(const MarkerArgs& a, const HydroArgs& h, E qx, E qy, int b, int q,
                                            typename Storage<S>::C (&part)[5]) {
     using C = typename Storage<S>::C;
+    // the node's flow first: its loads are in flight while the moments are formed
+    int i, j;
+    const bool fluid = fit_node<C, E>(a, qx, qy, b, q, i, j);
+    C pk, uk, vk;
+    node_flow<S>(a, h, i, j, pk, uk, vk);
     const Stencil<C> st = stencil_at<C, E>(a, qx, qy);
     C M00 = 0, M01 = 0, M02 = 0, M11 = 0, M12 = 0, M22 = 0;
 #pragma unroll
@@ -195,12 +213,8 @@ __device__ __forceinline__ void probe_part(const MarkerArgs& a, const HydroArgs&
         }
 #pragma unroll
     for (int r = 0; r < 5; ++r) part[r] = C(0);
+    if (!fluid) return;
     const NodeOf<C> nd = node_of<C>(st, b, q);
-    if (!nd.rowok) return;
-    int i, j;
-    stencil_node<C>(a, st, b, q, i, j);
-    C pk, uk, vk;
-    node_flow<S>(a, h, i, j, pk, uk, vk);
     const C w = nd.wx * nd.wy;
     // inverse of the symmetric moment matrix by its adjugate; with one fluid
     // row (or none) the y derivative is undetermined: the value falls back to
@@ -233,11 +247,15 @@ template <typename S, typename E>
 __device__ __forceinline__ void vertex_part(const MarkerArgs& a, const HydroArgs& h, E xv, E yv, int b, int q,
                                             typename Storage<S>::C (&part)[5]) {
     using C = typename Storage<S>::C;
+    int i, j;
+    const bool fluid = fit_node<C, E>(a, xv, yv, b, q, i, j);
+    C pk, uk, vk;
+    node_flow<S>(a, h, i, j, pk, uk, vk);
     const Stencil<C> st = stencil_at<C, E>(a, xv, yv);
 #pragma unroll
     for (int r = 0; r < 5; ++r) part[r] = C(0);
+    if (!fluid) return;
     const NodeOf<C> nd = node_of<C>(st, b, q);
-    if (!nd.rowok) return;
     C w = nd.wx * nd.wy;
     if (st.nrow < 3) {
         C M00 = 0, M01 = 0, M02 = 0, M11 = 0, M12 = 0, M22 = 0, sw = 0;
@@ -261,10 +279,6 @@ __device__ __forceinline__ void vertex_part(const MarkerArgs& a, const HydroArgs
         if (det > C(1e-10)) w = hdiv(w * (c0 + c1 * nd.rx + c2 * nd.ry), det);
         else w = sw > C(0) ? hdiv(w, sw) : C(0);
     }
-    int i, j;
-    stencil_node<C>(a, st, b, q, i, j);
-    C pk, uk, vk;
-    node_flow<S>(a, h, i, j, pk, uk, vk);
     part[0] = w * uk;
     part[1] = w * vk;
 }

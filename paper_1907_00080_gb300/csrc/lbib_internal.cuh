@@ -156,14 +156,18 @@ struct MarkerArgs {
     const int* seg_v0;        // [nseg] first global vertex
     const int* seg_n;         // [nseg]
     float4* seg_box;          // [nseg] centre x wrapped to [0,nx), centre y, half extents
-    const int* mem_seg_off;   // segments of membrane m: [mem_seg_off[m], mem_seg_off[m+1])
+    // groups of kGroupV vertices (four segments), boxes a little wide: the
+    // first stage of the screening
+    int ngroup;
+    const int4* group;        // [ngroup] {membrane, first segment, first global vertex, vertices}
+    float4* group_box;        // [ngroup] as seg_box
     // work units: (membrane, first local vertex, vertex count); the force kernel
     // cuts every membrane into chunks of kChunkV vertices, the advance kernel
     // cuts kinematic membranes the same way and keeps rigid-projected ones whole
     int nfu, nau;
     int adv_threads;          // threads per advance block (the largest unit, rounded up to a warp)
-    const int4* fu;           // [nfu][2]: {m, k0, kn, off} {n, kind, lig0, nlig} (see kUnitInts)
-    const int4* au;           // [nau][2], same records
+    const int4* fu;           // [nfu][3] records (see kUnitInts)
+    const int4* au;           // [nau][3]
     // bonds
     int nlig, nrec;
     const int* lig_a;         // [nlig] first vertex of the ligand element
@@ -213,11 +217,17 @@ struct MarkerArgs {
     struct {
         float nx, ny, inv_nx, inv_ny, sigma, y_eq, inv_y_eq, d_rep, d_cut, d_break;
         float kf_dt, kr0_dt, beta_f, beta_r, inv_rc_w, inv_rc_h, rc_y0;
+        // no receptor is within reach of a ligand at y < y_reach[0], y_reach[1] < y < y_reach[2] (the largest
+        // gap between receptor heights, e.g. the channel between its walls) or y > y_reach[3]
+        float y_reach[4];
     } f;
     // ligands decided by each advance unit (the unit of their element's first
     // vertex, CSR); the second vertex of a unit's last element is the first of
     // the ring's next unit, local index = the unit's vertex count
     const int4* au_ligs;      // {ligand, local vertex a, local vertex b, 0} per unit ligand
+    void* area_part;          // [nau] sums of the chunks' interior elements (long rings, see ring_area_parts),
+                              // one position record {sum, unused} each; of the current X
+    const int* mem_au;        // [nmem] advance unit of the membrane's first chunk
     void* halo;               // [nau][2] X^n and X^{n-1} of each chunk's first vertex, written by the force
                               // kernel for the chunk before it in the ring (advance overwrites X, Xp)
     // dynamic particles (Sec. 2.4): compute-type [nv][2] arrays, meaningful on
@@ -248,8 +258,11 @@ struct HydroArgs {
 enum StatusBits { ST_NONFINITE = 1, ST_TILE_OVERFLOW = 2, ST_TIMEOUT = 4, ST_FIXRANGE = 8 };
 
 constexpr int kChunkV = 64;   // vertices per marker-kernel block (a multiple of 32)
-constexpr int kUnitInts = 8;  // ints per work-unit record (two int4)
+constexpr int kUnitInts = 12; // ints per work-unit record (three int4): {m, k0, kn, off} {n, kind, x, y} {first
+                              // segment, first group, segments, 0 of the membrane}; x, y: force units {0, advance
+                              // unit of the chunk or -1}, advance units {first ligand record, their number}
 constexpr int kSegV = 8;      // vertices per repulsion-screening segment (divides kChunkV)
+constexpr int kGroupV = 32;   // vertices per screening group: a warp's (divides kChunkV)
 
 // Copy kernel arguments (a struct of the library's argument types) into
 // shared memory, all threads of the block taking 8-byte words; ends with a
@@ -391,6 +404,8 @@ cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, cudaS
 cudaError_t launch_advance_batch(lbib_precision prec, bool dyn, const MarkerBatch& b, int threads, cudaStream_t s,
                                  bool chained = false);
 cudaError_t launch_seg_boxes(lbib_precision prec, const MarkerArgs& a, cudaStream_t s);
+// the long rings' chunk sums for the current positions (after X or Xp were set)
+cudaError_t launch_area_parts(lbib_precision prec, const MarkerArgs& a, cudaStream_t s);
 cudaError_t launch_areas(lbib_precision prec, const MarkerArgs& a, double* areas, cudaStream_t s);
 // dynamic_kernels.cu: hydrodynamic stresses and forcing terms of the dynamic
 // particles at the start of a step (before launch_forces)

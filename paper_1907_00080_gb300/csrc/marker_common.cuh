@@ -16,21 +16,19 @@ __device__ __forceinline__ float wrap_half(float d, float L) {
     return d > 0.5f * L ? d - L : (d < -0.5f * L ? d + L : d);
 }
 
-// force value to the fixed-point grid of the spread field (scaled by 2^52)
+// force value, in units of the fixed-point grid of the spread field (2^-52),
+// to the grid
 template <typename C> __device__ __forceinline__ long long to_fix(C v);
-template <> __device__ __forceinline__ long long to_fix<float>(float v) {
-    // exact: t = v 2^52 is either below 2^23 in magnitude (round it with a 32-bit
+template <> __device__ __forceinline__ long long to_fix<float>(float t) {
+    // exact: t is either below 2^23 in magnitude (round it with a 32-bit
     // conversion) or an integer whose mantissa is shifted into place
-    const float t = v * 4503599627370496.0f;
     if (fabsf(t) < 8388608.0f) return (long long)__float2int_rn(t);
     const int bits = __float_as_int(t);
     const int e = ((bits >> 23) & 0xff) - 150;  // t = mant 2^e with e >= 0 here
     const long long mag = (long long)((bits & 0x7fffff) | 0x800000) << (e < 40 ? e : 40);
     return bits < 0 ? -mag : mag;
 }
-template <> __device__ __forceinline__ long long to_fix<double>(double v) {
-    return __double2ll_rn(v * kFixScale);
-}
+template <> __device__ __forceinline__ long long to_fix<double>(double t) { return __double2ll_rn(t); }
 
 // Range of the fixed-point conversions.  The spread field holds w F per
 // (vertex, node) scaled by 2^52, the repulsion accumulators one magnitude per
@@ -120,115 +118,194 @@ __device__ __forceinline__ EdgeProducts<C> edge_products(E xL, E yL, E xv, E yv,
     return p;
 }
 
-// Enclosed area of membrane m by the shoelace formula about vertex 0, summed
-// by kAreaWarps warps in a fixed order (thread t of the group takes terms t,
-// t + 32 kAreaWarps, ...; each warp reduces its lanes by a fixed tree; the warp
-// partials are added in warp order), so every caller gets the same bits.  Call
-// from the kAreaWarps consecutive warps starting at `w0` (all their lanes);
-// `red` holds 32 kAreaWarps values; returns the area in every caller after the
-// named barrier `bar` (kAreaWarps * 32 threads).  off, n: the membrane's first
-// vertex and vertex count.
-constexpr int kAreaWarps = 4;
+// Enclosed area of a ring by the shoelace formula, summed in a fixed order, so
+// that every caller gets the same bits (the rest shape then has exactly its
+// rest area).
+//
+// Rings of up to kDirectArea vertices: about vertex 0, by the 64 lanes of two
+// consecutive warps starting at `w0`: four sums, of the terms k with k / 32 mod
+// 4 = 0 .. 3 (lane l of sum s takes terms 32 s + l + 128 i in order, the lanes
+// are reduced by a fixed tree), added in order.  `red` holds 4 values; the result is valid in the first warp's lanes after
+// the named barrier `bar` (64 threads).
+//
+// Longer rings: every block of the force kernel would walk the whole ring (27
+// blocks of 1700 vertices on the fine capillary, 9800 of their 18900 cycles).
+// Their chunks' interior elements are summed once, by the advance kernel where
+// it has the new positions at hand (chunk_area), about c = X^{n-1} of vertex 0;
+// the reader adds the elements between chunks and the chunks' sums
+// (ring_area_parts, one warp, result in lane 0).
+constexpr int kDirectArea = 256;
+template <typename E>
+__device__ __forceinline__ E cross_about(E cx, E cy, E xa, E ya, E xb, E yb) {
+    return esub(emul(esub(xa, cx), esub(yb, cy)), emul(esub(xb, cx), esub(ya, cy)));
+}
+// sum over the warp's lanes by a fixed tree, in lane 0
+template <typename E>
+__device__ __forceinline__ E warp_tree(E v, int lane) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        E t;
+        shfl_e(t, v, (lane + o) & 31);
+        v = eadd(v, t);
+    }
+    return v;
+}
 template <typename C>
-__device__ typename Ext<C>::E ring_area_group(const MarkerArgs& a, int off, int n, int w0,
-                                              typename Ext<C>::E* red, int bar) {
+__device__ typename Ext<C>::E ring_area_direct(const MarkerArgs& a, int off, int n, int w0,
+                                               typename Ext<C>::E* red, int bar) {
     using E = typename Ext<C>::E;
-    const int t = threadIdx.x - 32 * w0;  // 0 .. 32 kAreaWarps - 1
-    const int lane = t & 31, w = t >> 5;
+    const int t = threadIdx.x - 32 * w0;  // 0 .. 63
+    const int lane = t & 31;
     E xr, yr;
     load_pos<C>(a, off, xr, yr);
-    E acc = ezero<E>();
-    // kBatch terms per pass with all their loads issued first (long rings:
-    // one round trip per pass instead of one per term); same summation order
-    constexpr int kBatch = 4;
-    constexpr int stride = 32 * kAreaWarps;
-    for (int k0 = t; k0 < n; k0 += kBatch * stride) {
-        E xv[kBatch], yv[kBatch], xR[kBatch], yR[kBatch];
+    // two rows of terms at once, t + 128 i and t + 64 + 128 i, all loads of a
+    // pass issued first
+    E acc[2] = {ezero<E>(), ezero<E>()};
+    for (int k0 = t; k0 < n; k0 += 128) {
+        E xv[2], yv[2], xR[2], yR[2];
 #pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-            const int k = k0 + b * stride;
+        for (int q = 0; q < 2; ++q) {
+            const int k = k0 + 64 * q;
             const int kk = k < n ? k : 0;
-            const int R = kk == n - 1 ? 0 : kk + 1;
-            load_pos<C>(a, off + kk, xv[b], yv[b]);
-            load_pos<C>(a, off + R, xR[b], yR[b]);
+            load_pos<C>(a, off + kk, xv[q], yv[q]);
+            load_pos<C>(a, off + (kk == n - 1 ? 0 : kk + 1), xR[q], yR[q]);
         }
 #pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-            if (k0 + b * stride >= n) break;
-            const E term = esub(emul(esub(xv[b], xr), esub(yR[b], yr)), emul(esub(xR[b], xr), esub(yv[b], yr)));
-            acc = eadd(acc, term);
-        }
+        for (int q = 0; q < 2; ++q)
+            if (k0 + 64 * q < n) acc[q] = eadd(acc[q], cross_about<E>(xr, yr, xv[q], yv[q], xR[q], yR[q]));
     }
-    E* r = red + 32 * w;
-    r[lane] = acc;
     __syncwarp();
-    for (int o = 16; o > 0; o >>= 1) {
-        if (lane < o) r[lane] = eadd(r[lane], r[lane + o]);
-        __syncwarp();
-    }
-    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(32 * kAreaWarps) : "memory");
-    E s = red[0];
 #pragma unroll
-    for (int q = 1; q < kAreaWarps; ++q) s = eadd(s, red[32 * q]);
-    return emulc(s, C(0.5));
+    for (int q = 0; q < 2; ++q) {
+        acc[q] = warp_tree<E>(acc[q], lane);
+        if (lane == 0) red[(t >> 5) + 2 * q] = acc[q];
+    }
+    asm volatile("bar.sync %0, 64;" ::"r"(bar) : "memory");
+    return emulc(eadd(eadd(eadd(red[0], red[1]), red[2]), red[3]), C(0.5));
+}
+// one warp: the interior elements of a chunk of kn vertices, whose positions
+// pos(k, x, y) gives, about (cx, cy); in lane 0
+template <typename C, typename Pos>
+__device__ __forceinline__ typename Ext<C>::E chunk_area(int kn, int lane, typename Ext<C>::E cx,
+                                                         typename Ext<C>::E cy, Pos pos) {
+    using E = typename Ext<C>::E;
+    E acc = ezero<E>();
+#pragma unroll
+    for (int q = 0; q < kChunkV / 32; ++q) {
+        const int k = lane + 32 * q;
+        if (k + 1 < kn) {
+            E xa, ya, xb, yb;
+            pos(k, xa, ya);
+            pos(k + 1, xb, yb);
+            acc = eadd(acc, cross_about<E>(cx, cy, xa, ya, xb, yb));
+        }
+    }
+    __syncwarp();
+    return warp_tree<E>(acc, lane);
+}
+// one warp: area of a long ring from its chunks' sums; u0: advance unit of its
+// first chunk; in lane 0
+template <typename C>
+__device__ typename Ext<C>::E ring_area_parts(const MarkerArgs& a, int off, int n, int u0, int lane) {
+    using E = typename Ext<C>::E;
+    E cx, cy;
+    PosIO<C>::load(a.Xp, off, cx, cy);
+    E acc = ezero<E>();
+    const int nchunk = (n + kChunkV - 1) / kChunkV;
+    for (int i = lane; i < nchunk; i += 32) {
+        const int last = i + 1 == nchunk ? n - 1 : (i + 1) * kChunkV - 1;
+        E xa, ya, xb, yb, part, unused;
+        load_pos<C>(a, off + last, xa, ya);
+        load_pos<C>(a, off + (last == n - 1 ? 0 : last + 1), xb, yb);
+        PosIO<C>::load(a.area_part, u0 + i, part, unused);
+        acc = eadd(acc, eadd(part, cross_about<E>(cx, cy, xa, ya, xb, yb)));
+    }
+    __syncwarp();
+    return emulc(warp_tree<E>(acc, lane), C(0.5));
+}
+// the area of ring m by warps w0, w0 + 1 (the second only helps short rings);
+// valid in lane 0 of the first; au0: advance unit of its first chunk (long rings)
+template <typename C>
+__device__ __forceinline__ typename Ext<C>::E ring_area(const MarkerArgs& a, int off, int n, int au0, int w0,
+                                                        typename Ext<C>::E* red, int bar) {
+    if (n <= kDirectArea) return ring_area_direct<C>(a, off, n, w0, red, bar);
+    if ((threadIdx.x >> 5) == w0) return ring_area_parts<C>(a, off, n, au0, threadIdx.x & 31);
+    return ezero<typename Ext<C>::E>();
 }
 
-// four block-wide sums in the compute type at once (every thread gets all four
-// in its arguments); each by a fixed shuffle tree per warp, then every thread
-// adds the warps' partials in a fixed tree of eight (blocks have at most eight
-// warps).  One barrier: `red` (4 x 8) is the call's own.
-template <typename C>
-__device__ void block_sum4_c(C& v0, C& v1, C& v2, C& v3, C (*red)[8]) {
-    C v[4] = {v0, v1, v2, v3};
+// N block-wide sums in the compute type at once (every thread gets all of
+// them); each by a fixed shuffle tree per warp, then every thread adds the
+// warps' partials in a fixed tree of eight (blocks have at most eight warps).
+// One barrier: `red` is the call's own.
+template <typename C, int N>
+__device__ __forceinline__ void block_sum_c(C (&v)[N], C (*red)[8]) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] += __shfl_down_sync(kFull, v[q], o);
+        for (int q = 0; q < N; ++q) v[q] += __shfl_down_sync(kFull, v[q], o);
     const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if ((threadIdx.x & 31) == 0) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) red[q][w] = v[q];
+        for (int q = 0; q < N; ++q) red[q][w] = v[q];
     }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < N; ++q) {
         C t[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) t[k] = k < nw ? red[q][k] : C(0);
         v[q] = ((t[0] + t[4]) + (t[2] + t[6])) + ((t[1] + t[5]) + (t[3] + t[7]));
     }
-    v0 = v[0];
-    v1 = v[1];
-    v2 = v[2];
-    v3 = v[3];
 }
 
-// Box of one segment from positions held by a group of kSegV consecutive lanes
-// (lane g of the group holds vertex v0 + g; lanes past the segment end hold a
-// copy of the first vertex).  FP32 offsets from the first vertex; centre x
-// wrapped into [0, nx).  All 32 lanes call it.
+// Boxes of the segments and of the screening group that a warp's positions
+// form: lane l holds vertex l of the group; lanes g, g + 1, .. of a segment past
+// its end hold a copy of its first vertex.  FP32 offsets from the segment's
+// first vertex; centre x wrapped into [0, nx).  sg: this lane's segment (-1:
+// none), gr: the warp's group (-1: none).  The group's box is widened by 1e-3
+// (its own roundings stay below 1e-3 of a lattice unit).  All 32 lanes call it.
 template <typename C>
-__device__ __forceinline__ void seg_box_regs(const MarkerArgs& a, int sg, int lane, typename Ext<C>::E x,
+__device__ __forceinline__ void seg_box_regs(const MarkerArgs& a, int sg, int gr, int lane, typename Ext<C>::E x,
                                              typename Ext<C>::E y) {
     using E = typename Ext<C>::E;
     const int g0 = lane & ~(kSegV - 1);
-    // first vertex of the group, broadcast in its (hi, lo) parts
-    E ax, ay;
+    // first vertex of the segment, broadcast in its (hi, lo) parts
+    E ax, ay, wx, wy;
     shfl_e(ax, x, g0);
     shfl_e(ay, y, g0);
     const float ox = float(etoc(esub(x, ax))), oy = float(etoc(esub(y, ay)));
     float lo_x = ox, hi_x = ox, lo_y = oy, hi_y = oy;
+#pragma unroll
     for (int o = kSegV / 2; o > 0; o >>= 1) {
         lo_x = fminf(lo_x, __shfl_xor_sync(kFull, lo_x, o));
         hi_x = fmaxf(hi_x, __shfl_xor_sync(kFull, hi_x, o));
         lo_y = fminf(lo_y, __shfl_xor_sync(kFull, lo_y, o));
         hi_y = fmaxf(hi_y, __shfl_xor_sync(kFull, hi_y, o));
     }
+    const float Lx = a.f.nx;
     if (sg >= 0 && lane == g0) {
-        const float Lx = a.f.nx;
         const float cx = float(ehi(ax)) + 0.5f * (lo_x + hi_x);
         a.seg_box[sg] = make_float4(cx - Lx * floorf(cx * a.f.inv_nx), float(ehi(ay)) + 0.5f * (lo_y + hi_y),
                                     0.5f * (hi_x - lo_x), 0.5f * (hi_y - lo_y));
+    }
+    shfl_e(wx, x, 0);
+    shfl_e(wy, y, 0);
+    const float dx = float(etoc(esub(ax, wx))), dy = float(etoc(esub(ay, wy)));
+    lo_x = sg >= 0 ? lo_x + dx : 1e30f;
+    hi_x = sg >= 0 ? hi_x + dx : -1e30f;
+    lo_y = sg >= 0 ? lo_y + dy : 1e30f;
+    hi_y = sg >= 0 ? hi_y + dy : -1e30f;
+#pragma unroll
+    for (int o = kSegV; o < kGroupV; o <<= 1) {
+        lo_x = fminf(lo_x, __shfl_xor_sync(kFull, lo_x, o));
+        hi_x = fmaxf(hi_x, __shfl_xor_sync(kFull, hi_x, o));
+        lo_y = fminf(lo_y, __shfl_xor_sync(kFull, lo_y, o));
+        hi_y = fmaxf(hi_y, __shfl_xor_sync(kFull, hi_y, o));
+    }
+    if (gr >= 0 && lane == 0) {
+        const float cx = float(ehi(wx)) + 0.5f * (lo_x + hi_x);
+        a.group_box[gr] = make_float4(cx - Lx * floorf(cx * a.f.inv_nx), float(ehi(wy)) + 0.5f * (lo_y + hi_y),
+                                      0.5f * (hi_x - lo_x) + 1e-3f, 0.5f * (hi_y - lo_y) + 1e-3f);
     }
 }
 
@@ -251,28 +328,37 @@ __device__ __forceinline__ Shape<C> load_shape(const MarkerArgs& a, int v) {
     s.j0 = o.y;
     return s;
 }
+// (every node is read, rows outside the walls at the nearest row with their
+// weight 0: a branch per row made three round trips of one, 3400 cycles of the
+// advance kernel's chain)
 template <typename C>
 __device__ __forceinline__ void interp_vertex(const MarkerArgs& a, const Shape<C>& s, C& Ux, C& Uy) {
     const C* ux = static_cast<const C*>(a.ux);
     const C* uy = static_cast<const C*>(a.uy);
+    int i[3];
+    size_t row[3];
+    bool in[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        i[q] = s.i0 + q - 1;
+        i[q] = i[q] < 0 ? i[q] + a.nx : (i[q] >= a.nx ? i[q] - a.nx : i[q]);
+        int j = s.j0 + q - 1;
+        in[q] = !a.walls || (j >= 0 && j < a.ny);
+        j = a.walls ? min(max(j, 0), a.ny - 1) : (j < 0 ? j + a.ny : (j >= a.ny ? j - a.ny : j));
+        row[q] = (size_t)j * a.nx;
+    }
+    C u[9], v[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        u[k] = ux[row[k / 3] + i[k % 3]];
+        v[k] = uy[row[k / 3] + i[k % 3]];
+    }
     C sx = C(0), sy = C(0);
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        int j = s.j0 + b - 1;
-        if (a.walls) {
-            if (j < 0 || j >= a.ny) continue;
-        } else {
-            j = j < 0 ? j + a.ny : (j >= a.ny ? j - a.ny : j);
-        }
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            int i = s.i0 + q - 1;
-            i = i < 0 ? i + a.nx : (i >= a.nx ? i - a.nx : i);
-            const C w = s.w[b * 3 + q];
-            const size_t node = (size_t)j * a.nx + i;
-            sx += w * ux[node];
-            sy += w * uy[node];
-        }
+    for (int k = 0; k < 9; ++k) {
+        const C w = in[k / 3] ? s.w[k] : C(0);
+        sx += w * u[k];
+        sy += w * v[k];
     }
     Ux = sx;
     Uy = sy;
