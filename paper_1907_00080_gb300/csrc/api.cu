@@ -377,15 +377,8 @@ static lbib_status finalize(lbib_ctx* c) {
         if ((c->ny + c->ty - 1) / c->ty > kMaxGridY)
             return fail(c, LBIB_E_INVALID, "lattice too tall for the row-tile form: more than 65535 x 16 rows");
     }
-    // force flags per 32 nodes of a row, in both kernel forms: a flagged tile
-    // reads and later clears the spread force and writes u only there (with
-    // tiles of a whole block or segment, red cells that cross most of them
-    // made nearly every node pay those 40 bytes)
-    c->tile_w = 32;
-    c->tile_h = 1;
-    c->tiles_x = (c->nx + c->tile_w - 1) / c->tile_w;
-    c->tiles_y = (c->ny + c->tile_h - 1) / c->tile_h;
-    c->ntiles = c->tiles_x * c->tiles_y;
+    c->tiles_x = (c->nx + 31) / 32;
+    c->ntiles = c->tiles_x * c->ny;
 
     const int nv = c->nv, nm = c->nmem, nl = c->nlig;
     const int nr = c->have_receptors ? (int)(c->h_rec.size() / 2) : 0;
@@ -611,8 +604,8 @@ static lbib_status finalize(lbib_ctx* c) {
     int* d_rcs = ar.take<int>(rcell_start.size());
     int* d_rci = ar.take<int>(rcell_ids.size());
     void* d_rcpos = ar.take<double>(2 * (size_t)nr);
-    c->flags[0] = ar.take<int>(c->ntiles);
-    c->flags[1] = ar.take<int>(c->ntiles);
+    c->flags[0] = ar.take<unsigned>(c->ntiles);
+    c->flags[1] = ar.take<unsigned>(c->ntiles);
     c->d_areas = ar.take<double>(nm + 1);
     int* d_fu = ar.take<int>(fu.size());
     int* d_au = ar.take<int>(au.size());
@@ -731,7 +724,7 @@ static lbib_status finalize(lbib_ctx* c) {
     a.sigma = c->bp.sigma; a.y_eq = c->bp.y_eq; a.d_cut = c->bp.d_cut; a.d_break = c->bp.d_break;
     a.kf_dt = c->bp.kf_dt; a.kr0_dt = c->bp.kr0_dt; a.beta_f = c->bp.beta_f; a.beta_r = c->bp.beta_r;
     a.seed = c->bp.seed; a.instance = c->bp.instance;
-    a.tile_w = c->tile_w; a.tile_h = c->tile_h; a.tiles_x = c->tiles_x; a.tiles_y = c->tiles_y;
+    a.tiles_x = c->tiles_x;
     a.status = c->d_status;
     a.f.nx = (float)c->nx; a.f.ny = (float)c->ny; a.f.inv_nx = (float)a.inv_nx; a.f.inv_ny = (float)a.inv_ny;
     a.f.sigma = (float)a.sigma; a.f.y_eq = (float)a.y_eq; a.f.inv_y_eq = (float)a.inv_y_eq;
@@ -792,8 +785,6 @@ static LbArgs lb_args(const lbib_ctx* c, int src, int gpar, int clear_other) {
     // cost DRAM bandwidth)
     l.g_prefetch = !c->no_g_prefetch &&
                    (size_t)c->nx * c->ny * (2 * 9 * c->pop_elem + sizeof(longlong2)) <= (size_t)64 << 20;
-    l.tile_w = c->tile_w;
-    l.tile_h = c->tile_h;
     l.tiles_x = c->tiles_x;
     l.status = c->d_status;
     if (c->nv == 0) {

@@ -123,6 +123,39 @@ __device__ __forceinline__ int wrap_index(int i, int n, float inv_n) {
     return r < 0 ? r + n : (r >= n ? r - n : r);
 }
 
+// flag the nodes of a stencil (origin wrapped into the lattice), one word of
+// three neighbouring nodes' bits at a time
+__device__ __forceinline__ void flag_nodes(const MarkerArgs& a, int i0, int j0) {
+    const int il = i0 == 0 ? a.nx - 1 : i0 - 1, ir = i0 + 1 == a.nx ? 0 : i0 + 1;
+    const int wl = il >> 5, wm = i0 >> 5, wr = ir >> 5;
+    unsigned bl = 1u << (il & 31), bm = 1u << (i0 & 31), br = 1u << (ir & 31);
+    // (a row of 32 k + 1 nodes has its last node alone in a word)
+    if (wr == wl) {
+        bl |= br;
+        br = 0u;
+    }
+    if (wm == wl) {
+        bl |= bm;
+        bm = 0u;
+    } else if (wm == wr) {
+        br |= bm;
+        bm = 0u;
+    }
+#pragma unroll
+    for (int b = -1; b <= 1; ++b) {
+        int j = j0 + b;
+        if (a.walls) {
+            if (j < 0 || j >= a.ny) continue;
+        } else {
+            j = j < 0 ? j + a.ny : (j >= a.ny ? j - a.ny : j);
+        }
+        unsigned* row = a.flags + (size_t)j * a.tiles_x;
+        atomicOr(row + wl, bl);
+        if (br) atomicOr(row + wr, br);
+        if (bm) atomicOr(row + wm, bm);
+    }
+}
+
 // IB shape functions at a position: nine nearest nodes, Roma weights, MLS
 // (basis 1, dx, dy) re-solved where wall rows drop out.  Node indices are
 // clamped so that a runaway position still stays in range; the advance kernel
@@ -400,6 +433,7 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
             reinterpret_cast<int2*>(a.stencil)[v] = make_int2(i0w, j0s);
             s_i0[j] = i0w;
             s_j0[j] = j0s;
+            flag_nodes(a, i0w, j0s);
         }
     } else if (wid == 4) {
         const int own0 = a.fu[3 * unit + 2].y + k0 / kGroupV;
@@ -570,7 +604,7 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
     }
     __syncthreads();
     // spreading (Sec. 2.2, the transpose of the interpolation): w_j F_v into the
-    // fixed-point force field; flag the fused-kernel tiles hit
+    // fixed-point force field
     for (int p = tid; p < 9 * kn; p += kForceThreads) {
         const int j = p / 9, q9 = p - 9 * j;
         const int b = q9 / 3, q = q9 - 3 * b;
@@ -590,7 +624,6 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
         unsigned long long* gp = reinterpret_cast<unsigned long long*>(a.gsum + (size_t)jj * a.nx + ii);
         atomicAdd(gp, (unsigned long long)to_fix<C>(gx));
         atomicAdd(gp + 1, (unsigned long long)to_fix<C>(gy));
-        a.flags[(jj / a.tile_h) * a.tiles_x + ii / a.tile_w] = 1;
     }
 }
 

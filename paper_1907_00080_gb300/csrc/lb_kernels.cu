@@ -1,5 +1,5 @@
 // Lattice-Boltzmann kernels: the fused pull-stream + bounce-back + moments +
-// Guo-forced BGK collision with the spread IB force read per flagged tile (the
+// Guo-forced BGK collision with the spread IB force read per flagged node (the
 // hot kernel), and the small helpers that convert between the stored
 // post-collision deviations and user-facing populations.
 //
@@ -35,7 +35,7 @@ __device__ __forceinline__ void load_pack(const S* __restrict__ row, int x0, boo
 // 32*VEC consecutive x of one row, so every row predicate is warp-uniform; the
 // x-shifted pulls load aligned vectors and take the single off-vector element
 // from the neighbouring lane (or, at the warp edge, with one scalar load).
-// IB: 0 no markers; 1 the spread force read in the tiles the spreading
+// IB: 0 no markers; 1 the spread force read at the nodes the spreading
 // flagged; 2 the same, with every node's force read up front (see below)
 // The tile (bx, by) of the lattice `a`: the body of the single-lattice kernel
 // (bx, by = blockIdx) and of the batched kernel (one block per (lattice, tile)).
@@ -87,12 +87,9 @@ __device__ __forceinline__ void lb_tile(const LbArgs& a, int bx, int by) {
         dep_trigger();
     }
 
-    // ---- this thread's force tile and its flags: during a step the row-tile
-    // form flags segments of 32 nodes of one row (tile_w = 32, tile_h = 1), so
-    // the threads that share a flag are lanes of one warp; in the fields-only
-    // read-back the tiles may be those of the persistent form.  On lattices
-    // that stay in L2, the spread force of every node is read with the flags
-    // (the field is zero outside the tiles this step's spreading touched)
+    // ---- the flag words of this thread's nodes, which lie in one word (x0 is a
+    // multiple of VEC).  On lattices that stay in L2, the spread force of every
+    // node is read with the flags (the field is zero at the other nodes)
     // instead of after them
     longlong2 gpre[VEC];
     const bool pre_g = IB == 2 && a.g_prefetch && ok;
@@ -100,11 +97,12 @@ __device__ __forceinline__ void lb_tile(const LbArgs& a, int bx, int by) {
 #pragma unroll
         for (int k = 0; k < VEC; ++k) gpre[k] = a.gsum[(size_t)y * nx + x0 + k];
     }
-    int t = 0, flag = 0, flag_o = 0;
-    if (HAS_IB) {
-        t = (min(y, ny - 1) / a.tile_h) * a.tiles_x + min(x0, nx - 1) / a.tile_w;
-        flag = a.flags[t];
-        if (a.clear_other) flag_o = a.flags_other[t];
+    size_t t = 0;
+    unsigned word = 0, word_o = 0;
+    if (HAS_IB && ok) {
+        t = (size_t)y * a.tiles_x + (x0 >> 5);
+        word = a.flags[t];
+        if (a.clear_other) word_o = a.flags_other[t];
     }
 
     // ---- pull streaming (Eq. BGK left side) with half-way bounce-back: the
@@ -144,15 +142,10 @@ __device__ __forceinline__ void lb_tile(const LbArgs& a, int bx, int by) {
         Gx[k] = LbConst<C>::gx(a);
         Gy[k] = LbConst<C>::gy(a);
     }
-    bool flagged = false;
+    const unsigned flagged = HAS_IB ? (word >> (x0 & 31)) & ((1u << VEC) - 1u) : 0u;
     if (HAS_IB) {
-        flagged = flag != 0;
-        const bool fo = flag_o != 0;
-        // every thread has read flags_other[t] before it is cleared
-        if (a.tile_h == 1 && a.tile_w <= 32 * VEC && 32 % a.tile_w == 0) __syncwarp();
-        else __syncthreads();
         const size_t node = (size_t)y * nx + x0;
-        if (flagged && ok) {
+        if (flagged) {
 #pragma unroll
             for (int k = 0; k < VEC; ++k) {
                 const longlong2 g = pre_g ? gpre[k] : a.gsum[node + k];
@@ -160,13 +153,15 @@ __device__ __forceinline__ void lb_tile(const LbArgs& a, int bx, int by) {
                 Gy[k] += from_fix<C>(g.y);
             }
         }
-        if (fo) {
-            if (ok) {
+        // every thread has read its word of flags_other before it is cleared (the
+        // threads of a word are lanes of one warp)
+        __syncwarp();
+        if (word_o) {
+            if ((word_o >> (x0 & 31)) & ((1u << VEC) - 1u)) {
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) a.gclear[node + k] = make_longlong2(0, 0);
             }
-            // one thread per flag: the one at the tile's first node
-            if (ok && x0 % a.tile_w == 0 && y % a.tile_h == 0) a.flags_other[t] = 0;
+            if ((x0 & 31) == 0) a.flags_other[t] = 0;
         }
     }
 

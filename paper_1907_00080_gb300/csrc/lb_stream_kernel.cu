@@ -11,9 +11,8 @@
 // thread takes NPT consecutive nodes: one vector shared-memory load per
 // direction (plus one element for the x-shifted directions) and one vector
 // global store per direction.  The spread IB force is read straight from
-// global memory where the segment's 32-node force tiles hold markers (their
-// flags are fetched kStages segments ahead by one warp and kept in shared
-// memory with the stage).
+// global memory at the flagged nodes (the flag words are fetched segments
+// ahead by one warp and kept in shared memory with the stage).
 //
 // Staged row of direction i (HALO = one 16-byte chunk on each side):
 //   [x0 - HALO, x0 + W + HALO) of plane i, row y - e_iy   (interior rows)
@@ -22,8 +21,7 @@
 // copy of the other end of the row, for the three directions that pull
 // across that end (e_ix = 1 at x = 0, e_ix = -1 at x = NX - 1).  The arithmetic per node is
 // collide_node(), the same as the row-tile kernel's, so both forms give the
-// same bits.  The force tiles are 32 nodes of one row, as in the row-tile
-// form.  The same bodies serve one lattice (arguments in the kernel's
+// same bits.  The same bodies serve one lattice (arguments in the kernel's
 // parameters) and a batch of lattices (ensemble members: the work list runs
 // over all members' segments, and the member's arguments are copied into the
 // stage's slot of shared memory when its segment is staged).
@@ -55,7 +53,8 @@ struct Geom {
     static constexpr int SMEM = kStages * STAGE_BYTES;
     static_assert(ROW_BYTES % 16 == 0, "16-byte aligned stage rows");
     static_assert(NPT <= H, "a thread's nodes never straddle the end of a row");
-    static_assert(W / 32 <= 64, "the tile flags of a segment fit two 32-bit masks");
+    static constexpr int NF = W / 32;                      // flag words of a segment (one bit per node)
+    static_assert(NF <= 64, "a warp fetches the flag words of a segment, two a lane");
 };
 
 template <typename T, int V>
@@ -207,13 +206,13 @@ struct ManyLattices {
     __device__ ItemRef staged_pos(long long, int st) const { return s_pos[st]; }
 };
 
-// Force-tile flags of one item (segment): W / 32 tiles of 32 nodes, lane q of
-// the fetching warp taking tiles q and q + 32.  Fetched kStages items ahead into
+// Flag words of one item (segment): W / 32 words of 32 nodes, lane q of the
+// fetching warp taking words q and q + 32.  Fetched three items ahead into
 // registers, stored into the stage's shared slot once that stage is free.
 // The fetch also keeps where the item lies (p, and m, its member in a batch)
 // for its staging.
 struct FlagRegs {
-    int f[2], o[2];
+    unsigned f[2], o[2];
     ItemRef p;
     int m;
 };
@@ -236,17 +235,57 @@ __device__ __forceinline__ void fetch_flags(const Items& it, long long item, int
         }
     }
 }
-// the whole warp: the item's flags as bit masks (tile q: bit q % 32 of word
-// q / 32), written by lane 0 into the stage's slot {flags 0-31, 32-63,
-// other parity's 0-31, 32-63}
-__device__ __forceinline__ void keep_flags(const FlagRegs& r, int lane, uint4* slot) {
-    const unsigned f0 = __ballot_sync(0xffffffffu, r.f[0] != 0), f1 = __ballot_sync(0xffffffffu, r.f[1] != 0);
-    const unsigned o0 = __ballot_sync(0xffffffffu, r.o[0] != 0), o1 = __ballot_sync(0xffffffffu, r.o[1] != 0);
-    if (lane == 0) *slot = make_uint4(f0, f1, o0, o1);
+// A flag word in a stage's slot: a bit per consumer thread (its NPT nodes), so
+// that the slots stay small (32 full words twice in four stages took the third
+// CTA of an SM from 16-bit storage with four nodes a thread: 64-member FP16
+// ensemble 150 -> 161 us per step).
+template <int NPT>
+struct ThreadBits {
+    using Word = unsigned;
+    __device__ static unsigned of(unsigned w) { return w; }
+    __device__ static unsigned at(unsigned w, int j0) { return (w >> (j0 & 31)) & ((1u << NPT) - 1u); }
+};
+template <>
+struct ThreadBits<4> {
+    using Word = unsigned char;
+    __device__ static unsigned of(unsigned w) {
+        w |= w >> 1;
+        w = (w | w >> 2) & 0x11111111u;
+        w = (w | w >> 3) & 0x03030303u;
+        w = (w | w >> 6) & 0x000f000fu;
+        return (w | w >> 12) & 0xffu;
+    }
+    __device__ static unsigned at(unsigned w, int j0) { return w >> (j0 >> 2 & 7) & 1u; }
+};
+template <>
+struct ThreadBits<8> {
+    using Word = unsigned char;
+    __device__ static unsigned of(unsigned w) {
+        w |= w >> 1;
+        w |= w >> 2;
+        w = (w | w >> 4) & 0x01010101u;
+        w = (w | w >> 7) & 0x00030003u;
+        return (w | w >> 14) & 0xfu;
+    }
+    __device__ static unsigned at(unsigned w, int j0) { return w >> (j0 >> 3 & 3) & 1u; }
+};
+// the stage's slot: this step's words, then the other parity's
+template <int NPT>
+struct FlagSlot {
+    static constexpr int NF = kThreads * NPT / 32;
+    typename ThreadBits<NPT>::Word f[NF], o[NF];
+};
+template <int NPT>
+__device__ __forceinline__ void keep_flags(const FlagRegs& r, int lane, FlagSlot<NPT>& slot) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int q = lane + 32 * h;
+        if (q < FlagSlot<NPT>::NF) {
+            slot.f[q] = ThreadBits<NPT>::of(r.f[h]);
+            slot.o[q] = ThreadBits<NPT>::of(r.o[h]);
+        }
+    }
 }
-// tile q's flag and other-parity flag from a stage's masks
-__device__ __forceinline__ int flag_of(const uint4& m, int q) { return ((q < 32 ? m.x : m.y) >> (q & 31)) & 1; }
-__device__ __forceinline__ int flag_other_of(const uint4& m, int q) { return ((q < 32 ? m.z : m.w) >> (q & 31)) & 1; }
 
 // Stage the nine source rows of `item` (plane i row y - e_iy, or plane opp(i)
 // row y at a wall; W nodes and a 16-byte halo each side, the periodic ends by
@@ -323,16 +362,18 @@ __device__ __forceinline__ S stored(typename Storage<S>::C c, float scl) {
 }
 
 // One thread's NPT nodes of a staged segment: pull from the stage, add the
-// spread force where its tile is flagged, collide, store; write u where
-// flagged; clear the other parity's force where its tile was flagged (and the
-// flag, by the thread at the tile's first node).  Three forms, chosen per warp
+// spread force if one of them is flagged (`flag`; the field is zero at nodes
+// that are not), collide, store; write u if flagged; clear the other parity's
+// force if it was flagged there (`flag_o`; the words themselves are cleared by
+// consume_warp).  Three forms, chosen per warp
 // (see consume_warp), with the same arithmetic per node: EDGE, a row next to a
 // wall (bounce-back pulls and the Zou-He rebuild checked per direction);
-// otherwise FORCED, a warp with a flagged force tile among its own, or neither,
+// otherwise FORCED, a warp with a flagged node among its own, or neither,
 // where the body force is the only force and the collision's force terms are
 // the same for every node.
 template <typename S, int NPT, bool WALLS, bool FORCED, bool EDGE>
-__device__ __forceinline__ void consume(const LbArgs& A, ItemRef p, const S* sp, int j0, int flag, int flag_o) {
+__device__ __forceinline__ void consume(const LbArgs& A, ItemRef p, const S* sp, int j0, unsigned flag,
+                                        unsigned flag_o) {
     using C = typename Storage<S>::C;
     using Gm = Geom<S, NPT>;
     constexpr int H = Gm::H;
@@ -451,27 +492,29 @@ __device__ __forceinline__ void consume(const LbArgs& A, ItemRef p, const S* sp,
     if (flag_o) {
 #pragma unroll
         for (int q = 0; q < NPT; ++q) A.gclear[node0 + q] = make_longlong2(0, 0);
-        // the tile's flag was fetched kStages segments ago; nothing reads it again
-        if (((p.x0 + j0) & 31) == 0) A.flags_other[(long long)y * A.tiles_x + ((p.x0 + j0) >> 5)] = 0;
     }
 }
 
 // A consumer warp's part of a staged segment (the threads with nodes in it):
 // with SPLIT, the form of consume for the warp, from the segment's row and the
-// flags of the NPT force tiles the warp covers (tiles warp * NPT .. + NPT - 1,
-// all in one word of the stage's masks), a choice uniform over the warp;
-// without, the general form for every warp (the barrier schedule: on the
-// FP32 probe the three forms took 7% longer there, for 13% fewer
-// instructions, while the producer-warp kernels gained).
+// flag words of the 32 NPT nodes the warp covers, a choice uniform over the
+// warp; without, the general form for every warp (the barrier schedule: on the
+// FP32 probe the three forms took 7% longer there, for 13% fewer instructions,
+// while the producer-warp kernels gained).
 template <typename S, int NPT, bool WALLS, bool SPLIT>
-__device__ __forceinline__ void consume_warp(const LbArgs& A, ItemRef p, const S* sp, int tid, const uint4& fm) {
-    static_assert(32 % NPT == 0, "a warp's tiles lie in one mask word");
-    const int j0 = tid * NPT, q0 = (tid >> 5) * NPT;
-    const int flag = flag_of(fm, j0 >> 5), flag_o = flag_other_of(fm, j0 >> 5);
-    const unsigned warp_tiles = ((q0 < 32 ? fm.x : fm.y) >> (q0 & 31)) & ((1u << NPT) - 1u);
+__device__ __forceinline__ void consume_warp(const LbArgs& A, ItemRef p, const S* sp, int tid,
+                                             const FlagSlot<NPT>& fm) {
+    const int j0 = tid * NPT, q0 = (tid >> 5) * NPT, q = j0 >> 5;
+    const unsigned flag = ThreadBits<NPT>::at(fm.f[q], j0), flag_o = ThreadBits<NPT>::at(fm.o[q], j0);
+    if (fm.o[q] != 0u && (j0 & 31) == 0)
+        // the word was fetched segments ago; nothing reads it again
+        A.flags_other[(long long)p.y * A.tiles_x + (p.x0 >> 5) + q] = 0;
+    unsigned any = 0;
+#pragma unroll
+    for (int k = 0; k < NPT; ++k) any |= fm.f[q0 + k];
     if (!SPLIT || (WALLS && (p.y == 0 || p.y == A.ny - 1)))
         consume<S, NPT, WALLS, true, true>(A, p, sp, j0, flag, flag_o);
-    else if (warp_tiles != 0u)
+    else if (any != 0u)
         consume<S, NPT, WALLS, true, false>(A, p, sp, j0, flag, flag_o);
     else
         consume<S, NPT, WALLS, false, false>(A, p, sp, j0, flag, flag_o);
@@ -482,7 +525,7 @@ __device__ __forceinline__ void consume_warp(const LbArgs& A, ItemRef p, const S
 // its own arrival on the stage's "empty" barrier), warp 8 produces: lane 0
 // waits for that barrier (eight arrivals once the consumers have passed the
 // segment), the lanes store
-// the segment's tile flags, lane 0 sets the expected bytes, then lanes 0-8
+// the segment's flags, lane 0 sets the expected bytes, then lanes 0-8
 // each issue the copies of one direction.  Stage s also has a "full" barrier
 // (the producer's expect-tx plus the copies' bytes).  Issuing from nine lanes
 // instead of one thread keeps the producer ahead of the short 16-bit segments.
@@ -493,7 +536,7 @@ __device__ __forceinline__ void stream_ws(const Items& it) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kStages];
     __shared__ __align__(8) unsigned long long empty[kStages];
-    __shared__ uint4 s_fm[kStages];  // tile-flag masks of each stage's item (see keep_flags)
+    __shared__ FlagSlot<NPT> s_fm[kStages];  // each stage's flag words
     __shared__ int s_last_issued[kStages];
     __shared__ volatile int s_abort;
 
@@ -517,7 +560,7 @@ __device__ __forceinline__ void stream_ws(const Items& it) {
     const int warp = tid >> 5, lane = tid & 31;
     if (warp == kConsumerWarps) {
         // ---- producer: stage segment k once the consumers have left the
-        // segment k - kStages that used the same stage; its tile flags were
+        // segment k - kStages that used the same stage; its flags were
         // fetched three segments ahead (their latency stays off the producer's path)
         // prologue: the rows of the first kStages items (populations alone, which
         // the force kernel leaves alone), beside the tail of the predecessor;
@@ -554,7 +597,7 @@ __device__ __forceinline__ void stream_ws(const Items& it) {
             stop = __shfl_sync(0xffffffffu, stop, 0);
             if (stop) break;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            keep_flags(r0, lane, &s_fm[stage]);
+            keep_flags<NPT>(r0, lane, s_fm[stage]);
             it.stage_args(r0.p, r0.m, stage, lane);
             __syncwarp();
             const LbArgs& A = it.staged(stage);
@@ -613,7 +656,7 @@ __device__ __forceinline__ void stream_ws(const Items& it) {
 }
 
 // Barrier schedule (FP32, FP64): 256 threads; a CTA barrier ends each segment;
-// then warp 0 refills the stage with the segment kStages ahead: the tile flags
+// then warp 0 refills the stage with the segment kStages ahead: the flags
 // it fetched at the start of this one, the arguments (batches), the expected
 // bytes and the nine row copies (lanes 0-8, one direction each).
 template <typename S, int NPT, bool WALLS, typename Items>
@@ -622,7 +665,7 @@ __device__ __forceinline__ void stream_bar(const Items& it) {
     constexpr int W = Gm::W;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kStages];
-    __shared__ uint4 s_fm[kStages];  // tile-flag masks of each stage's item (see keep_flags)
+    __shared__ FlagSlot<NPT> s_fm[kStages];  // each stage's flag words
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long n_items = it.count();
@@ -675,7 +718,7 @@ __device__ __forceinline__ void stream_bar(const Items& it) {
             if (k < my_n) fetch_flags<W>(it, first + (long long)k * stride, lane, r[k], 0);
 #pragma unroll
         for (int k = 0; k < kStages; ++k)
-            if (k < my_n) keep_flags(r[k], lane, &s_fm[k]);
+            if (k < my_n) keep_flags<NPT>(r[k], lane, s_fm[k]);
     } else {
         dep_wait();
     }
@@ -704,7 +747,7 @@ __device__ __forceinline__ void stream_bar(const Items& it) {
         bad = __syncthreads_or(!ok) != 0;
         if (bad) break;
         if (warp == 0 && k + kStages < my_n) {
-            keep_flags(nf, lane, &s_fm[stage]);
+            keep_flags<NPT>(nf, lane, s_fm[stage]);
             issue(k + kStages, nf);
         }
     }

@@ -5,11 +5,11 @@
 //                each holds the post-collision deviations d*_i = f*_i - w_i of
 //                one step (pull scheme: the fused kernel streams while reading)
 //   u field      ux, uy [NY][NX] of the compute type, written by the fused
-//                kernel only in tiles that IB stencils touch
+//                kernel only at nodes that IB stencils touch
 //   markers      X^n, X^{n-1} as interleaved (x, y) doubles; F^n, U^n, the nine
 //                shape-function weights and the stencil origin per vertex
 //   IB force     two fixed-point (int64 x 2) per-node fields alternating with the
-//                step parity, plus a flag per fused-kernel tile that spreading touched
+//                step parity, plus a flag bit per node that spreading touched
 //   adhesion     per ligand: element vertices, bond, candidate; per receptor:
 //                position, owner, claim; receptors bucketed in a uniform grid
 #pragma once
@@ -90,8 +90,10 @@ template <> struct Storage<__nv_bfloat16> {
 // The IB force is spread into a per-node fixed-point field (int64 pairs scaled
 // by 2^52): integer addition is associative, so the atomics of the spreading
 // give the same bits in any order.  Two fields alternate with the step parity;
-// tiles that a step's spreading touched are flagged, and the fused kernel of
-// the following step zeroes them again.
+// nodes that a step's spreading touched are flagged, a bit each, and the fused
+// kernel of the following step zeroes them again.  (Flags of 32 nodes made 52%
+// of the 64-capillary ensemble's nodes pay the 40 bytes of a flagged node,
+// where the stencils touch 9%.)
 constexpr double kFixScale = 4503599627370496.0;          // 2^52
 constexpr double kFixInv = 1.0 / 4503599627370496.0;      // 2^-52
 
@@ -103,10 +105,10 @@ struct LbArgs {
     double* rho_out;       // fields mode: rho, ux, uy as doubles (may be null)
     double* ux_out;
     double* uy_out;
-    const longlong2* gsum; // [N] fixed-point IB force of this step (flagged tiles)
-    longlong2* gclear;     // [N] the other parity's field, zeroed in its flagged tiles
-    const int* flags;      // [ntiles] force tiles (32 nodes of a row) this step's spreading touched
-    int* flags_other;      // [ntiles] tiles the previous step's spreading touched
+    const longlong2* gsum; // [N] fixed-point IB force of this step (flagged nodes)
+    longlong2* gclear;     // [N] the other parity's field, zeroed at its flagged nodes
+    const unsigned* flags; // [ny][tiles_x] nodes this step's spreading touched, a bit each: word x / 32 of a row
+    unsigned* flags_other; // the nodes the previous step's spreading touched
     int clear_other;       // 1 during a step, 0 for read-backs and profiling
     int nx, ny;
     double omega;          // 1/tau
@@ -122,7 +124,7 @@ struct LbArgs {
     float uwf_bot, uwf_top;
     int fields_only;       // 1: write rho/ux/uy doubles, skip populations
     int g_prefetch;        // row tiles: read the spread force of every node up front (L2-resident lattices)
-    int tile_w, tile_h, tiles_x;  // force-tile geometry of the flags (32 x 1 nodes; tiles_x = ceil(nx / 32))
+    int tiles_x;           // flag words per row, ceil(nx / 32)
     int* status;           // device status word (StatusBits)
 };
 
@@ -202,10 +204,10 @@ struct MarkerArgs {
     double d_cut2;            // (d_cut (1 + 1e-12))^2, a conservative pre-check
     double sigma, y_eq, d_cut, d_break, kf_dt, kr0_dt, beta_f, beta_r;
     uint64_t seed, instance;
-    // tiles of the fused kernel, spreading target of this step
-    int tile_w, tile_h, tiles_x, tiles_y;
+    // spreading target of this step
+    int tiles_x;
     longlong2* gsum;
-    int* flags;
+    unsigned* flags;
     // step counter (this and the previous parity) and status
     long long* d_step;
     const long long* step_prev;
@@ -446,7 +448,7 @@ struct lbib_ctx {
 
     int vec = 0, ty = 0;      // tiling of the fused kernel (ty = 0: persistent bulk-copy form, vec = npt)
     int stream_grid = 0;      // CTAs of the persistent form (SMs x resident CTAs)
-    int tile_w = 0, tile_h = 0, tiles_x = 0, tiles_y = 0, ntiles = 0;
+    int tiles_x = 0, ntiles = 0;          // flag words per row and in all
 
     // host-side membrane staging
     std::vector<double> h_xy;
@@ -471,7 +473,7 @@ struct lbib_ctx {
     size_t dmem_bytes = 0;
     lbib::MarkerArgs ma{};
     longlong2* G[2] = {nullptr, nullptr};   // fixed-point IB force fields (by parity)
-    int* flags[2] = {nullptr, nullptr};      // spread-touched tiles (by parity)
+    unsigned* flags[2] = {nullptr, nullptr};  // spread-touched nodes (by parity)
     double* d_areas = nullptr;
     double* xy_stage = nullptr;             // 2*nv doubles for marker read/write
     double* d_obs = nullptr;                // 8*nmem doubles of membrane observables (lazy)
