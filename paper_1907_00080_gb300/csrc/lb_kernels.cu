@@ -61,6 +61,13 @@ __device__ __forceinline__ void lb_tile(const LbArgs& a, int bx, int by) {
         dep_wait();
         dep_trigger();
     }
+    // (FP64, and one node a thread with markers: every node's own element of the
+    // shifted directions is read straight away.  The off-vector elements and
+    // their shuffles cost FP64 the registers that hide its pipe's latency,
+    // 60-member ensemble 1720 -> 1650 us per step, and the latency-bound small
+    // lattices their issue slots, capillary 12.1 -> 11.0 us; a 1501 x 333 lattice
+    // without markers is faster with the aligned loads, 7.6 against 8.1 us)
+    constexpr bool kDirect = (VEC == 1 && HAS_IB) || sizeof(S) == 8;
     C f[9][VEC], edge[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
@@ -74,6 +81,15 @@ __device__ __forceinline__ void lb_tile(const LbArgs& a, int bx, int by) {
         edge[i] = C(0);
         // (bounce-back: the population that left this node toward the wall comes back reversed)
         const S* row = bb ? src + (size_t)opp(i) * N + (size_t)y * nx : src + (size_t)i * N + (size_t)sy * nx;
+        if (kDirect && cx(i) != 0) {
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) {
+                int sx = bb ? x0 + k : x0 + k - cx(i);
+                sx = sx < 0 ? sx + nx : (sx >= nx ? sx - nx : sx);
+                f[i][k] = ok ? C(Storage<S>::load(row[sx], inv)) : C(0);
+            }
+            continue;
+        }
         load_pack<S, VEC>(row, x0, ok, inv, f[i]);
         if (cx(i) == 1) {
             if (lane == 0 && ok && !bb) edge[i] = Storage<S>::load(row[x0 == 0 ? nx - 1 : x0 - 1], inv);
@@ -116,6 +132,8 @@ __device__ __forceinline__ void lb_tile(const LbArgs& a, int bx, int by) {
             const C w = C(cx(i)) * wall_term<C>(a, cy(i) > 0);
 #pragma unroll
             for (int k = 0; k < VEC; ++k) f[i][k] += w;
+        } else if (kDirect) {
+            continue;
         } else if (cx(i) == 1) {
             // needs x0-1 .. x0+VEC-2
             C prev = __shfl_up_sync(FULL, f[i][VEC - 1], 1);
