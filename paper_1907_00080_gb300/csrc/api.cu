@@ -18,7 +18,8 @@ using namespace lbib;
 
 namespace {
 
-constexpr int kChunk = 16;  // steps per captured chunk graph (even)
+constexpr int kChunkLog2 = 4;
+constexpr int kChunk = 1 << kChunkLog2;  // steps per captured chunk graph of an ensemble (even)
 constexpr int kMaxGridY = 65535;  // largest y extent of a launch grid
 
 lbib_status fail(lbib_ctx* c, lbib_status st, const std::string& msg) {
@@ -330,7 +331,8 @@ extern "C" lbib_status lbib_set_wall_velocity(lbib_ctx* c, double u_bottom, doub
     if (!c) return LBIB_E_INVALID;
     if (c->walls == LBIB_WALLS_NONE) return fail(c, LBIB_E_INVALID, "moving walls need walls");
     if (!std::isfinite(u_bottom) || !std::isfinite(u_top)) return fail(c, LBIB_E_INVALID, "non-finite wall velocity");
-    if (c->graphs_ready || c->steps > 0) return fail(c, LBIB_E_STATE, "wall velocities are fixed at the first step");
+    if (c->graphs_ready || c->in_ensemble || c->steps > 0)
+        return fail(c, LBIB_E_STATE, "wall velocities are fixed at the first step");
     c->uw_bot = u_bottom;
     c->uw_top = u_top;
     choose_scale(c);
@@ -864,7 +866,7 @@ static cudaError_t enqueue_step(lbib_ctx* c, int src, cudaStream_t s, bool first
 // discard the captured step graphs (they are captured again on next use)
 static void drop_graphs(lbib_ctx* c) {
     for (int s = 0; s < 2; ++s)
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < lbib_ctx::kGraphs; ++k) {
             if (c->graph[s][k]) cudaGraphExecDestroy(c->graph[s][k]);
             if (c->graph_tmpl[s][k]) cudaGraphDestroy(c->graph_tmpl[s][k]);
             c->graph[s][k] = nullptr;
@@ -873,43 +875,55 @@ static void drop_graphs(lbib_ctx* c) {
     c->graphs_ready = false;
 }
 
-static lbib_status build_graphs(lbib_ctx* c) {
-    if (c->graphs_ready) return LBIB_OK;
+// the graph of 1 << k steps that start from buffer `start`
+static lbib_status build_graph(lbib_ctx* c, int start, int k) {
+    if (c->graph[start][k]) return LBIB_OK;
     cudaStream_t cap;
     CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
-    for (int start = 0; start < 2; ++start) {
-        for (int kind = 0; kind < 2; ++kind) {
-            cudaGraph_t g;
-            cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-            if (e != cudaSuccess) {
-                cudaStreamDestroy(cap);
-                return cuda_fail(c, e, "begin capture");
-            }
-            const int nsteps = kind == 0 ? 1 : kChunk;
-            int src = start;
-            cudaError_t le = cudaSuccess;
-            for (int k = 0; k < nsteps && le == cudaSuccess; ++k) {
-                le = enqueue_step(c, src, cap, k == 0, k == nsteps - 1);
-                src = 1 - src;
-            }
-            e = cudaStreamEndCapture(cap, &g);
-            if (le != cudaSuccess || e != cudaSuccess) {
-                cudaStreamDestroy(cap);
-                return cuda_fail(c, le != cudaSuccess ? le : e, "capture step");
-            }
-            e = cudaGraphInstantiate(&c->graph[start][kind], g, 0);
-            c->graph_tmpl[start][kind] = g;  // an ensemble embeds it as a child graph
-            if (e != cudaSuccess) {
-                cudaStreamDestroy(cap);
-                return cuda_fail(c, e, "instantiate step graph");
-            }
-        }
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) {
+        cudaStreamDestroy(cap);
+        return cuda_fail(c, e, "begin capture");
     }
+    const int nsteps = 1 << k;
+    int src = start;
+    cudaError_t le = cudaSuccess;
+    for (int q = 0; q < nsteps && le == cudaSuccess; ++q) {
+        le = enqueue_step(c, src, cap, q == 0, q == nsteps - 1);
+        src = 1 - src;
+    }
+    e = cudaStreamEndCapture(cap, &g);
     cudaStreamDestroy(cap);
+    if (le != cudaSuccess || e != cudaSuccess) {
+        if (g) cudaGraphDestroy(g);
+        return cuda_fail(c, le != cudaSuccess ? le : e, "capture step");
+    }
+    e = cudaGraphInstantiate(&c->graph[start][k], g, 0);
+    c->graph_tmpl[start][k] = g;  // an ensemble embeds it as a child graph
+    if (e != cudaSuccess) {
+        c->graph[start][k] = nullptr;
+        return cuda_fail(c, e, "instantiate step graph");
+    }
+    return LBIB_OK;
+}
+
+// ready to step: single steps from either buffer
+static lbib_status build_graphs(lbib_ctx* c) {
+    if (c->graphs_ready) return LBIB_OK;
+    for (int start = 0; start < 2; ++start) {
+        const lbib_status st = build_graph(c, start, 0);
+        if (st != LBIB_OK) return st;
+    }
     c->graphs_ready = true;
     return LBIB_OK;
 }
 
+// Sequences of 2, 4, .. 32 steps are captured when a call first needs them: a
+// call of n steps is a few launches for any n (7 steps were seven launches of
+// one step each, with a boundary of 2 us between them), and a first call
+// captures little more than it runs.  Within a capture of the caller's own
+// nothing is captured anew: the sequences there are serve any n.
 extern "C" lbib_status lbib_step(lbib_ctx* c, int64_t n) {
     if (!c || n < 0) return LBIB_E_INVALID;
     if (c->poisoned) return fail(c, LBIB_E_STATE, "context poisoned by an earlier device-side failure");
@@ -917,15 +931,18 @@ extern "C" lbib_status lbib_step(lbib_ctx* c, int64_t n) {
     if (st != LBIB_OK) return st;
     st = build_graphs(c);
     if (st != LBIB_OK) return st;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(c->stream, &cs));
     int64_t left = n;
-    while (left >= kChunk) {
-        CK(cudaGraphLaunch(c->graph[c->cur][1], c->stream));
-        left -= kChunk;  // even number of steps: the buffer roles are unchanged
-    }
     while (left > 0) {
-        CK(cudaGraphLaunch(c->graph[c->cur][0], c->stream));
-        c->cur = 1 - c->cur;
-        --left;
+        int k = 0;
+        while (k + 1 < lbib_ctx::kGraphs && left >= (int64_t)2 << k) ++k;
+        if (cs != cudaStreamCaptureStatusNone)
+            while (k > 0 && !c->graph[c->cur][k]) --k;
+        if ((st = build_graph(c, c->cur, k)) != LBIB_OK) return st;
+        CK(cudaGraphLaunch(c->graph[c->cur][k], c->stream));
+        if (k == 0) c->cur = 1 - c->cur;  // an even number of steps leaves the buffer roles
+        left -= (int64_t)1 << k;
     }
     c->steps += n;
     if (n > 0) c->fields_valid = true;
@@ -1299,11 +1316,7 @@ extern "C" const char* lbib_last_error(const lbib_ctx* c) { return c ? c->err.c_
 extern "C" void lbib_destroy(lbib_ctx* c) {
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
-    for (int s = 0; s < 2; ++s)
-        for (int k = 0; k < 2; ++k) {
-            if (c->graph[s][k]) cudaGraphExecDestroy(c->graph[s][k]);
-            if (c->graph_tmpl[s][k]) cudaGraphDestroy(c->graph_tmpl[s][k]);
-        }
+    drop_graphs(c);
     for (int b = 0; b < 2; ++b)
         if (c->f[b]) cudaFree(c->f[b]);
     if (c->ux) cudaFree(c->ux);
@@ -1546,8 +1559,13 @@ static lbib_status ensemble_build(lbib_ensemble* e) {
             for (size_t i = 0; i < e->m.size(); ++i) {
                 lbib_ctx* c = e->m[i];
                 cudaGraphNode_t node;
-                const cudaError_t r = cudaGraphAddChildGraphNode(&node, g, nullptr, 0,
-                                                                 c->graph_tmpl[e->cur0[i] ^ flip][kind]);
+                const int k = kind == 0 ? 0 : kChunkLog2, start = e->cur0[i] ^ flip;
+                const lbib_status st = build_graph(c, start, k);
+                if (st != LBIB_OK) {
+                    cudaGraphDestroy(g);
+                    return ens_fail(e, st, c->err);
+                }
+                const cudaError_t r = cudaGraphAddChildGraphNode(&node, g, nullptr, 0, c->graph_tmpl[start][k]);
                 if (r != cudaSuccess) {
                     cudaGraphDestroy(g);
                     return ens_fail(e, LBIB_E_CUDA, std::string("add member graph: ") + cudaGetErrorString(r));
@@ -1581,8 +1599,8 @@ extern "C" lbib_status lbib_ensemble_create(lbib_ctx* const* members, int32_t n,
             c->no_g_prefetch = true;
             drop_graphs(c);
         }
-        if (st == LBIB_OK) st = build_graphs(c);
         if (st != LBIB_OK) return st;
+        c->in_ensemble = true;
         if (cudaStreamSynchronize(c->stream) != cudaSuccess) return LBIB_E_CUDA;
     }
     lbib_ensemble* e = new lbib_ensemble();

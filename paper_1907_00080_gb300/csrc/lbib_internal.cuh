@@ -487,10 +487,13 @@ struct lbib_ctx {
     bool fields_valid = false;
     bool poisoned = false;
 
-    // captured step graphs: [start buffer][0: one step, 1: chunk of kChunk steps]
-    cudaGraphExec_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
-    cudaGraph_t graph_tmpl[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // kept for ensembles
-    bool graphs_ready = false;
+    // captured step graphs: [start buffer][k], 1 << k steps; single steps from the
+    // first use on, longer ones when a call first needs them
+    static constexpr int kGraphs = 6;
+    cudaGraphExec_t graph[2][kGraphs] = {};
+    cudaGraph_t graph_tmpl[2][kGraphs] = {};  // kept for ensembles
+    bool graphs_ready = false;   // set up to step
+    bool in_ensemble = false;
     bool no_g_prefetch = false;  // set for ensemble members (see lb_args)
 
     std::string err;

@@ -91,3 +91,19 @@ def test_ensemble_steps_together_and_apart(precision, tiling):
         same(state(a), state(b))
     one.close()
     many.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 7, 31, 32, 33, 63, 65])
+def test_any_number_of_steps(n):
+    """captured sequences of 1, 2, 4, .. 32 steps: any n, from either buffer"""
+    wl = inputs.capsule_128x32(bonds="stress")
+    a, b = (lbib.Simulation(wl, precision="f32") for _ in range(2))
+    for s in (a, b):
+        s.step(1)
+    a.step(n)
+    for _ in range(n):
+        b.step(1)
+    assert lbib.lbib_step_count(a.ctx) == lbib.lbib_step_count(b.ctx) == n + 1
+    same(state(a), state(b))
+    a.close()
+    b.close()
