@@ -23,6 +23,14 @@
 namespace lbib {
 namespace {
 
+// s += c x for c = -1, 0, 1 known at compile time.  (A product by 0 is an
+// instruction of the slow FP64 pipe that the compiler has to keep: these were
+// 25 of the 175 of the collision's transpose.)
+__device__ __forceinline__ void add_signed(double& s, int c, double x) {
+    if (c > 0) s += x;
+    else if (c < 0) s -= x;
+}
+
 // Transpose of collide_node<double> at one node.  d: pulled deviations, (Gx, Gy)
 // total force; yb: adjoints of the nine outputs d*_i, (ubx, uby) adjoint of the
 // velocity output.  Returns the adjoints of d and of G.  With eu_i = e_i.u and
@@ -38,8 +46,8 @@ __device__ __forceinline__ void collide_node_rev(const double (&d)[9], double Gx
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         drho += d[i];
-        jx += cx(i) * d[i];
-        jy += cy(i) * d[i];
+        add_signed(jx, cx(i), d[i]);
+        add_signed(jy, cy(i), d[i]);
     }
     const double rho = 1.0 + drho, r = 1.0 / rho;
     const double px = jx + 0.5 * Gx, py = jy + 0.5 * Gy;
@@ -68,10 +76,10 @@ __device__ __forceinline__ void collide_node_rev(const double (&d)[9], double Gx
         Sc += eu * eu * yE;
         const double deu = b * yO + (2.0 * c * eu + h * eG) * yE;  // along e_ip
         const double deG = g * yO + h * eu * yE;
-        uxb += cx(ip[p]) * deu;
-        uyb += cy(ip[p]) * deu;
-        Gbx += cx(ip[p]) * deG;
-        Gby += cy(ip[p]) * deG;
+        add_signed(uxb, cx(ip[p]), deu);
+        add_signed(uyb, cy(ip[p]), deu);
+        add_signed(Gbx, cx(ip[p]), deG);
+        add_signed(Gby, cy(ip[p]), deG);
     }
     // a, b, c -> drho, rho, u.u, u.G
     double drhob = om * Sa;
@@ -89,7 +97,11 @@ __device__ __forceinline__ void collide_node_rev(const double (&d)[9], double Gx
     drhob += rhob;
     const double omc = 1.0 - om;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) db[i] = omc * yb[i] + drhob + cx(i) * jxb + cy(i) * jyb;
+    for (int i = 0; i < 9; ++i) {
+        db[i] = om == 1.0 ? drhob : omc * yb[i] + drhob;
+        add_signed(db[i], cx(i), jxb);
+        add_signed(db[i], cy(i), jyb);
+    }
 }
 
 // velocity output of the collision at `node` (the field the markers interpolate)
@@ -181,17 +193,17 @@ __global__ void k_a_collide(const AdjointArgs a) {
     }
 }
 
-// Tasks of k_a_forces (blockIdx.y): one dual evaluation each, of the force
+// Tasks of k_a_forces: one dual evaluation each, of the force
 // terms of vertex v that depend on one seed.  Position seeds X_{v+d}: the
 // bending moment at v-1 depends on d in -2..0, the one at v on -1..1, the one
 // at v+1 on 0..2; bonds, stretching and the area penalty on -1..1.
 struct AdjTask {
-    signed char kind, d, coord;  // kind: a SeedKind, or kRepTask / kWeightsTask
+    signed char kind, d, coord;  // kind: a SeedKind, or kWeightsTask
     unsigned char terms;
 };
-constexpr int kRepTask = 100, kWeightsTask = 101;
+constexpr int kWeightsTask = 101;
 constexpr unsigned char kOther = kTermBond | kTermStretch | kTermArea;
-constexpr int kNumTasks = 33;
+constexpr int kNumTasks = 32;
 __constant__ AdjTask c_tasks[kNumTasks] = {
     // x coordinate
     {kPos, -2, 0, kTermBendL},
@@ -208,84 +220,68 @@ __constant__ AdjTask c_tasks[kNumTasks] = {
     // parameters and the area
     {kArea, 0, 0, kTermArea}, {kKs, 0, 0, kTermStretch}, {kSigma, 0, 0, kTermBond},
     {kKb, 0, 0, kTermBendL}, {kKb, 0, 0, kTermBendV}, {kKb, 0, 0, kTermBendR},
-    // repulsion pairs, shape functions against x_v and y_v
-    {kRepTask, 0, 0, 0}, {kWeightsTask, 0, 0, 0}, {kWeightsTask, 0, 1, 0}};
+    // shape functions against x_v and y_v
+    {kWeightsTask, 0, 0, 0}, {kWeightsTask, 0, 1, 0}};
 
-// Adjoint of the total Lagrangian force on vertex v and of its shape functions.
-// Bonds, stretching, bending and the area penalty depend on X_{v-2} .. X_{v+2},
-// the membrane's area, k_s, k_b and sigma: one dual evaluation per (seed, term
-// group) gives that part of the column dF_v/d(seed), and F_v-bar . column is
-// added to the seed's adjoint.  The repulsion -sum_b c0 d_vb^{-5/2} n_v (Eq.
-// repFor) is transposed pair by pair: through d_vb into X_v and X_b, and through
-// the vertex normal n_v into X_{v-1}, X_v, X_{v+1}.  The shape functions of v
-// depend on X_v alone (two seeds).  Each (vertex, task) is one thread: the FP64
-// chains are long, and one thread per vertex would leave most SMs idle.
-__global__ void k_a_forces(const AdjointArgs a) {
+// F_v-bar = sum_k W_vk G-bar(x_k), the spreading G(x_k) += W_vk F_v transposed,
+// and (gF, 9 values or null) the shape functions' share G-bar(x_k) . F_v
+__device__ __forceinline__ void force_adjoint(const AdjointArgs& a, int v, double& Fbx, double& Fby, double* gF) {
     const TangentArgs& t = a.t;
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= t.m.nv) return;
-    const AdjTask q = c_tasks[blockIdx.y];
-    // the spreading G(x_k) += W_vk F_v transposed: F_v-bar = sum_k W_vk G-bar(x_k),
-    // and the shape functions' share G-bar(x_k) . F_v
     const int i0 = t.st[2 * v], j0 = t.st[2 * v + 1];
     const double Fx = t.Fv[2 * v], Fy = t.Fv[2 * v + 1];
-    double Fbx = 0.0, Fby = 0.0, gF[9];
+    Fbx = Fby = 0.0;
+#pragma unroll
     for (int k = 0; k < 9; ++k) {
-        gF[k] = 0.0;
+        if (gF) gF[k] = 0.0;
         if (t.m.walls && (j0 + k / 3 - 1 < 0 || j0 + k / 3 - 1 >= t.m.ny)) continue;
         const size_t node = t_node(t, i0, j0, k);
         const double w = t.Wv[9 * v + k];
         const double gbx = a.Gbar[2 * node], gby = a.Gbar[2 * node + 1];
         Fbx += w * gbx;
         Fby += w * gby;
-        gF[k] = gbx * Fx + gby * Fy;
+        if (gF) gF[k] = gbx * Fx + gby * Fy;
     }
-    double* XB = a.XB_out;
-    if (q.kind == kWeightsTask) {
-        dual w[9];
-        bool in[9];
-        int si, sj;
-        t_vertex_weights(t, v, Seed{kPos, v, q.coord, -1}, w, in, si, sj);
-        double acc = 0.0;
-        for (int k = 0; k < 9; ++k)
-            if (in[k]) acc += (a.Wbar[9 * v + k] + gF[k]) * w[k].d;
-        atomicAdd(&XB[2 * v + q.coord], acc);
-        return;
-    }
+}
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Adjoint of the repulsion -sum_b c0 d_vb^{-5/2} n_v (Eq. repFor) of vertex v,
+// by one warp: transposed pair by pair, through d_vb into X_v and X_b, and
+// through the vertex normal n_v into X_{v-1}, X_v, X_{v+1}.  The lanes share the
+// other membranes' vertices, and the six columns of the normal.  (One thread
+// per vertex walked every vertex of each membrane in reach by itself: 128 us of
+// the 225 us of an adjoint step with two neighbouring red cells.)
+__device__ __forceinline__ void a_repulsion(const AdjointArgs& a, int v) {
+    const TangentArgs& t = a.t;
+    const int lane = threadIdx.x;
+    double Fbx, Fby;
+    force_adjoint(a, v, Fbx, Fby, nullptr);
     if (Fbx == 0.0 && Fby == 0.0) return;
     const int m = t_mem_of(t, v);
     const int off = t.m.mem_off[m], n = t.m.mem_n[m], k = v - off;
-    if (q.kind != kRepTask) {
-        if (q.kind == kSigma && t.m.nlig == 0) return;
-        const int u = q.kind == kPos ? t_ring(off, n, k + q.d) : -1;
-        dual fx, fy;
-        t_vertex_force(t, v, m, Seed{q.kind, u, q.coord, m}, fx, fy, q.terms);
-        const double g = Fbx * fx.d + Fby * fy.d;
-        double* dst = q.kind == kPos ? &XB[2 * u + q.coord]
-                      : q.kind == kArea ? &a.Abar[m]
-                      : q.kind == kKs   ? &a.ks_bar[m]
-                      : q.kind == kKb   ? &a.kb_bar[m]
-                                        : a.sigma_bar;
-        atomicAdd(dst, g);
-        return;
-    }
-    // the repulsion pairs of v
-    if (t.m.nmem < 2) return;
+    double* XB = a.XB_out;
     const double* X = static_cast<const double*>(t.m.X);
     const double xv = X[2 * v], yv = X[2 * v + 1];
     bool have_g = false;
-    VGeo g;
-    double nbx = 0.0, nby = 0.0, xvb = 0.0, yvb = 0.0;
+    double gnx = 0.0, gny = 0.0, nbx = 0.0, nby = 0.0, xvb = 0.0, yvb = 0.0;
     for (int mb = 0; mb < t.m.nmem; ++mb) {
         if (mb == m || !t_near_box(t, mb, xv, yv)) continue;
-        if (!have_g) {
-            g = t_vgeo(t, off, n, k, tangent_seed());
-            have_g = true;
-        }
-        const double gnx = g.nx.v, gny = g.ny.v;
         const int o2 = t.m.mem_off[mb], n2 = t.m.mem_n[mb];
-        for (int b = o2; b < o2 + n2; ++b) {
-            if (!t_rep_candidate(t, xv, yv, b)) continue;
+        for (int base = o2; base < o2 + n2; base += 32) {
+            const int b = base + lane;
+            const bool cand = b < o2 + n2 && t_rep_candidate(t, xv, yv, b);
+            if (!__any_sync(0xffffffffu, cand)) continue;
+            if (!have_g) {
+                const VGeo g = t_vgeo(t, off, n, k, tangent_seed());
+                gnx = g.nx.v;
+                gny = g.ny.v;
+                have_g = true;
+            }
+            if (!cand) continue;
             const double dxv = t_wrap_x(t, dual(xv - X[2 * b])).v;
             const double dyv = t_wrap_y(t, dual(yv - X[2 * b + 1])).v;
             // magnitude and its two partials with respect to (dx, dy)
@@ -305,16 +301,67 @@ __global__ void k_a_forces(const AdjointArgs a) {
         }
     }
     if (!have_g) return;
-    atomicAdd(&XB[2 * v], xvb);
-    atomicAdd(&XB[2 * v + 1], yvb);
-    if (nbx == 0.0 && nby == 0.0) return;
-    for (int dk = -1; dk <= 1; ++dk) {
-        const int u = t_ring(off, n, k + dk);
-        for (int c = 0; c < 2; ++c) {
-            const VGeo gs = t_vgeo(t, off, n, k, Seed{kPos, u, c, -1});
-            atomicAdd(&XB[2 * u + c], nbx * gs.nx.d + nby * gs.ny.d);
-        }
+    xvb = warp_sum(xvb);
+    yvb = warp_sum(yvb);
+    nbx = warp_sum(nbx);
+    nby = warp_sum(nby);
+    if (lane == 0) {
+        atomicAdd(&XB[2 * v], xvb);
+        atomicAdd(&XB[2 * v + 1], yvb);
     }
+    if ((nbx == 0.0 && nby == 0.0) || lane >= 6) return;
+    const int u = t_ring(off, n, k + lane / 2 - 1), c = lane & 1;
+    const VGeo gs = t_vgeo(t, off, n, k, Seed{kPos, u, c, -1});
+    atomicAdd(&XB[2 * u + c], nbx * gs.nx.d + nby * gs.ny.d);
+}
+
+// Adjoint of the total Lagrangian force on vertex v and of its shape functions.
+// Bonds, stretching, bending and the area penalty depend on X_{v-2} .. X_{v+2},
+// the membrane's area, k_s, k_b and sigma: one dual evaluation per (seed, term
+// group) gives that part of the column dF_v/d(seed), and F_v-bar . column is
+// added to the seed's adjoint.  The shape functions of v depend on X_v alone
+// (two seeds).  Each (vertex, task) is one thread: the FP64 chains are long, and
+// one thread per vertex would leave most SMs idle.  The repulsion takes a warp
+// a vertex (a_repulsion), in the launch's first blocks.
+__global__ void k_a_forces(const AdjointArgs a) {
+    const TangentArgs& t = a.t;
+    const int nrep = t.m.nmem > 1 ? t.m.nv : 0;
+    if ((int)blockIdx.x < nrep) {
+        a_repulsion(a, blockIdx.x);
+        return;
+    }
+    const int nvb = (t.m.nv + 31) / 32, blk = blockIdx.x - nrep;
+    const int v = (blk % nvb) * 32 + threadIdx.x;
+    if (v >= t.m.nv) return;
+    const AdjTask q = c_tasks[blk / nvb];
+    double Fbx, Fby, gF[9];
+    force_adjoint(a, v, Fbx, Fby, gF);
+    double* XB = a.XB_out;
+    if (q.kind == kWeightsTask) {
+        dual w[9];
+        bool in[9];
+        int si, sj;
+        t_vertex_weights(t, v, Seed{kPos, v, q.coord, -1}, w, in, si, sj);
+        double acc = 0.0;
+        for (int k = 0; k < 9; ++k)
+            if (in[k]) acc += (a.Wbar[9 * v + k] + gF[k]) * w[k].d;
+        atomicAdd(&XB[2 * v + q.coord], acc);
+        return;
+    }
+    if (Fbx == 0.0 && Fby == 0.0) return;
+    const int m = t_mem_of(t, v);
+    const int off = t.m.mem_off[m], n = t.m.mem_n[m], k = v - off;
+    if (q.kind == kSigma && t.m.nlig == 0) return;
+    const int u = q.kind == kPos ? t_ring(off, n, k + q.d) : -1;
+    dual fx, fy;
+    t_vertex_force(t, v, m, Seed{q.kind, u, q.coord, m}, fx, fy, q.terms);
+    const double g = Fbx * fx.d + Fby * fy.d;
+    double* dst = q.kind == kPos ? &XB[2 * u + q.coord]
+                  : q.kind == kArea ? &a.Abar[m]
+                  : q.kind == kKs   ? &a.ks_bar[m]
+                  : q.kind == kKb   ? &a.kb_bar[m]
+                                    : a.sigma_bar;
+    atomicAdd(dst, g);
 }
 
 // Adjoint of the enclosed area (shoelace): dA/dx_v = (y_{v+1} - y_{v-1}) / 2,
@@ -431,7 +478,7 @@ cudaError_t launch_adjoint_step(const AdjointArgs& a, cudaStream_t s) {
     // FP64-bound: 128-thread blocks, up to 16 per SM
     k_a_collide<<<(int)std::min<size_t>((N + 127) / 128, 152 * 16), 128, 0, s>>>(a);
     if (t.m.nv > 0) {
-        k_a_forces<<<dim3(nvb, kNumTasks), 32, 0, s>>>(a);
+        k_a_forces<<<(t.m.nmem > 1 ? t.m.nv : 0) + nvb * kNumTasks, 32, 0, s>>>(a);
         k_a_area<<<nvb, 32, 0, s>>>(a);
     }
     return cudaGetLastError();
