@@ -373,9 +373,9 @@ def lbib_main(args):
     roofline["share_of_kernel_time"] = top["ms_per_launch"] / sum(k["ms_per_launch"] for k in kernels)
     roofline["note"] = ("dominant kernel of the ensemble's time step (all 64 members in one launch), timed alone "
                         "with CUDA events on a scratch copy; algorithmic bytes = 9 populations read + 9 written "
-                        "per node (frac_with_ib also counts the IB coupling's bytes in the flagged force tiles: "
-                        "force read, velocity written, other parity cleared); traffic from the ncu summary of "
-                        "the same kernel under profiles/")
+                        "per node (frac_with_ib also counts the IB coupling's bytes in the flagged groups of "
+                        "nodes, one group per thread: force read, velocity written, other parity cleared); "
+                        "traffic from the ncu summary of the same kernel under profiles/")
 
     probe = probe16 = None
     if not args.no_probe and rank == 0:
@@ -454,8 +454,9 @@ def ensemble_kernels(lbib, torch, stream, wls, tiling, groups, precision, pk, tr
     with torch.cuda.stream(stream):
         scratch.step(4)
         scratch.sync()
-        # the force tiles the fused kernel reads, from the markers' positions
-        flagged = sum(flagged_nodes(wl, m.markers()) for wl, m in zip(wls, scratch.members))
+        # the nodes whose force the fused kernel reads, from the markers'
+        # positions: the groups of nodes that one of its threads takes
+        flagged = sum(flagged_nodes(wl, m.markers(), tiling[0]) for wl, m in zip(wls, scratch.members))
         kms = lbib.lbib_ensemble_profile_kernels(scratch.ens, 200)
     scratch.close()
     alg = [0, 0, 0]
@@ -588,13 +589,14 @@ def alg_bytes_per_launch(precision, wl):
     return forces, fused, advance
 
 
-def flagged_nodes(wl, xy):
-    """Nodes of the 32-node force tiles that the spreading of markers at xy
-    (N, 2) flags: the tiles holding a node of some marker's 3 x 3 stencil
-    (origin floor(x + 1/2), rows outside the walls dropped), as the force
-    kernel flags them."""
+def flagged_nodes(wl, xy, width=32):
+    """Nodes of the aligned groups of `width` nodes of one row that hold a node
+    of some marker's 3 x 3 stencil (origin floor(x + 1/2), rows outside the
+    walls dropped).  The force kernel flags the stencils' nodes one by one (a
+    bit per node); the fused kernels take a thread's group of VEC or NPT
+    nodes with the general collision as soon as one of them is flagged."""
     import numpy as np
-    tx = (wl.nx + 31) // 32
+    tx = (wl.nx + width - 1) // width
     i0 = np.floor(xy[:, 0] + 0.5).astype(np.int64)
     j0 = np.floor(xy[:, 1] + 0.5).astype(np.int64)
     tiles = set()
@@ -604,17 +606,17 @@ def flagged_nodes(wl, xy):
         jj = jj % wl.ny
         for dx in (-1, 0, 1):
             ii = (i0 + dx) % wl.nx
-            tiles.update((jj[ok] * tx + ii[ok] // 32).tolist())
-    # the last tile of a row is short when NX is not a multiple of 32
-    last = wl.nx - 32 * (tx - 1)
-    return sum(last if t % tx == tx - 1 else 32 for t in tiles)
+            tiles.update((jj[ok] * tx + ii[ok] // width).tolist())
+    # the last group of a row is short when NX is not a multiple of the width
+    last = wl.nx - width * (tx - 1)
+    return sum(last if t % tx == tx - 1 else width for t in tiles)
 
 
 def ib_bytes_per_flagged_node(precision):
-    """Fused-kernel bytes of the IB coupling per node of a flagged force tile:
-    the fixed-point force read (16), the velocity written for the
+    """Fused-kernel bytes of the IB coupling per node of a thread's flagged
+    group: the fixed-point force read (16), the velocity written for the
     interpolation (2 values of the compute type) and the other parity's force
-    cleared (16; its tiles are the previous step's, about as many)."""
+    cleared (16; its nodes are the previous step's, about as many)."""
     cs = 8 if precision == "f64" else 4
     return 16 + 2 * cs + 16
 

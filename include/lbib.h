@@ -252,7 +252,7 @@ lbib_status lbib_diagnostics(lbib_ctx* ctx, double* mass, double* areas);
 /* ---------------------------------------------------------------- ensembles
  * A batch of independent simulations (e.g. a sweep over release positions,
  * capillary numbers and bond strengths on channels of different lengths)
- * advanced together, one CUDA graph launch per chunk of 16 steps.  The paper
+ * advanced together, one CUDA graph launch per chunk of 16 steps or a single step.  The paper
  * runs its cases one by one; this is a throughput form only: every member
  * computes exactly what it computes alone with the same tiling (bitwise).
  * Two forms, chosen at creation:
@@ -576,7 +576,7 @@ lbib_status lbib_profile_kernels(lbib_ctx* ctx, int32_t reps, double* ms_per_lau
 lbib_status lbib_profile_hydro(lbib_ctx* ctx, int32_t reps, double* ms_per_launch);
 
 /* Number of kernels one time step launches (for launch accounting; with
- * membranes, every captured sequence of 1 or 16 steps ends with one small
+ * membranes, every captured sequence of 1, 2, 4, .. 32 steps ends with one small
  * launch more, which settles the last step's bonds). */
 int32_t lbib_kernels_per_step(const lbib_ctx* ctx);
 

@@ -109,29 +109,42 @@ bool valid_stream(lbib_precision p, int npt, int nx) {
 }
 
 void default_tiling(const lbib_ctx* c, int* vec, int* ty) {
-    // lattices whose two population buffers exceed L2 (129 MB) stream through
-    // the persistent bulk-copy form, which keeps enough bytes in flight for DRAM
-    // (FP64 stays on row tiles: it is bound by the FP64 pipe, not by DRAM)
+    // Row tiles, or the persistent bulk-copy form.  Since the row tiles' loads
+    // run beside the force kernel and their flags are single bits, FP32 keeps
+    // enough bytes in flight with them at any size (us per step, row tiles 4,2 /
+    // persistent 2,0: lattices without markers 3000 x 1000 33.4 / 37.5, 8192 x
+    // 2048 173.6 / 213.0, 520 x 5000 31.2 / 56.1; with markers 8192 x 1024 101.5 /
+    // 106.0).  With the two population buffers a little above L2 (129 MB) the
+    // two come within 2 % with markers (2048 x 1024 33.95 / 34.2), and the
+    // persistent form stays there, and for lattices taller than two rows a
+    // block can cover.
+    // 16-bit storage moves half the bytes per instruction and needs the
+    // persistent form's bulk copies beyond L2 (4096 x 2048 52 us at 4,0, 79-82
+    // with row tiles) and from 2^21 nodes on (2048 x 1400 18.8 / 26.1; below,
+    // 2000 x 667 with markers 20.3 / 19.3, 1536 x 1200 16.0 / 13.8), given rows
+    // that fill its segments of 1024 nodes to 70 % (1032 x 2500 at 4,0 29.3, at
+    // 2,0 26.2).  (FP64 stays on row tiles: it is bound by the FP64 pipe.)
     const double two_buffers = 2.0 * 9.0 * (double)c->pop_elem * c->nx * c->ny;
-    const int npt = c->prec == LBIB_F32 ? 2 : 4;
-    if (c->prec != LBIB_F64 && two_buffers > 128e6 && valid_stream(c->prec, npt, c->nx)) {
-        *vec = npt;
-        *ty = 0;
-        return;
-    }
     const long long nodes = (long long)c->nx * c->ny;
-    // 16-bit storage from a million nodes on: the row tiles' occupancy is capped
-    // by registers and they wait on their loads, while the persistent form's
-    // bulk copies keep the bytes in flight (512-node segments for L2-sized lattices)
-    const bool half = c->prec == LBIB_F32_STORE_F16 || c->prec == LBIB_F32_STORE_BF16;
-    if (half && nodes >= (1LL << 20) && valid_stream(c->prec, 2, c->nx)) {
-        *vec = 2;
-        *ty = 0;
-        return;
+    if (c->prec == LBIB_F32) {
+        if (two_buffers > 128e6 && (two_buffers < 160e6 || c->ny > 2 * kMaxGridY) && valid_stream(c->prec, 2, c->nx)) {
+            *vec = 2;
+            *ty = 0;
+            return;
+        }
+    } else if (c->prec != LBIB_F64) {
+        const int segs = (c->nx + 1023) / 1024;
+        const bool full_rows = 10LL * c->nx >= 7LL * 1024 * segs;
+        const int npt = two_buffers > 128e6 || full_rows ? 4 : 2;
+        if (nodes >= (1LL << 21) && valid_stream(c->prec, npt, c->nx)) {
+            *vec = npt;
+            *ty = 0;
+            return;
+        }
     }
     int v = c->prec == LBIB_F64 ? 2 : 4;
     while (v > 1 && !valid_vec(c->prec, v, c->nx)) v /= 2;
-    const long long N = (long long)c->nx * c->ny;
+    const long long N = nodes;
     // small lattices: fewer nodes per thread so that every SM has warps to switch between
     while (v > 1 && N / v < 152LL * 1024 && valid_vec(c->prec, v / 2, c->nx)) v /= 2;
     const long long tiles_x = (c->nx + 32LL * v - 1) / (32LL * v);
@@ -1594,7 +1607,7 @@ extern "C" lbib_status lbib_ensemble_create(lbib_ctx* const* members, int32_t n,
         if (c->device != dev || c->poisoned) return LBIB_E_INVALID;
         lbib_status st = finalize(c);
         if (st == LBIB_OK && !c->no_g_prefetch) {
-            // the members' row tiles read the force field only in flagged tiles
+            // the members' row tiles read the force field only at flagged nodes
             if (cudaStreamSynchronize(c->stream) != cudaSuccess) return LBIB_E_CUDA;
             c->no_g_prefetch = true;
             drop_graphs(c);

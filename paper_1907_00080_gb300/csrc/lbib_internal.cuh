@@ -100,7 +100,7 @@ constexpr double kFixInv = 1.0 / 4503599627370496.0;      // 2^-52
 struct LbArgs {
     const void* src;       // post-collision deviations of step n-1
     void* dst;             // post-collision deviations of step n
-    void* ux;              // u field (compute type), written in flagged tiles
+    void* ux;              // u field (compute type), written where a thread's nodes hold a flagged one
     void* uy;
     double* rho_out;       // fields mode: rho, ux, uy as doubles (may be null)
     double* ux_out;
