@@ -248,15 +248,15 @@ __global__ void __launch_bounds__(512) k_lb_step(const LbArgs a) {
 // search for the member, no division for the tile, and the arguments are read
 // from the launch parameters where they are used.  These steps came before a
 // block's first load and were a third of its life: 64-member ensemble, FP32
-// tiles 4,1: 202.6 -> 177.2 us per step, BF16 4,2: 208.4 -> 150.5, ten members
+// tiles 4,1: 202.6 -> 177.2 us per step, BF16 4,2: 208.4 -> 151, ten members
 // BF16 4,1: 32.8 -> 27.7.
 template <typename S, int VEC, bool WALLS>
 __global__ void __launch_bounds__(512) k_lb_grid_batch(const __grid_constant__ LbBatch b) {
     const int m = blockIdx.z;
-    const LbArgs& a = b.a[m];
-    // (beyond the member's own grid)
-    if ((int)blockIdx.x >= b.tiles_x[m] || (int)(blockIdx.y * blockDim.y) >= a.ny) return;
-    lb_tile<S, VEC, WALLS, 1>(a, blockIdx.x, blockIdx.y);
+    // (beyond the member's own grid; the unsigned comparison leaves FP32 VEC 4 at 79
+    // registers, a signed one at 85 and two warps per SM less: 187.9 us)
+    if (blockIdx.x >= (unsigned)b.tiles_x[m] || (int)(blockIdx.y * blockDim.y) >= b.a[m].ny) return;
+    lb_tile<S, VEC, WALLS, 1>(b.a[m], blockIdx.x, blockIdx.y);
 }
 
 // The same as one list of the members' tiles, row by row, for members of very
