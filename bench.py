@@ -440,7 +440,7 @@ def lbib_main(args):
 KERNEL_NAMES = ("k_forces (forces, IB weights, spreading)", "k_lb_step / k_lb_stream (fused collide-stream)",
                 "k_advance (interpolation, advance, bonds)")
 ENSEMBLE_KERNEL_NAMES = ("k_forces_batch (forces, IB weights, spreading; all members)",
-                         "k_lb_stream_ws_batch / k_lb_step_batch (fused collide-stream; all members)",
+                         "k_lb_grid_batch / k_lb_stream_ws_batch (fused collide-stream; all members)",
                          "k_advance_batch (interpolation, advance, bonds; all members)")
 
 
