@@ -932,6 +932,18 @@ static lbib_status build_graphs(lbib_ctx* c) {
     return LBIB_OK;
 }
 
+// one time step by the context's captured single step.  (Joining an ensemble
+// drops the captured steps: whoever launches them has them built.)
+static lbib_status launch_single_step(lbib_ctx* c) {
+    const lbib_status st = build_graph(c, c->cur, 0);
+    if (st != LBIB_OK) return st;
+    CK(cudaGraphLaunch(c->graph[c->cur][0], c->stream));
+    c->cur = 1 - c->cur;
+    c->steps += 1;
+    c->fields_valid = true;
+    return LBIB_OK;
+}
+
 // Sequences of 2, 4, .. 32 steps are captured when a call first needs them: a
 // call of n steps is a few launches for any n (7 steps were seven launches of
 // one step each, with a boundary of 2 us between them), and a first call
@@ -1922,10 +1934,8 @@ extern "C" lbib_status lbib_tangent_step(lbib_tangent* t, int64_t n) {
         a.step = c->steps;
         CK(launch_tangent_step(a, c->stream));
         // the primal step (its captured one-step graph) follows on the same stream
-        CK(cudaGraphLaunch(c->graph[c->cur][0], c->stream));
-        c->cur = 1 - c->cur;
-        c->steps += 1;
-        c->fields_valid = true;
+        const lbib_status st = launch_single_step(c);
+        if (st != LBIB_OK) return st;
         t->cf = 1 - t->cf;
         const int op = t->ip;
         t->ip = t->ix;
@@ -2232,9 +2242,8 @@ extern "C" lbib_status lbib_adjoint_reverse(lbib_adjoint* a) {
                 if (c->nlig) CK(d2d(a->tape_bond + (size_t)k * nl, c->bond[c->cur], 4 * (size_t)c->nlig));
             }
             const int src = c->cur;
-            CK(cudaGraphLaunch(c->graph[c->cur][0], c->stream));
-            c->cur = 1 - c->cur;
-            c->steps += 1;
+            const lbib_status st = launch_single_step(c);
+            if (st != LBIB_OK) return st;
             if (nvr && f64) {
                 // what the step computed, in one launch
                 CopyList l{};
@@ -2561,11 +2570,8 @@ extern "C" lbib_status lbib_slabs_step(lbib_slabs* g, int64_t n) {
         if (c->poisoned) return slabs_fail(g, LBIB_E_STATE, "a slab is poisoned by an earlier device-side failure");
     for (int64_t k = 0; k < n; ++k) {
         for (lbib_ctx* c : g->s) {
-            const cudaError_t e = cudaGraphLaunch(c->graph[c->cur][0], c->stream);
-            if (e != cudaSuccess) return slabs_fail(g, LBIB_E_CUDA, std::string("slab step: ") + cudaGetErrorString(e));
-            c->cur = 1 - c->cur;
-            c->steps += 1;
-            c->fields_valid = true;
+            const lbib_status st = launch_single_step(c);
+            if (st != LBIB_OK) return slabs_fail(g, st, "slab step: " + c->err);
         }
         const cudaError_t e = slabs_exchange(g);
         if (e != cudaSuccess) return slabs_fail(g, LBIB_E_CUDA, std::string("halo exchange: ") + cudaGetErrorString(e));
