@@ -912,12 +912,14 @@ static lbib_status build_graph(lbib_ctx* c, int start, int k) {
         if (g) cudaGraphDestroy(g);
         return cuda_fail(c, le != cudaSuccess ? le : e, "capture step");
     }
-    e = cudaGraphInstantiate(&c->graph[start][k], g, 0);
-    c->graph_tmpl[start][k] = g;  // an ensemble embeds it as a child graph
+    cudaGraphExec_t exec = nullptr;
+    e = cudaGraphInstantiate(&exec, g, 0);
     if (e != cudaSuccess) {
-        c->graph[start][k] = nullptr;
+        cudaGraphDestroy(g);
         return cuda_fail(c, e, "instantiate step graph");
     }
+    c->graph[start][k] = exec;
+    c->graph_tmpl[start][k] = g;  // an ensemble embeds it as a child graph
     return LBIB_OK;
 }
 
@@ -947,30 +949,42 @@ static lbib_status launch_single_step(lbib_ctx* c) {
 // Sequences of 2, 4, .. 32 steps are captured when a call first needs them: a
 // call of n steps is a few launches for any n (7 steps were seven launches of
 // one step each, with a boundary of 2 us between them), and a first call
-// captures little more than it runs.  Within a capture of the caller's own
-// nothing is captured anew: the sequences there are serve any n.
+// captures little more than it runs.  All of a call's sequences are captured
+// before its first launch, so that a call which cannot capture one has enqueued
+// nothing, and the state follows every launch.  (Within a capture of the
+// caller's own a launch of a graph is an error of the runtime's: refused before
+// anything is captured.)
 extern "C" lbib_status lbib_step(lbib_ctx* c, int64_t n) {
     if (!c || n < 0) return LBIB_E_INVALID;
     if (c->poisoned) return fail(c, LBIB_E_STATE, "context poisoned by an earlier device-side failure");
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(c->stream, &cs));
+    if (n > 0 && cs != cudaStreamCaptureStatusNone)
+        return cuda_fail(c, cudaErrorStreamCaptureUnsupported, "time steps within a stream capture");
     lbib_status st = finalize(c);
     if (st != LBIB_OK) return st;
     st = build_graphs(c);
     if (st != LBIB_OK) return st;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    CK(cudaStreamIsCapturing(c->stream, &cs));
-    int64_t left = n;
-    while (left > 0) {
+    // the longest sequences first; all start from the buffer of now, since only a
+    // single step, the last one, changes the buffer roles
+    auto longest = [](int64_t left) {
         int k = 0;
         while (k + 1 < lbib_ctx::kGraphs && left >= (int64_t)2 << k) ++k;
-        if (cs != cudaStreamCaptureStatusNone)
-            while (k > 0 && !c->graph[c->cur][k]) --k;
+        return k;
+    };
+    for (int64_t left = n; left > 0;) {
+        const int k = longest(left);
         if ((st = build_graph(c, c->cur, k)) != LBIB_OK) return st;
+        left &= ((int64_t)1 << k) - 1;
+    }
+    for (int64_t left = n; left > 0;) {
+        const int k = longest(left);
         CK(cudaGraphLaunch(c->graph[c->cur][k], c->stream));
-        if (k == 0) c->cur = 1 - c->cur;  // an even number of steps leaves the buffer roles
+        if (k == 0) c->cur = 1 - c->cur;
+        c->steps += (int64_t)1 << k;
+        c->fields_valid = true;
         left -= (int64_t)1 << k;
     }
-    c->steps += n;
-    if (n > 0) c->fields_valid = true;
     return LBIB_OK;
 }
 
