@@ -555,7 +555,8 @@ lbib_status lbib_get_tiling(const lbib_ctx* ctx, int32_t* vec, int32_t* ty);
  * the context's stream (ping-pong between the two population buffers, with the
  * IB force of the last completed step frozen), bracketed by CUDA events, and
  * return the mean duration of one launch in milliseconds.  This advances the
- * populations without the Lagrangian part, so use it on a scratch context.
+ * populations without the Lagrangian part (markers, bonds and step count stay),
+ * so use it on a scratch context.
  * Errors: LBIB_E_STATE before the first step. */
 lbib_status lbib_profile_fused(lbib_ctx* ctx, int32_t reps, double* ms_per_launch);
 

@@ -1266,6 +1266,16 @@ extern "C" lbib_status lbib_membrane_observables(lbib_ctx* c, double* out) {
     return LBIB_OK;
 }
 
+// Profiling launches swap the population buffers each time.  Bonds, their
+// decisions, the step counter and the force fields go by the buffer that a step
+// starts from: after an odd number of launches the populations go back into it.
+static cudaError_t back_in_buffer(lbib_ctx* c, int buf) {
+    if (c->cur == buf) return cudaSuccess;
+    c->cur = buf;
+    return cudaMemcpyAsync(c->f[buf], c->f[1 - buf], 9 * (size_t)c->nx * c->ny * c->pop_elem,
+                           cudaMemcpyDeviceToDevice, c->stream);
+}
+
 extern "C" lbib_status lbib_profile_fused(lbib_ctx* c, int32_t reps, double* ms_per_launch) {
     if (!c || reps < 1 || !ms_per_launch) return LBIB_E_INVALID;
     if (!c->finalized || c->steps == 0) return fail(c, LBIB_E_STATE, "profile after at least one step");
@@ -1273,7 +1283,7 @@ extern "C" lbib_status lbib_profile_fused(lbib_ctx* c, int32_t reps, double* ms_
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     // the force field of the last completed step stays fixed for every launch
-    const int gpar = 1 - c->cur;
+    const int start = c->cur, gpar = 1 - start;
     LbArgs l = lb_args(c, c->cur, gpar, 0);
     CK(cudaEventRecord(e0, c->stream));
     for (int r = 0; r < reps; ++r) {
@@ -1285,6 +1295,7 @@ extern "C" lbib_status lbib_profile_fused(lbib_ctx* c, int32_t reps, double* ms_
         c->cur = 1 - c->cur;
     }
     CK(cudaEventRecord(e1, c->stream));
+    CK(back_in_buffer(c, start));
     CK(cudaEventSynchronize(e1));
     float ms = 0.f;
     CK(cudaEventElapsedTime(&ms, e0, e1));
@@ -1325,7 +1336,7 @@ extern "C" lbib_status lbib_profile_kernels(lbib_ctx* c, int32_t reps, double* m
     for (int r = 0; r < reps && has_ib; ++r) CK(launch_forces(c->prec, a, false, c->stream));
     CK(cudaEventRecord(ev[1], c->stream));
     // fused collide-stream, ping-pong between the buffers
-    const int gpar = 1 - c->cur;
+    const int start = c->cur, gpar = 1 - start;
     LbArgs l = lb_args(c, c->cur, gpar, 0);
     CK(cudaEventRecord(ev[2], c->stream));
     for (int r = 0; r < reps; ++r) {
@@ -1335,6 +1346,7 @@ extern "C" lbib_status lbib_profile_kernels(lbib_ctx* c, int32_t reps, double* m
         c->cur = 1 - c->cur;
     }
     CK(cudaEventRecord(ev[3], c->stream));
+    CK(back_in_buffer(c, start));
     // interpolation + advance + bond kinetics
     CK(cudaEventRecord(ev[4], c->stream));
     for (int r = 0; r < reps && has_ib; ++r) CK(launch_advance(c->prec, a, c->stream));
