@@ -678,7 +678,7 @@ __global__ void __launch_bounds__(256) k_settle(const MarkerArgs a) {
     dep_wait();
     settle_bonds(a);
 }
-__global__ void __launch_bounds__(256) k_settle_batch(const MarkerArgs* __restrict__ args) {
+__global__ void __launch_bounds__(256) k_settle_batch(const MarkerArgs* args) {
     __shared__ MarkerArgs s_a;
     stage_args(&s_a, args + blockIdx.x);
     dep_wait();

@@ -18,7 +18,7 @@ struct alignas(sizeof(S) * VEC) Pack {
 };
 
 template <typename S, int VEC>
-__device__ __forceinline__ void load_pack(const S* __restrict__ row, int x0, bool ok, float inv,
+__device__ __forceinline__ void load_pack(const S* row, int x0, bool ok, float inv,
                                           typename Storage<S>::C (&out)[VEC]) {
     using C = typename Storage<S>::C;
     if (ok) {
@@ -49,7 +49,7 @@ __device__ __forceinline__ void lb_tile(const LbArgs& a, int bx, int by) {
     const int x0 = (bx * 32 + lane) * VEC;
     const bool ok = (y < ny) && (x0 < nx);
     const size_t N = (size_t)nx * ny;
-    const S* __restrict__ src = static_cast<const S*>(a.src);
+    const S* src = static_cast<const S*>(a.src);
     const float inv = a.inv_scale;
 
     // ---- prologue: the pulled rows, as loaded (aligned vectors), and the single

@@ -297,7 +297,7 @@ __device__ __forceinline__ void stage_rows(const LbArgs& A, ItemRef p, uint32_t 
     constexpr int H = Gm::H, W = Gm::W;
     const int nx = A.nx, ny = A.ny;
     const size_t N = (size_t)nx * ny;
-    const S* __restrict__ src = static_cast<const S*>(A.src);
+    const S* src = static_cast<const S*>(A.src);
     const int wlen = min(W, nx - p.x0);
     const unsigned row_bytes = (unsigned)((wlen + 2 * H) * sizeof(S));
     const bool interior = p.x0 >= H && p.x0 + wlen + H <= nx;
