@@ -247,9 +247,8 @@ extern "C" lbib_status lbib_create(const lbib_lattice* lat, double tau, const do
             return LBIB_E_OOM;
         }
     }
-    const size_t u_bytes = (N + c->nx) * c->cmp_elem;  // and a row of zeros (interp_vertex)
-    e = cudaMalloc(&c->ux, u_bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&c->uy, u_bytes);
+    e = cudaMalloc(&c->ux, N * c->cmp_elem);
+    if (e == cudaSuccess) e = cudaMalloc(&c->uy, N * c->cmp_elem);
     c->n_partials = 1024;
     if (e == cudaSuccess) e = cudaMalloc(&c->partials, sizeof(double) * c->n_partials);
     if (e == cudaSuccess) e = cudaMalloc(&c->dscalar, sizeof(double) * 8);
@@ -259,8 +258,8 @@ extern "C" lbib_status lbib_create(const lbib_lattice* lat, double tau, const do
         lbib_destroy(c);
         return LBIB_E_OOM;
     }
-    e = cudaMemsetAsync(c->ux, 0, u_bytes, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->uy, 0, u_bytes, c->stream);
+    e = cudaMemsetAsync(c->ux, 0, N * c->cmp_elem, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->uy, 0, N * c->cmp_elem, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_step, 0, 2 * sizeof(long long), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = init_populations(c);
@@ -743,7 +742,6 @@ static lbib_status finalize(lbib_ctx* c) {
     a.tiles_x = c->tiles_x;
     a.status = c->d_status;
     a.f.nx = (float)c->nx; a.f.ny = (float)c->ny; a.f.inv_nx = (float)a.inv_nx; a.f.inv_ny = (float)a.inv_ny;
-    a.f.wrap_ny = a.walls ? 0.f : (float)c->ny;
     a.f.sigma = (float)a.sigma; a.f.y_eq = (float)a.y_eq; a.f.inv_y_eq = (float)a.inv_y_eq;
     a.f.d_rep = (float)a.d_rep; a.f.d_cut = (float)a.d_cut; a.f.d_break = (float)a.d_break;
     a.f.kf_dt = (float)a.kf_dt; a.f.kr0_dt = (float)a.kr0_dt; a.f.beta_f = (float)a.beta_f;
@@ -1543,10 +1541,11 @@ static lbib_status ensemble_batch_tables(lbib_ensemble* e, int ngroups) {
 
 // one time step of every member of group g in the batched form, at phase p
 // (first: of a captured sequence, see enqueue_step)
-static cudaError_t ensemble_batch_step(const lbib_ensemble* e, int g, int p, cudaStream_t s, bool first, bool last) {
+static cudaError_t ensemble_batch_step(lbib_ensemble* e, int g, int p, cudaStream_t s, bool first, bool last) {
     const lbib_ctx* c0 = e->m[0];
     const bool walls = c0->walls != LBIB_WALLS_NONE;
-    cudaError_t r = launch_forces_batch(c0->prec, e->fbb[p][g], !first, s, !first);
+    e->fbb[p][g].settle = first ? 0 : 1;
+    cudaError_t r = launch_forces_batch(c0->prec, e->fbb[p][g], s, !first);
     if (r == cudaSuccess)
         r = c0->ty > 0 ? launch_lb_batch(c0->prec, c0->vec, c0->ty, walls, e->lbb[p][g], s, true)
                        : launch_lb_stream_batch(c0->prec, c0->vec, walls, e->stream_grid, e->lbb[p][g], s, true);

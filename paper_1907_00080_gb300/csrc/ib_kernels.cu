@@ -222,8 +222,7 @@ __device__ __forceinline__ void shape_functions(const MarkerArgs& a, E xv, E yv,
 // Eq. repFor screening by one warp, in two stages: groups (32 vertices) of
 // other membranes whose box comes within d_rep of this chunk's box (the union
 // of its one or two groups' boxes), and of those the segments.  Hits join the
-// block's candidate list in any order: the repulsion sums are over integers, and
-// a pair rounds the same whether its segment is staged, listed or just walked.
+// block's candidate list in any order (order_candidates).
 // The groups cut the boxes that every block reads to a quarter (64 instead of
 // 228 on the 640 x 160 capillary, one pass of the loop below).
 struct Candidates {
@@ -286,6 +285,32 @@ __device__ __forceinline__ void screen_segments(const MarkerArgs& a, int m, int 
     }
 }
 
+// Candidates beyond the staging space, all threads of the block: the list in
+// ascending order, its first kStageSeg staged.  A staged pair and a listed one
+// round differently (offsets from the segment's anchor, or a difference of two
+// positions), so which segments are staged must not depend on the order in
+// which the screening's lanes found them; up to kStageSeg hits are all staged
+// and more than kMaxCand all walked, in any order.  (A thread ranks its hit
+// against the others; the blocks that come here have 48 segments and more
+// within range, and no other block pays for it.)
+__device__ __forceinline__ void order_candidates(const MarkerArgs& a, int ncand, const Candidates& s_c) {
+    static_assert(kMaxCand <= kForceThreads, "one candidate per thread");
+    const int tid = threadIdx.x;
+    const int sg = s_c.seg[tid < ncand ? tid : 0];
+    int rank = 0;
+    for (int q = 0; q < ncand; ++q) rank += s_c.seg[q] < sg ? 1 : 0;
+    __syncthreads();
+    if (tid < ncand) {
+        s_c.seg[rank] = sg;
+        if (rank < kStageSeg) {
+            s_c.v0[rank] = a.seg_v0[sg];
+            s_c.nv[rank] = a.seg_n[sg];
+            s_c.box[rank] = a.seg_box[sg];
+        }
+    }
+    __syncthreads();
+}
+
 // One block per work unit (a chunk of up to kChunkV consecutive vertices of one
 // membrane).  The kernel is a chain of dependent loads and FP32 divisions and
 // square roots, so the parts of a vertex's force go to different warps and
@@ -342,6 +367,7 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
     __shared__ __align__(16) C s_cox[kStageSeg][kSegV], s_coy[kStageSeg][kSegV];
     __shared__ int s_cn[kStageSeg], s_cv0[kStageSeg];
     const Rest<C>* rest = static_cast<const Rest<C>*>(a.rest);
+    const Candidates cand{&s_ncand, s_cand, s_cv0, s_cn, s_cbox};
     // (with dynamic particles the predecessor is the hydrodynamic kernel, which
     // started after the positions were complete: its results are waited for
     // where they are used)
@@ -441,8 +467,7 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
         if (lane == 0) s_ncand = 0;
         __syncwarp();
         if (!a.has_dyn) dep_wait();
-        if (a.nmem > 1)
-            screen_segments(a, m, own0, kn, lane, Candidates{&s_ncand, s_cand, s_cv0, s_cn, s_cbox});
+        if (a.nmem > 1) screen_segments(a, m, own0, kn, lane, cand);
     } else if (wid == 5) {
         if (!halo_here && lane < 2) {
             // the halo vertices k0 - 1 (slot 0) and k0 + kn (slot kn + 1)
@@ -487,6 +512,7 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
     {
         const int ncand = s_ncand;
         const bool all_segs = ncand > kMaxCand;  // list overflow: screen every segment
+        if (ncand > kStageSeg && !all_segs) order_candidates(a, ncand, cand);
         if (ncand > 0) {
             // Eq. repFor against vertices of other membranes closer than d_rep, over
             // (candidate segment, vertex) pairs; the magnitudes of each vertex are
@@ -521,7 +547,6 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
             const E xv = s_x[j], yv = s_y[j];
             const float hx = float(ehi(xv)), hy = float(ehi(yv));
             const float xvw = hx - a.f.nx * floorf(hx * a.f.inv_nx);
-            const float yvw = hy - a.f.wrap_ny * floorf(hy * a.f.inv_ny);
             bool bad = false;
             for (int ci = tid / kChunkV; ci < nscan && j < kn; ci += kForceThreads / kChunkV) {
                 const bool staged = !all_segs && ci < kStageSeg;
@@ -529,7 +554,7 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
                 if (all_segs && a.seg_mem[sg] == m) continue;
                 const float4 bx = staged ? s_cbox[ci] : a.seg_box[sg];
                 const float ddx = wrap_half(xvw - bx.x, a.f.nx);
-                float ddy = yvw - bx.y;
+                float ddy = hy - bx.y;
                 if (!a.walls) ddy = wrap_half(ddy, a.f.ny);
                 if (fabsf(ddx) > bx.z + reach || fabsf(ddy) > bx.w + reach) continue;
                 C mags = C(0);
@@ -552,17 +577,13 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
                         if (d < drep) mags += c_rep * sqrt(C(1) / (d * d * d * d * d));
                     }
                 } else {
-                    // (by the offsets from the anchor too)
                     const int nb = a.seg_n[sg], b0 = a.seg_v0[sg];
-                    E xa, ya;
-                    load_pos<C>(a, b0, xa, ya);
-                    const C dxa = etoc(ewrap(esub(xv, xa), par<C>(a.nx, a.f.nx), par<C>(a.inv_nx, a.f.inv_nx)));
-                    C dya = etoc(esub(yv, ya));
-                    if (!a.walls) dya = etoc(ewrap(esub(yv, ya), par<C>(a.ny, a.f.ny), par<C>(a.inv_ny, a.f.inv_ny)));
                     for (int g = 0; g < nb; ++g) {
                         E xb, yb;
                         load_pos<C>(a, b0 + g, xb, yb);
-                        const C dx = dxa - etoc(esub(xb, xa)), dy = dya - etoc(esub(yb, ya));
+                        const C dx = etoc(ewrap(esub(xv, xb), par<C>(a.nx, a.f.nx), par<C>(a.inv_nx, a.f.inv_nx)));
+                        C dy = etoc(esub(yv, yb));
+                        if (!a.walls) dy = etoc(ewrap(esub(yv, yb), par<C>(a.ny, a.f.ny), par<C>(a.inv_ny, a.f.inv_ny)));
                         const C d = sqrt(dx * dx + dy * dy);
                         if (d < drep) mags += c_rep * sqrt(C(1) / (d * d * d * d * d));
                     }
@@ -641,18 +662,14 @@ __global__ void __launch_bounds__(kForceThreads) k_forces(const MarkerArgs a, co
 // Batched form: the force units of up to kBatchMax contexts (ensemble
 // members) in one launch, one block per (member, unit).  The member's
 // arguments are staged in shared memory.
-// (FP32: four blocks per SM, the batch's thousands of blocks are limited by how
-// many fit, not by one block's latency.  FP64: three.  At four the 64 registers
-// spill 268 bytes of stores and 200 of loads: 64 members 94.4 us against 89.8,
-// 10 members 25.5 against 24.8; 32 members 54.6 against 58.7, their whole step
-// 659.4 against 658.2.)
+// (four blocks per SM: the batch's thousands of blocks are limited by how many
+// fit, not by one block's latency)
 template <typename C>
-__global__ void __launch_bounds__(kForceThreads, sizeof(C) == 8 ? 3 : 4)
-    k_forces_batch(const __grid_constant__ MarkerBatch b, const bool settle) {
+__global__ void __launch_bounds__(kForceThreads, 4) k_forces_batch(const __grid_constant__ MarkerBatch b) {
     __shared__ MarkerArgs s_a;
     const int m = marker_member(b, blockIdx.x);
     stage_args(&s_a, b.args + m);
-    forces_unit<C>(s_a, blockIdx.x - b.off[m], settle);
+    forces_unit<C>(s_a, blockIdx.x - b.off[m], b.settle != 0);
 }
 
 // the end of a launch sequence: the last step's bond decisions, one block per
@@ -737,12 +754,12 @@ cudaError_t launch_forces(lbib_precision prec, const MarkerArgs& a, bool settle,
                          chained, a, settle);
 }
 
-cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, bool settle, cudaStream_t s, bool chained) {
+cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, cudaStream_t s, bool chained) {
     if (b.n < 1 || b.n > kBatchMax) return cudaErrorInvalidValue;
     const int nunits = b.off[b.n];
     if (nunits <= 0) return cudaSuccess;
     return launch_kernel(is_f64(prec) ? k_forces_batch<double> : k_forces_batch<float>, nunits, kForceThreads, 0, s,
-                         chained, b, settle);
+                         chained, b);
 }
 
 cudaError_t launch_settle(const MarkerArgs& a, cudaStream_t s) {

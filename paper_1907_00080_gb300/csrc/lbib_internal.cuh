@@ -4,9 +4,8 @@
 //   populations  two buffers A/B, [9][NY][NX] of the storage type, x fastest;
 //                each holds the post-collision deviations d*_i = f*_i - w_i of
 //                one step (pull scheme: the fused kernel streams while reading)
-//   u field      ux, uy [NY + 1][NX] of the compute type, written by the fused
-//                kernel only at nodes that IB stencils touch; the row after the
-//                lattice's last stays zero
+//   u field      ux, uy [NY][NX] of the compute type, written by the fused
+//                kernel only at nodes that IB stencils touch
 //   markers      X^n, X^{n-1} as interleaved (x, y) doubles; F^n, U^n, the nine
 //                shape-function weights and the stencil origin per vertex
 //   IB force     two fixed-point (int64 x 2) per-node fields alternating with the
@@ -158,7 +157,7 @@ struct MarkerArgs {
     const int* seg_mem;       // [nseg]
     const int* seg_v0;        // [nseg] first global vertex
     const int* seg_n;         // [nseg]
-    float4* seg_box;          // [nseg] centre x wrapped to [0,nx), centre y (without walls to [0,ny)), half extents
+    float4* seg_box;          // [nseg] centre x wrapped to [0,nx), centre y, half extents
     // groups of kGroupV vertices (four segments), boxes a little wide: the
     // first stage of the screening
     int ngroup;
@@ -219,7 +218,6 @@ struct MarkerArgs {
     // FP32 copies of the scalar parameters (no double->float conversion in the kernels)
     struct {
         float nx, ny, inv_nx, inv_ny, sigma, y_eq, inv_y_eq, d_rep, d_cut, d_break;
-        float wrap_ny;            // the period in y of the screening boxes: ny without walls, 0 with them
         float kf_dt, kr0_dt, beta_f, beta_r, inv_rc_w, inv_rc_h, rc_y0;
         // no receptor is within reach of a ligand at y < y_reach[0], y_reach[1] < y < y_reach[2] (the largest
         // gap between receptor heights, e.g. the channel between its walls) or y > y_reach[3]
@@ -297,14 +295,14 @@ __device__ __forceinline__ int batch_member(const int* off, int n, int b) {
     }
     return lo;
 }
-// fused kernel: the members' arguments themselves are parameters
+// fused kernel: the members' arguments themselves are parameters (192 B each)
 struct LbBatch {
     int n;
     int off[kBatchMax + 1];     // row tiles: first block of each member; persistent form: first segment
     int tiles_x[kBatchMax];     // row tiles: tiles per row; persistent form: segments per row
     LbArgs a[kBatchMax];
 };
-// marker kernels: the members' arguments stay in global memory
+// marker kernels: the members' arguments (744 B each) stay in global memory
 // block -> member for the first kBlockTable blocks of a launch (one parameter
 // load where a search over off[] would take several dependent ones)
 constexpr int kBlockTable = 8192;
@@ -313,6 +311,7 @@ struct MarkerBatch {
     int n;
     int off[kBatchMax + 1];     // first block of each member's units
     const MarkerArgs* args;     // [n]
+    int settle;                 // force kernel: settle the previous step's bond decisions
     unsigned char member[kBlockTable];  // member of block b < min(off[n], kBlockTable)
 };
 __device__ __forceinline__ int marker_member(const MarkerBatch& b, int blk) {
@@ -403,8 +402,7 @@ cudaError_t launch_settle_batch(const MarkerArgs* args, int n, cudaStream_t s);
 cudaError_t launch_advance(lbib_precision prec, const MarkerArgs& a, cudaStream_t s, bool chained = false);
 // batched marker kernels of up to kBatchMax contexts (b.off[b.n] blocks); the
 // advance blocks have `threads` threads (the widest member's)
-cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, bool settle, cudaStream_t s,
-                                bool chained = false);
+cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, cudaStream_t s, bool chained = false);
 cudaError_t launch_advance_batch(lbib_precision prec, bool dyn, const MarkerBatch& b, int threads, cudaStream_t s,
                                  bool chained = false);
 cudaError_t launch_seg_boxes(lbib_precision prec, const MarkerArgs& a, cudaStream_t s);

@@ -261,8 +261,7 @@ __device__ __forceinline__ void block_sum_c(C (&v)[N], C (*red)[8]) {
 // Boxes of the segments and of the screening group that a warp's positions
 // form: lane l holds vertex l of the group; lanes g, g + 1, .. of a segment past
 // its end hold a copy of its first vertex.  FP32 offsets from the segment's
-// first vertex; centre x wrapped into [0, nx), and without walls centre y into
-// [0, ny) (rings may lie several periods apart).  sg: this lane's segment (-1:
+// first vertex; centre x wrapped into [0, nx).  sg: this lane's segment (-1:
 // none), gr: the warp's group (-1: none).  The group's box is widened by 1e-3
 // (its own roundings stay below 1e-3 of a lattice unit).  All 32 lanes call it.
 template <typename C>
@@ -283,11 +282,10 @@ __device__ __forceinline__ void seg_box_regs(const MarkerArgs& a, int sg, int gr
         lo_y = fminf(lo_y, __shfl_xor_sync(kFull, lo_y, o));
         hi_y = fmaxf(hi_y, __shfl_xor_sync(kFull, hi_y, o));
     }
-    auto wrapped_y = [&](float cy) { return cy - a.f.wrap_ny * floorf(cy * a.f.inv_ny); };
     const float Lx = a.f.nx;
     if (sg >= 0 && lane == g0) {
         const float cx = float(ehi(ax)) + 0.5f * (lo_x + hi_x);
-        a.seg_box[sg] = make_float4(cx - Lx * floorf(cx * a.f.inv_nx), wrapped_y(float(ehi(ay)) + 0.5f * (lo_y + hi_y)),
+        a.seg_box[sg] = make_float4(cx - Lx * floorf(cx * a.f.inv_nx), float(ehi(ay)) + 0.5f * (lo_y + hi_y),
                                     0.5f * (hi_x - lo_x), 0.5f * (hi_y - lo_y));
     }
     shfl_e(wx, x, 0);
@@ -306,7 +304,7 @@ __device__ __forceinline__ void seg_box_regs(const MarkerArgs& a, int sg, int gr
     }
     if (gr >= 0 && lane == 0) {
         const float cx = float(ehi(wx)) + 0.5f * (lo_x + hi_x);
-        a.group_box[gr] = make_float4(cx - Lx * floorf(cx * a.f.inv_nx), wrapped_y(float(ehi(wy)) + 0.5f * (lo_y + hi_y)),
+        a.group_box[gr] = make_float4(cx - Lx * floorf(cx * a.f.inv_nx), float(ehi(wy)) + 0.5f * (lo_y + hi_y),
                                       0.5f * (hi_x - lo_x) + 1e-3f, 0.5f * (hi_y - lo_y) + 1e-3f);
     }
 }
@@ -330,11 +328,9 @@ __device__ __forceinline__ Shape<C> load_shape(const MarkerArgs& a, int v) {
     s.j0 = o.y;
     return s;
 }
-// (every node is read, rows outside the walls at the row of zeros after the
-// field's last: a branch per row made three round trips of one, 3400 cycles of
-// the advance kernel's chain.  The nearest fluid row would not do: for a marker
-// beyond a wall no stencil flagged it, and what an earlier step left there, not
-// finite perhaps, does not vanish by a weight of 0.)
+// (every node is read, rows outside the walls at the nearest row with their
+// weight 0: a branch per row made three round trips of one, 3400 cycles of the
+// advance kernel's chain)
 template <typename C>
 __device__ __forceinline__ void interp_vertex(const MarkerArgs& a, const Shape<C>& s, C& Ux, C& Uy) {
     const C* ux = static_cast<const C*>(a.ux);
@@ -348,7 +344,7 @@ __device__ __forceinline__ void interp_vertex(const MarkerArgs& a, const Shape<C
         i[q] = i[q] < 0 ? i[q] + a.nx : (i[q] >= a.nx ? i[q] - a.nx : i[q]);
         int j = s.j0 + q - 1;
         in[q] = !a.walls || (j >= 0 && j < a.ny);
-        j = a.walls ? (in[q] ? j : a.ny) : (j < 0 ? j + a.ny : (j >= a.ny ? j - a.ny : j));
+        j = a.walls ? min(max(j, 0), a.ny - 1) : (j < 0 ? j + a.ny : (j >= a.ny ? j - a.ny : j));
         row[q] = (size_t)j * a.nx;
     }
     C u[9], v[9];
