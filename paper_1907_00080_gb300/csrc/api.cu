@@ -1541,11 +1541,10 @@ static lbib_status ensemble_batch_tables(lbib_ensemble* e, int ngroups) {
 
 // one time step of every member of group g in the batched form, at phase p
 // (first: of a captured sequence, see enqueue_step)
-static cudaError_t ensemble_batch_step(lbib_ensemble* e, int g, int p, cudaStream_t s, bool first, bool last) {
+static cudaError_t ensemble_batch_step(const lbib_ensemble* e, int g, int p, cudaStream_t s, bool first, bool last) {
     const lbib_ctx* c0 = e->m[0];
     const bool walls = c0->walls != LBIB_WALLS_NONE;
-    e->fbb[p][g].settle = first ? 0 : 1;
-    cudaError_t r = launch_forces_batch(c0->prec, e->fbb[p][g], s, !first);
+    cudaError_t r = launch_forces_batch(c0->prec, e->fbb[p][g], !first, s, !first);
     if (r == cudaSuccess)
         r = c0->ty > 0 ? launch_lb_batch(c0->prec, c0->vec, c0->ty, walls, e->lbb[p][g], s, true)
                        : launch_lb_stream_batch(c0->prec, c0->vec, walls, e->stream_grid, e->lbb[p][g], s, true);
@@ -1785,7 +1784,7 @@ extern "C" lbib_status lbib_ensemble_profile_kernels(lbib_ensemble* e, int32_t r
     for (int k = 0; k < 4; ++k) ECK(cudaEventCreate(&ev[k]));
     ECK(cudaEventRecord(ev[0], e->stream));
     for (int r = 0; r < reps; ++r)
-        for (int g = 0; g < G; ++g) ECK(launch_forces_batch(c0->prec, e->fbb[e->flip][g], e->stream));
+        for (int g = 0; g < G; ++g) ECK(launch_forces_batch(c0->prec, e->fbb[e->flip][g], false, e->stream));
     ECK(cudaEventRecord(ev[1], e->stream));
     for (int r = 0; r < reps; ++r)
         for (int g = 0; g < G; ++g) {

@@ -665,11 +665,12 @@ __global__ void __launch_bounds__(kForceThreads) k_forces(const MarkerArgs a, co
 // (four blocks per SM: the batch's thousands of blocks are limited by how many
 // fit, not by one block's latency)
 template <typename C>
-__global__ void __launch_bounds__(kForceThreads, 4) k_forces_batch(const __grid_constant__ MarkerBatch b) {
+__global__ void __launch_bounds__(kForceThreads, 4)
+    k_forces_batch(const __grid_constant__ MarkerBatch b, const bool settle) {
     __shared__ MarkerArgs s_a;
     const int m = marker_member(b, blockIdx.x);
     stage_args(&s_a, b.args + m);
-    forces_unit<C>(s_a, blockIdx.x - b.off[m], b.settle != 0);
+    forces_unit<C>(s_a, blockIdx.x - b.off[m], settle);
 }
 
 // the end of a launch sequence: the last step's bond decisions, one block per
@@ -754,12 +755,12 @@ cudaError_t launch_forces(lbib_precision prec, const MarkerArgs& a, bool settle,
                          chained, a, settle);
 }
 
-cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, cudaStream_t s, bool chained) {
+cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, bool settle, cudaStream_t s, bool chained) {
     if (b.n < 1 || b.n > kBatchMax) return cudaErrorInvalidValue;
     const int nunits = b.off[b.n];
     if (nunits <= 0) return cudaSuccess;
     return launch_kernel(is_f64(prec) ? k_forces_batch<double> : k_forces_batch<float>, nunits, kForceThreads, 0, s,
-                         chained, b);
+                         chained, b, settle);
 }
 
 cudaError_t launch_settle(const MarkerArgs& a, cudaStream_t s) {

@@ -295,14 +295,14 @@ __device__ __forceinline__ int batch_member(const int* off, int n, int b) {
     }
     return lo;
 }
-// fused kernel: the members' arguments themselves are parameters (192 B each)
+// fused kernel: the members' arguments themselves are parameters
 struct LbBatch {
     int n;
     int off[kBatchMax + 1];     // row tiles: first block of each member; persistent form: first segment
     int tiles_x[kBatchMax];     // row tiles: tiles per row; persistent form: segments per row
     LbArgs a[kBatchMax];
 };
-// marker kernels: the members' arguments (744 B each) stay in global memory
+// marker kernels: the members' arguments stay in global memory
 // block -> member for the first kBlockTable blocks of a launch (one parameter
 // load where a search over off[] would take several dependent ones)
 constexpr int kBlockTable = 8192;
@@ -311,7 +311,6 @@ struct MarkerBatch {
     int n;
     int off[kBatchMax + 1];     // first block of each member's units
     const MarkerArgs* args;     // [n]
-    int settle;                 // force kernel: settle the previous step's bond decisions
     unsigned char member[kBlockTable];  // member of block b < min(off[n], kBlockTable)
 };
 __device__ __forceinline__ int marker_member(const MarkerBatch& b, int blk) {
@@ -402,7 +401,8 @@ cudaError_t launch_settle_batch(const MarkerArgs* args, int n, cudaStream_t s);
 cudaError_t launch_advance(lbib_precision prec, const MarkerArgs& a, cudaStream_t s, bool chained = false);
 // batched marker kernels of up to kBatchMax contexts (b.off[b.n] blocks); the
 // advance blocks have `threads` threads (the widest member's)
-cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, cudaStream_t s, bool chained = false);
+cudaError_t launch_forces_batch(lbib_precision prec, const MarkerBatch& b, bool settle, cudaStream_t s,
+                                bool chained = false);
 cudaError_t launch_advance_batch(lbib_precision prec, bool dyn, const MarkerBatch& b, int threads, cudaStream_t s,
                                  bool chained = false);
 cudaError_t launch_seg_boxes(lbib_precision prec, const MarkerArgs& a, cudaStream_t s);
