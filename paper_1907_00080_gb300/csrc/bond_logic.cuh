@@ -56,12 +56,13 @@ __device__ __forceinline__ unsigned long long bond_draw(const MarkerArgs& a, lon
 }
 __device__ __forceinline__ double uniform_of(unsigned long long k) { return (double)k * 0x1.0p-53; }
 // k 2^-53 < t and k 2^-53 > t for an FP32 threshold t < 2: exact (t 2^53 is a
-// scaling by a power of two), without the slow FP64 pipe
+// scaling by a power of two), without the slow FP64 pipe; neither for NaN
+// (0 times an overflow in the FP32 probability: the FP64 one decides)
 __device__ __forceinline__ bool draw_below(unsigned long long k, float t) {
     return t > 0.f && k < __float2ull_ru(t * 0x1.0p53f);
 }
 __device__ __forceinline__ bool draw_above(unsigned long long k, float t) {
-    return !(t >= 0.f) || k > __float2ull_rd(t * 0x1.0p53f);
+    return t < 0.f || (t >= 0.f && k > __float2ull_rd(t * 0x1.0p53f));
 }
 
 // forward (formation) and reverse (rupture) probabilities per step, FP64
