@@ -247,8 +247,9 @@ extern "C" lbib_status lbib_create(const lbib_lattice* lat, double tau, const do
             return LBIB_E_OOM;
         }
     }
-    e = cudaMalloc(&c->ux, N * c->cmp_elem);
-    if (e == cudaSuccess) e = cudaMalloc(&c->uy, N * c->cmp_elem);
+    const size_t u_bytes = (N + c->nx) * c->cmp_elem;  // and a row of zeros (interp_vertex)
+    e = cudaMalloc(&c->ux, u_bytes);
+    if (e == cudaSuccess) e = cudaMalloc(&c->uy, u_bytes);
     c->n_partials = 1024;
     if (e == cudaSuccess) e = cudaMalloc(&c->partials, sizeof(double) * c->n_partials);
     if (e == cudaSuccess) e = cudaMalloc(&c->dscalar, sizeof(double) * 8);
@@ -258,8 +259,8 @@ extern "C" lbib_status lbib_create(const lbib_lattice* lat, double tau, const do
         lbib_destroy(c);
         return LBIB_E_OOM;
     }
-    e = cudaMemsetAsync(c->ux, 0, N * c->cmp_elem, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->uy, 0, N * c->cmp_elem, c->stream);
+    e = cudaMemsetAsync(c->ux, 0, u_bytes, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->uy, 0, u_bytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_step, 0, 2 * sizeof(long long), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = init_populations(c);

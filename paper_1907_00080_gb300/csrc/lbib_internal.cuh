@@ -4,8 +4,9 @@
 //   populations  two buffers A/B, [9][NY][NX] of the storage type, x fastest;
 //                each holds the post-collision deviations d*_i = f*_i - w_i of
 //                one step (pull scheme: the fused kernel streams while reading)
-//   u field      ux, uy [NY][NX] of the compute type, written by the fused
-//                kernel only at nodes that IB stencils touch
+//   u field      ux, uy [NY + 1][NX] of the compute type, written by the fused
+//                kernel only at nodes that IB stencils touch; the row after the
+//                lattice's last stays zero
 //   markers      X^n, X^{n-1} as interleaved (x, y) doubles; F^n, U^n, the nine
 //                shape-function weights and the stencil origin per vertex
 //   IB force     two fixed-point (int64 x 2) per-node fields alternating with the

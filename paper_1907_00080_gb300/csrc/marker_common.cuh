@@ -328,9 +328,11 @@ __device__ __forceinline__ Shape<C> load_shape(const MarkerArgs& a, int v) {
     s.j0 = o.y;
     return s;
 }
-// (every node is read, rows outside the walls at the nearest row with their
-// weight 0: a branch per row made three round trips of one, 3400 cycles of the
-// advance kernel's chain)
+// (every node is read, rows outside the walls at the row of zeros after the
+// field's last: a branch per row made three round trips of one, 3400 cycles of
+// the advance kernel's chain.  The nearest fluid row would not do: for a marker
+// beyond a wall no stencil flagged it, and what an earlier step left there, not
+// finite perhaps, does not vanish by a weight of 0.)
 template <typename C>
 __device__ __forceinline__ void interp_vertex(const MarkerArgs& a, const Shape<C>& s, C& Ux, C& Uy) {
     const C* ux = static_cast<const C*>(a.ux);
@@ -344,7 +346,7 @@ __device__ __forceinline__ void interp_vertex(const MarkerArgs& a, const Shape<C
         i[q] = i[q] < 0 ? i[q] + a.nx : (i[q] >= a.nx ? i[q] - a.nx : i[q]);
         int j = s.j0 + q - 1;
         in[q] = !a.walls || (j >= 0 && j < a.ny);
-        j = a.walls ? min(max(j, 0), a.ny - 1) : (j < 0 ? j + a.ny : (j >= a.ny ? j - a.ny : j));
+        j = a.walls ? (in[q] ? j : a.ny) : (j < 0 ? j + a.ny : (j >= a.ny ? j - a.ny : j));
         row[q] = (size_t)j * a.nx;
     }
     C u[9], v[9];
