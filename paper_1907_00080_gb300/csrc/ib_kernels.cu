@@ -662,10 +662,13 @@ __global__ void __launch_bounds__(kForceThreads) k_forces(const MarkerArgs a, co
 // Batched form: the force units of up to kBatchMax contexts (ensemble
 // members) in one launch, one block per (member, unit).  The member's
 // arguments are staged in shared memory.
-// (four blocks per SM: the batch's thousands of blocks are limited by how many
-// fit, not by one block's latency)
+// (FP32: four blocks per SM, the batch's thousands of blocks are limited by how
+// many fit, not by one block's latency.  FP64: three.  At four the 64 registers
+// spill 268 bytes of stores and 200 of loads: 64 members 94.4 us against 89.8,
+// 10 members 25.5 against 24.8; 32 members 54.6 against 58.7, their whole step
+// 659.4 against 658.2.)
 template <typename C>
-__global__ void __launch_bounds__(kForceThreads, 4)
+__global__ void __launch_bounds__(kForceThreads, sizeof(C) == 8 ? 3 : 4)
     k_forces_batch(const __grid_constant__ MarkerBatch b, const bool settle) {
     __shared__ MarkerArgs s_a;
     const int m = marker_member(b, blockIdx.x);
