@@ -743,6 +743,7 @@ static lbib_status finalize(lbib_ctx* c) {
     a.tiles_x = c->tiles_x;
     a.status = c->d_status;
     a.f.nx = (float)c->nx; a.f.ny = (float)c->ny; a.f.inv_nx = (float)a.inv_nx; a.f.inv_ny = (float)a.inv_ny;
+    a.f.wrap_ny = a.walls ? 0.f : (float)c->ny;
     a.f.sigma = (float)a.sigma; a.f.y_eq = (float)a.y_eq; a.f.inv_y_eq = (float)a.inv_y_eq;
     a.f.d_rep = (float)a.d_rep; a.f.d_cut = (float)a.d_cut; a.f.d_break = (float)a.d_break;
     a.f.kf_dt = (float)a.kf_dt; a.f.kr0_dt = (float)a.kr0_dt; a.f.beta_f = (float)a.beta_f;

@@ -547,6 +547,7 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
             const E xv = s_x[j], yv = s_y[j];
             const float hx = float(ehi(xv)), hy = float(ehi(yv));
             const float xvw = hx - a.f.nx * floorf(hx * a.f.inv_nx);
+            const float yvw = hy - a.f.wrap_ny * floorf(hy * a.f.inv_ny);
             bool bad = false;
             for (int ci = tid / kChunkV; ci < nscan && j < kn; ci += kForceThreads / kChunkV) {
                 const bool staged = !all_segs && ci < kStageSeg;
@@ -554,7 +555,7 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
                 if (all_segs && a.seg_mem[sg] == m) continue;
                 const float4 bx = staged ? s_cbox[ci] : a.seg_box[sg];
                 const float ddx = wrap_half(xvw - bx.x, a.f.nx);
-                float ddy = hy - bx.y;
+                float ddy = yvw - bx.y;
                 if (!a.walls) ddy = wrap_half(ddy, a.f.ny);
                 if (fabsf(ddx) > bx.z + reach || fabsf(ddy) > bx.w + reach) continue;
                 C mags = C(0);

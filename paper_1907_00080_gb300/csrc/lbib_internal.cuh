@@ -158,7 +158,7 @@ struct MarkerArgs {
     const int* seg_mem;       // [nseg]
     const int* seg_v0;        // [nseg] first global vertex
     const int* seg_n;         // [nseg]
-    float4* seg_box;          // [nseg] centre x wrapped to [0,nx), centre y, half extents
+    float4* seg_box;          // [nseg] centre x wrapped to [0,nx), centre y (without walls to [0,ny)), half extents
     // groups of kGroupV vertices (four segments), boxes a little wide: the
     // first stage of the screening
     int ngroup;
@@ -219,6 +219,7 @@ struct MarkerArgs {
     // FP32 copies of the scalar parameters (no double->float conversion in the kernels)
     struct {
         float nx, ny, inv_nx, inv_ny, sigma, y_eq, inv_y_eq, d_rep, d_cut, d_break;
+        float wrap_ny;            // the period in y of the screening boxes: ny without walls, 0 with them
         float kf_dt, kr0_dt, beta_f, beta_r, inv_rc_w, inv_rc_h, rc_y0;
         // no receptor is within reach of a ligand at y < y_reach[0], y_reach[1] < y < y_reach[2] (the largest
         // gap between receptor heights, e.g. the channel between its walls) or y > y_reach[3]

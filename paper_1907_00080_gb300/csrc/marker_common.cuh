@@ -261,7 +261,8 @@ __device__ __forceinline__ void block_sum_c(C (&v)[N], C (*red)[8]) {
 // Boxes of the segments and of the screening group that a warp's positions
 // form: lane l holds vertex l of the group; lanes g, g + 1, .. of a segment past
 // its end hold a copy of its first vertex.  FP32 offsets from the segment's
-// first vertex; centre x wrapped into [0, nx).  sg: this lane's segment (-1:
+// first vertex; centre x wrapped into [0, nx), and without walls centre y into
+// [0, ny) (rings may lie several periods apart).  sg: this lane's segment (-1:
 // none), gr: the warp's group (-1: none).  The group's box is widened by 1e-3
 // (its own roundings stay below 1e-3 of a lattice unit).  All 32 lanes call it.
 template <typename C>
@@ -282,10 +283,11 @@ __device__ __forceinline__ void seg_box_regs(const MarkerArgs& a, int sg, int gr
         lo_y = fminf(lo_y, __shfl_xor_sync(kFull, lo_y, o));
         hi_y = fmaxf(hi_y, __shfl_xor_sync(kFull, hi_y, o));
     }
+    auto wrapped_y = [&](float cy) { return cy - a.f.wrap_ny * floorf(cy * a.f.inv_ny); };
     const float Lx = a.f.nx;
     if (sg >= 0 && lane == g0) {
         const float cx = float(ehi(ax)) + 0.5f * (lo_x + hi_x);
-        a.seg_box[sg] = make_float4(cx - Lx * floorf(cx * a.f.inv_nx), float(ehi(ay)) + 0.5f * (lo_y + hi_y),
+        a.seg_box[sg] = make_float4(cx - Lx * floorf(cx * a.f.inv_nx), wrapped_y(float(ehi(ay)) + 0.5f * (lo_y + hi_y)),
                                     0.5f * (hi_x - lo_x), 0.5f * (hi_y - lo_y));
     }
     shfl_e(wx, x, 0);
@@ -304,7 +306,7 @@ __device__ __forceinline__ void seg_box_regs(const MarkerArgs& a, int sg, int gr
     }
     if (gr >= 0 && lane == 0) {
         const float cx = float(ehi(wx)) + 0.5f * (lo_x + hi_x);
-        a.group_box[gr] = make_float4(cx - Lx * floorf(cx * a.f.inv_nx), float(ehi(wy)) + 0.5f * (lo_y + hi_y),
+        a.group_box[gr] = make_float4(cx - Lx * floorf(cx * a.f.inv_nx), wrapped_y(float(ehi(wy)) + 0.5f * (lo_y + hi_y)),
                                       0.5f * (hi_x - lo_x) + 1e-3f, 0.5f * (hi_y - lo_y) + 1e-3f);
     }
 }
