@@ -222,7 +222,8 @@ __device__ __forceinline__ void shape_functions(const MarkerArgs& a, E xv, E yv,
 // Eq. repFor screening by one warp, in two stages: groups (32 vertices) of
 // other membranes whose box comes within d_rep of this chunk's box (the union
 // of its one or two groups' boxes), and of those the segments.  Hits join the
-// block's candidate list in any order (order_candidates).
+// block's candidate list in any order: the repulsion sums are over integers, and
+// a pair rounds the same whether its segment is staged, listed or just walked.
 // The groups cut the boxes that every block reads to a quarter (64 instead of
 // 228 on the 640 x 160 capillary, one pass of the loop below).
 struct Candidates {
@@ -285,32 +286,6 @@ __device__ __forceinline__ void screen_segments(const MarkerArgs& a, int m, int 
     }
 }
 
-// Candidates beyond the staging space, all threads of the block: the list in
-// ascending order, its first kStageSeg staged.  A staged pair and a listed one
-// round differently (offsets from the segment's anchor, or a difference of two
-// positions), so which segments are staged must not depend on the order in
-// which the screening's lanes found them; up to kStageSeg hits are all staged
-// and more than kMaxCand all walked, in any order.  (A thread ranks its hit
-// against the others; the blocks that come here have 48 segments and more
-// within range, and no other block pays for it.)
-__device__ __forceinline__ void order_candidates(const MarkerArgs& a, int ncand, const Candidates& s_c) {
-    static_assert(kMaxCand <= kForceThreads, "one candidate per thread");
-    const int tid = threadIdx.x;
-    const int sg = s_c.seg[tid < ncand ? tid : 0];
-    int rank = 0;
-    for (int q = 0; q < ncand; ++q) rank += s_c.seg[q] < sg ? 1 : 0;
-    __syncthreads();
-    if (tid < ncand) {
-        s_c.seg[rank] = sg;
-        if (rank < kStageSeg) {
-            s_c.v0[rank] = a.seg_v0[sg];
-            s_c.nv[rank] = a.seg_n[sg];
-            s_c.box[rank] = a.seg_box[sg];
-        }
-    }
-    __syncthreads();
-}
-
 // One block per work unit (a chunk of up to kChunkV consecutive vertices of one
 // membrane).  The kernel is a chain of dependent loads and FP32 divisions and
 // square roots, so the parts of a vertex's force go to different warps and
@@ -367,7 +342,6 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
     __shared__ __align__(16) C s_cox[kStageSeg][kSegV], s_coy[kStageSeg][kSegV];
     __shared__ int s_cn[kStageSeg], s_cv0[kStageSeg];
     const Rest<C>* rest = static_cast<const Rest<C>*>(a.rest);
-    const Candidates cand{&s_ncand, s_cand, s_cv0, s_cn, s_cbox};
     // (with dynamic particles the predecessor is the hydrodynamic kernel, which
     // started after the positions were complete: its results are waited for
     // where they are used)
@@ -467,7 +441,8 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
         if (lane == 0) s_ncand = 0;
         __syncwarp();
         if (!a.has_dyn) dep_wait();
-        if (a.nmem > 1) screen_segments(a, m, own0, kn, lane, cand);
+        if (a.nmem > 1)
+            screen_segments(a, m, own0, kn, lane, Candidates{&s_ncand, s_cand, s_cv0, s_cn, s_cbox});
     } else if (wid == 5) {
         if (!halo_here && lane < 2) {
             // the halo vertices k0 - 1 (slot 0) and k0 + kn (slot kn + 1)
@@ -512,7 +487,6 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
     {
         const int ncand = s_ncand;
         const bool all_segs = ncand > kMaxCand;  // list overflow: screen every segment
-        if (ncand > kStageSeg && !all_segs) order_candidates(a, ncand, cand);
         if (ncand > 0) {
             // Eq. repFor against vertices of other membranes closer than d_rep, over
             // (candidate segment, vertex) pairs; the magnitudes of each vertex are
@@ -578,13 +552,17 @@ __device__ __forceinline__ void forces_unit(const MarkerArgs& a, int unit, bool 
                         if (d < drep) mags += c_rep * sqrt(C(1) / (d * d * d * d * d));
                     }
                 } else {
+                    // (by the offsets from the anchor too)
                     const int nb = a.seg_n[sg], b0 = a.seg_v0[sg];
+                    E xa, ya;
+                    load_pos<C>(a, b0, xa, ya);
+                    const C dxa = etoc(ewrap(esub(xv, xa), par<C>(a.nx, a.f.nx), par<C>(a.inv_nx, a.f.inv_nx)));
+                    C dya = etoc(esub(yv, ya));
+                    if (!a.walls) dya = etoc(ewrap(esub(yv, ya), par<C>(a.ny, a.f.ny), par<C>(a.inv_ny, a.f.inv_ny)));
                     for (int g = 0; g < nb; ++g) {
                         E xb, yb;
                         load_pos<C>(a, b0 + g, xb, yb);
-                        const C dx = etoc(ewrap(esub(xv, xb), par<C>(a.nx, a.f.nx), par<C>(a.inv_nx, a.f.inv_nx)));
-                        C dy = etoc(esub(yv, yb));
-                        if (!a.walls) dy = etoc(ewrap(esub(yv, yb), par<C>(a.ny, a.f.ny), par<C>(a.inv_ny, a.f.inv_ny)));
+                        const C dx = dxa - etoc(esub(xb, xa)), dy = dya - etoc(esub(yb, ya));
                         const C d = sqrt(dx * dx + dy * dy);
                         if (d < drep) mags += c_rep * sqrt(C(1) / (d * d * d * d * d));
                     }

@@ -1,12 +1,12 @@
-"""Repulsion of a block with 49 to 256 candidate segments: which of them are
-staged depends on the segments alone, not on the order in which they were found.
+"""Repulsion of a block with 49 candidate segments and more, of which 48 are staged,
+up to 256 listed, and all walked beyond that: a pair's force is the same bits on each
+way, so that it does not matter in which order the segments were found.
 
 A ring of 24 vertices, the first 40 vertices of a second ring within d_rep of it.
 The other vertices of the second ring, out of range of every vertex of the first,
 either lie inside the first ring (its block then has all of their segments as
 candidates) or far away (the block has five candidates, all staged).  The pairs in
-range are the same and are the staged ones both times (the lowest segments), so
-the first ring's forces have to be the same bits."""
+range are the same, so the first ring's forces have to be the same bits."""
 import numpy as np
 import pytest
 
@@ -34,8 +34,8 @@ def first_forces(wl):
 
 
 @pytest.mark.parametrize("prec", ["f64", "f32"])
-@pytest.mark.parametrize("n", [384, 400, 1000, 2048])  # 48, 50, 125 and 256 candidates
-def test_staged_segments(n, prec):
+@pytest.mark.parametrize("n", [384, 400, 1000, 2048, 2056])  # 48, 50, 125, 256 and 257 candidates
+def test_pairs_in_range(n, prec):
     far, near = (first_forces(rings(n, prec, k)) for k in (False, True))
     assert np.max(np.abs(far)) > 0
     assert np.array_equal(far, near)
@@ -43,7 +43,7 @@ def test_staged_segments(n, prec):
 
 @pytest.mark.parametrize("prec,tiling", [("f64", (2, 1)), ("f32", (2, 0)), ("f32", (4, 1))])
 def test_batched_members_match_single_runs(prec, tiling):
-    wls = [rings(n, prec, True, nx=128) for n in (400, 1000, 2048)]
+    wls = [rings(n, prec, True, nx=128) for n in (400, 1000, 2056)]
     ens = lbib.Ensemble(wls, precision=prec, tiling=tiling)
     assert ens.form == 1
     ens.step(5)
