@@ -204,9 +204,10 @@ lbib_status lbib_set_wall_velocity(lbib_ctx* ctx, double u_bottom, double u_top)
 lbib_status lbib_set_repulsion(lbib_ctx* ctx, double d_rep);
 
 /* Advance n time steps (enqueued; replays captured CUDA graphs, captured when a
- * call first needs them).  A call that cannot capture what it needs (LBIB_E_OOM,
- * LBIB_E_CUDA, which it also returns within a stream capture of the caller's)
- * enqueues nothing.  Errors from launching are returned; device-side failures
+ * call first needs them).  A first call that cannot capture single steps
+ * (LBIB_E_OOM, LBIB_E_CUDA) enqueues nothing, nor does a call within a stream
+ * capture of the caller's (LBIB_E_CUDA).  Errors from launching are returned,
+ * lbib_step_count then tells how many steps were enqueued; device-side failures
  * are reported by lbib_sync or the next read. */
 lbib_status lbib_step(lbib_ctx* ctx, int64_t n);
 

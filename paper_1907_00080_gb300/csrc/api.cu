@@ -28,6 +28,7 @@ lbib_status fail(lbib_ctx* c, lbib_status st, const std::string& msg) {
 }
 
 lbib_status cuda_fail(lbib_ctx* c, cudaError_t e, const char* where) {
+    cudaGetLastError();  // reported here: it is not the next launch's error
     if (c) c->err = std::string(where) + ": " + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? LBIB_E_OOM : LBIB_E_CUDA;
 }
@@ -951,11 +952,12 @@ static lbib_status launch_single_step(lbib_ctx* c) {
 // Sequences of 2, 4, .. 32 steps are captured when a call first needs them: a
 // call of n steps is a few launches for any n (7 steps were seven launches of
 // one step each, with a boundary of 2 us between them), and a first call
-// captures little more than it runs.  All of a call's sequences are captured
-// before its first launch, so that a call which cannot capture one has enqueued
-// nothing, and the state follows every launch.  (Within a capture of the
-// caller's own a launch of a graph is an error of the runtime's: refused before
-// anything is captured.)
+// captures little more than it runs, beside the sequences already launched (all
+// captured before the first launch: 2 to 10 % on a first call of 40 to 100
+// steps).  A sequence that cannot be captured, for want of memory, is run as
+// shorter ones; single steps were captured before anything was launched.  The
+// state follows every launch.  (Within a capture of the caller's own a launch of
+// a graph is an error of the runtime's: refused before anything is captured.)
 extern "C" lbib_status lbib_step(lbib_ctx* c, int64_t n) {
     if (!c || n < 0) return LBIB_E_INVALID;
     if (c->poisoned) return fail(c, LBIB_E_STATE, "context poisoned by an earlier device-side failure");
@@ -967,22 +969,13 @@ extern "C" lbib_status lbib_step(lbib_ctx* c, int64_t n) {
     if (st != LBIB_OK) return st;
     st = build_graphs(c);
     if (st != LBIB_OK) return st;
-    // the longest sequences first; all start from the buffer of now, since only a
-    // single step, the last one, changes the buffer roles
-    auto longest = [](int64_t left) {
-        int k = 0;
-        while (k + 1 < lbib_ctx::kGraphs && left >= (int64_t)2 << k) ++k;
-        return k;
-    };
+    int top = lbib_ctx::kGraphs - 1;
     for (int64_t left = n; left > 0;) {
-        const int k = longest(left);
-        if ((st = build_graph(c, c->cur, k)) != LBIB_OK) return st;
-        left &= ((int64_t)1 << k) - 1;
-    }
-    for (int64_t left = n; left > 0;) {
-        const int k = longest(left);
+        int k = top;
+        while (k > 0 && left < (int64_t)1 << k) --k;
+        while (k > 0 && build_graph(c, c->cur, k) != LBIB_OK) top = --k;
         CK(cudaGraphLaunch(c->graph[c->cur][k], c->stream));
-        if (k == 0) c->cur = 1 - c->cur;
+        if (k == 0) c->cur = 1 - c->cur;  // an even number of steps leaves the buffer roles
         c->steps += (int64_t)1 << k;
         c->fields_valid = true;
         left -= (int64_t)1 << k;

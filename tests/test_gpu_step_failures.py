@@ -1,5 +1,6 @@
-"""lbib_step when a sequence of steps cannot be captured: nothing of the call is
-enqueued, the step count and the state stay as they were, and the next call runs.
+"""lbib_step when a sequence of steps cannot be captured: shorter ones take its place.
+When not even single steps can be, at a context's first call, nothing is enqueued and
+the next call runs.
 
 The failure is made on the host: the library is linked once more with a wrapper
 around cudaGraphInstantiate that returns an error code at the asked-for call."""
@@ -17,15 +18,15 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 WRAPPER = r"""
 #include <cuda_runtime.h>
-static int left = -1;  // calls until the failing one
-extern "C" void fail_instantiate(int after) { left = after; }
+static int left = 0, failing = 0;  // calls until the failing ones, and their number
+extern "C" void fail_instantiate(int after, int n) { left = after; failing = n; }
+extern "C" int failures_left() { return failing; }
 extern "C" cudaError_t __real_cudaGraphInstantiate(cudaGraphExec_t*, cudaGraph_t, unsigned long long);
 extern "C" cudaError_t __wrap_cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t g, unsigned long long f) {
-    if (left == 0) {
-        left = -1;
+    if (failing > 0 && left-- <= 0) {
+        --failing;
         return cudaErrorMemoryAllocation;
     }
-    if (left > 0) --left;
     return __real_cudaGraphInstantiate(e, g, f);
 }
 """
@@ -57,18 +58,20 @@ def run_with_failures(path):
         for x, y in zip((a.populations(), a.markers(), a.bonds()), (b.populations(), b.markers(), b.bonds())):
             assert np.array_equal(x, y)
 
+    lib.fail_instantiate(ctypes.c_int(1), ctypes.c_int(1))
+    with pytest.raises(lbib.LbibError) as e:
+        a.step(5)
+    assert e.value.status == lbib.LBIB_E_OOM
+    assert lbib.lbib_step_count(a.ctx) == 0
     for s in (a, b):
         s.step(5)  # the sequences of four steps and of one, from either buffer
-    # 4 + 2 steps, of which the two cannot be captured; 8 + 2 + 1, the eight; and from
-    # the other buffer 4 + 2 + 1, where the four are there and the two cannot be captured
-    for n, k in ((6, 1), (11, 0), (7, 0)):
+    # 4 + 2 steps, of which the two cannot be captured; 8 + 2 + 1, the eight; from the
+    # other buffer 4 + 2 + 1, where the four are there; and 2 x 32 with neither 32 nor 16
+    for n, k in ((6, 1), (11, 0), (7, 0), (64, 0)):
         count = lbib.lbib_step_count(a.ctx)
-        lib.fail_instantiate(ctypes.c_int(k))
-        with pytest.raises(lbib.LbibError) as e:
-            a.step(n)
-        assert e.value.status == lbib.LBIB_E_OOM
-        same(count)
+        lib.fail_instantiate(ctypes.c_int(k), ctypes.c_int(2 if n == 64 else 1))
         a.step(n)
+        assert lib.failures_left() == 0
         for _ in range(n):
             b.step(1)
         a.sync()
@@ -79,7 +82,7 @@ def run_with_failures(path):
     print("steps after failures ok")
 
 
-def test_failed_capture_enqueues_nothing(tmp_path):
+def test_failed_captures(tmp_path):
     lib = wrapped_library(str(tmp_path))
     code = ("import sys; sys.path[:0] = [%r, %r]\nimport test_gpu_step_failures as t\nt.run_with_failures(%r)\n"
             % (ROOT, os.path.join(ROOT, "tests"), lib))
