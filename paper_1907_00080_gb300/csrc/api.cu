@@ -315,7 +315,6 @@ extern "C" lbib_status lbib_add_membrane(lbib_ctx* c, const double* xy, int32_t 
     c->h_mem_lig_off.push_back(c->nlig);
     c->nv += n;
     c->nmem += 1;
-    c->max_mem_n = std::max(c->max_mem_n, n);
     if (membrane_id_out) *membrane_id_out = m;
     return LBIB_OK;
 }
@@ -492,15 +491,15 @@ static lbib_status finalize(lbib_ctx* c) {
     std::vector<int> fu, au, mem_au(nm + 1, 0);
     for (int m = 0; m < nm; ++m) {
         const int n = c->h_mem_n[m], off = c->h_mem_off[m], kind = c->h_mem_kind[m];
-        const int s0 = mem_seg_off[m], g0 = mem_group_off[m], ns = mem_seg_off[m + 1] - s0;
+        const int s0 = mem_seg_off[m], g0 = mem_group_off[m];
         mem_au[m] = (int)(au.size() / kUnitInts);
         for (int k0 = 0; k0 < n; k0 += kChunkV) {
             const int u = whole_ring(kind) ? -1 : (int)(au.size() / kUnitInts);
-            fu.insert(fu.end(), {m, k0, std::min(kChunkV, n - k0), off, n, kind, 0, u, s0, g0, ns, 0});
+            fu.insert(fu.end(), {m, k0, std::min(kChunkV, n - k0), off, n, kind, 0, u, s0, g0, 0, 0});
             if (!whole_ring(kind))
-                au.insert(au.end(), {m, k0, std::min(kChunkV, n - k0), off, n, kind, 0, 0, s0, g0, ns, 0});
+                au.insert(au.end(), {m, k0, std::min(kChunkV, n - k0), off, n, kind, 0, 0, s0, g0, 0, 0});
         }
-        if (whole_ring(kind)) au.insert(au.end(), {m, 0, n, off, n, kind, 0, 0, s0, g0, ns, 0});
+        if (whole_ring(kind)) au.insert(au.end(), {m, 0, n, off, n, kind, 0, 0, s0, g0, 0, 0});
     }
     // ligands of each advance unit (that of their element's first vertex), as
     // records {ligand, local index of its element's two vertices, 0}; an
@@ -737,7 +736,6 @@ static lbib_status finalize(lbib_ctx* c) {
     a.rc_nx = rc_nx; a.rc_ny = rc_ny; a.rc_w = rc_w; a.rc_h = rc_h; a.rc_y0 = rc_y0;
     a.inv_rc_w = 1.0 / rc_w; a.inv_rc_h = 1.0 / rc_h;
     a.inv_y_eq = c->bp.y_eq > 0 ? 1.0 / c->bp.y_eq : 0.0;
-    a.d_cut2 = (c->bp.d_cut * (1.0 + 1e-12)) * (c->bp.d_cut * (1.0 + 1e-12));
     a.sigma = c->bp.sigma; a.y_eq = c->bp.y_eq; a.d_cut = c->bp.d_cut; a.d_break = c->bp.d_break;
     a.kf_dt = c->bp.kf_dt; a.kr0_dt = c->bp.kr0_dt; a.beta_f = c->bp.beta_f; a.beta_r = c->bp.beta_r;
     a.seed = c->bp.seed; a.instance = c->bp.instance;
@@ -1992,7 +1990,6 @@ struct Snap {
     void* f = nullptr;
     double *X = nullptr, *Xp = nullptr;
     int *bond = nullptr, *owner = nullptr, *owner_cell = nullptr;
-    float4* seg_box = nullptr;
     long long* d_step = nullptr;
     long long step = 0;
 };
@@ -2006,7 +2003,6 @@ size_t snap_bytes(const lbib_ctx* c) {
     a.take<int>(nlig);
     a.take<int>(nrec);
     a.take<int>(nrec);
-    a.take<float4>(c->nseg);
     a.take<long long>(1);
     return a.used + 256;
 }
@@ -2021,7 +2017,6 @@ void snap_layout(const lbib_ctx* c, Snap& s) {
     s.bond = a.take<int>(nlig);
     s.owner = a.take<int>(nrec);
     s.owner_cell = a.take<int>(nrec);
-    s.seg_box = a.take<float4>(c->nseg);
     s.d_step = a.take<long long>(1);
 }
 
@@ -2040,7 +2035,6 @@ cudaError_t snap_copy(lbib_ctx* c, Snap& s, bool to_snap) {
     if ((e = cp(s.bond, c->bond[c->cur], 4 * nlig)) != cudaSuccess) return e;
     if ((e = cp(s.owner, c->ma.owner, 4 * nrec)) != cudaSuccess) return e;
     if ((e = cp(s.owner_cell, c->ma.owner_cell, 4 * nrec)) != cudaSuccess) return e;
-    if ((e = cp(s.seg_box, c->ma.seg_box, sizeof(float4) * c->nseg)) != cudaSuccess) return e;
     if ((e = cp(s.d_step, c->d_step + c->cur, 8)) != cudaSuccess) return e;
     if (!to_snap && (e = refresh_markers(c, c->stream)) != cudaSuccess) return e;
     if (to_snap) s.step = c->steps;

@@ -787,32 +787,20 @@ __global__ void __launch_bounds__(kBlock, ctas_per_sm(Geom<S, NPT>::SMEM))
     __shared__ ItemRef s_pos[kStages];
     stream_ws<S, NPT, WALLS>(ManyLattices<S, NPT>{b, s_args, s_pos});
 }
-template <typename S, int NPT, bool WALLS>
-__global__ void __launch_bounds__(kThreads) k_lb_stream_bar_batch(const __grid_constant__ LbBatch b) {
-    __shared__ LbArgs s_args[kStages];
-    __shared__ ItemRef s_pos[kStages];
-    stream_bar<S, NPT, WALLS>(ManyLattices<S, NPT>{b, s_args, s_pos});
-}
 
 // the producer-warp schedule for 16-bit storage, the barrier schedule otherwise
 // (measured on the 8192 x 2048 probe: FP32 npt 2 199 us vs 223 us; FP16 npt 4
-// 158 us vs 138 us)
-template <typename S>
-constexpr bool kWarpSpecialised = sizeof(S) == 2;
-// batches: the staging of a segment also copies its member's arguments, which
-// keeps the producer warp off the consumers' path in every storage type
-template <typename S>
-constexpr bool kBatchWarpSpecialised = true;
+// 158 us vs 138 us); batches: the staging of a segment also copies its member's
+// arguments, which keeps the producer warp off the consumers' path in every
+// storage type
+template <typename S, bool BATCH>
+constexpr bool kWarpSpecialised = BATCH || sizeof(S) == 2;
 
 template <typename S, int NPT, bool WALLS, bool BATCH>
 constexpr auto stream_kernel() {
-    if constexpr (BATCH) {
-        if constexpr (kBatchWarpSpecialised<S>) return k_lb_stream_ws_batch<S, NPT, WALLS>;
-        else return k_lb_stream_bar_batch<S, NPT, WALLS>;
-    } else {
-        if constexpr (kWarpSpecialised<S>) return k_lb_stream_ws<S, NPT, WALLS>;
-        else return k_lb_stream_bar<S, NPT, WALLS>;
-    }
+    if constexpr (BATCH) return k_lb_stream_ws_batch<S, NPT, WALLS>;
+    else if constexpr (kWarpSpecialised<S, false>) return k_lb_stream_ws<S, NPT, WALLS>;
+    else return k_lb_stream_bar<S, NPT, WALLS>;
 }
 
 template <typename S, int NPT, bool WALLS, bool BATCH>
@@ -820,8 +808,7 @@ cudaError_t prepare_t(int* grid) {
     auto kern = stream_kernel<S, NPT, WALLS, BATCH>();
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Geom<S, NPT>::SMEM);
     if (e != cudaSuccess) return e;
-    const bool ws = BATCH ? kBatchWarpSpecialised<S> : kWarpSpecialised<S>;
-    const int threads = ws ? kBlock : kThreads;
+    const int threads = kWarpSpecialised<S, BATCH> ? kBlock : kThreads;
     int occ = 0, dev = 0, nsm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, Geom<S, NPT>::SMEM)) != cudaSuccess)
         return e;
@@ -842,7 +829,7 @@ cudaError_t dispatch(bool prepare, bool walls, int grid, int* grid_out, const Lb
         if (batch) return walls ? prepare_t<S, NPT, true, true>(grid_out) : prepare_t<S, NPT, false, true>(grid_out);
         return walls ? prepare_t<S, NPT, true, false>(grid_out) : prepare_t<S, NPT, false, false>(grid_out);
     }
-    const int threads = (batch ? kBatchWarpSpecialised<S> : kWarpSpecialised<S>) ? kBlock : kThreads;
+    const int threads = (batch ? kWarpSpecialised<S, true> : kWarpSpecialised<S, false>) ? kBlock : kThreads;
     long long items;
     if (batch) {
         if (b->n < 1 || b->n > kBatchMax) return cudaErrorInvalidValue;

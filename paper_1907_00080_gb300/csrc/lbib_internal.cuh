@@ -202,7 +202,6 @@ struct MarkerArgs {
     int rc_nx, rc_ny;         // receptor grid
     double rc_w, rc_h, rc_y0; // cell size, y origin
     double inv_rc_w, inv_rc_h, inv_y_eq;
-    double d_cut2;            // (d_cut (1 + 1e-12))^2, a conservative pre-check
     double sigma, y_eq, d_cut, d_break, kf_dt, kr0_dt, beta_f, beta_r;
     uint64_t seed, instance;
     // spreading target of this step
@@ -259,12 +258,12 @@ struct HydroArgs {
 
 // ST_FIXRANGE: a spread force or a repulsion magnitude left the range of its
 // fixed-point accumulator (see clamp_fix)
-enum StatusBits { ST_NONFINITE = 1, ST_TILE_OVERFLOW = 2, ST_TIMEOUT = 4, ST_FIXRANGE = 8 };
+enum StatusBits { ST_NONFINITE = 1, ST_TIMEOUT = 4, ST_FIXRANGE = 8 };
 
 constexpr int kChunkV = 64;   // vertices per marker-kernel block (a multiple of 32)
 constexpr int kUnitInts = 12; // ints per work-unit record (three int4): {m, k0, kn, off} {n, kind, x, y} {first
-                              // segment, first group, segments, 0 of the membrane}; x, y: force units {0, advance
-                              // unit of the chunk or -1}, advance units {first ligand record, their number}
+                              // segment and group of the membrane, 0, 0}; x, y: force units {0, advance unit of
+                              // the chunk or -1}, advance units {first ligand record, their number}
 constexpr int kSegV = 8;      // vertices per repulsion-screening segment (divides kChunkV)
 constexpr int kGroupV = 32;   // vertices per screening group: a warp's (divides kChunkV)
 
@@ -469,7 +468,6 @@ struct lbib_ctx {
 
     // device marker state (allocated at finalize)
     bool finalized = false;
-    int max_mem_n = 0;
     int nseg = 0;
     void* dmem = nullptr;     // one arena for all marker / tile / bond arrays
     size_t dmem_bytes = 0;
