@@ -255,9 +255,9 @@ lbib_status lbib_diagnostics(lbib_ctx* ctx, double* mass, double* areas);
 /* ---------------------------------------------------------------- ensembles
  * A batch of independent simulations (e.g. a sweep over release positions,
  * capillary numbers and bond strengths on channels of different lengths)
- * advanced together, one CUDA graph launch per chunk of 16 steps or a single step.  The paper
- * runs its cases one by one; this is a throughput form only: every member
- * computes exactly what it computes alone with the same tiling (bitwise).
+ * advanced together, one CUDA graph launch per chunk of 16 steps or a single step.
+ * The paper runs its cases one by one; this is a throughput form only: every
+ * member computes exactly what it computes alone with the same tiling (bitwise).
  * Two forms, chosen at creation:
  *  - batched (lbib_ensemble_form = 1): when all members share the precision,
  *    the walls and the form and shape of the fused kernel (lbib_set_tiling:
@@ -536,10 +536,12 @@ lbib_status lbib_membrane_observables(lbib_ctx* ctx, double* out);
 lbib_status lbib_population_mass_noalloc(const double* f, int64_t n_nodes, double* mass, void* stream);
 
 /* Form and tile shape of the fused collide-stream kernel.  Must precede the
- * first step; 0,0 picks the default: for F32 and 16-bit storage the
- * persistent form when the two population buffers exceed 128 MB, for 16-bit
- * storage also from 2^20 nodes on (segments of 512 nodes), else a row-tile
- * shape.
+ * first step; 0,0 picks the default.  F64: row tiles.  F32: row tiles, but the
+ * persistent form (2, 0) while the two population buffers take 128 to 160 MB,
+ * and above that on lattices of more than 131,070 rows.  16-bit storage: row
+ * tiles below 2^21 nodes; from there on the persistent form, (4, 0) where the
+ * rows fill its segments of 1024 nodes to 70 % or the two buffers exceed 128 MB,
+ * else (2, 0).  Rows that are no multiple of 16 bytes of storage: row tiles.
  *  ty in 1..16: row tiles, vec consecutive x nodes per thread and ty rows per
  *    block; vec divides NX, with vec in {1,2} (F64), {1,2,4} (F32), {2,4,8}
  *    (16-bit storage).

@@ -115,10 +115,13 @@ void default_tiling(const lbib_ctx* c, int* vec, int* ty) {
     // enough bytes in flight with them at any size (us per step, row tiles 4,2 /
     // persistent 2,0: lattices without markers 3000 x 1000 33.4 / 37.5, 8192 x
     // 2048 173.6 / 213.0, 520 x 5000 31.2 / 56.1; with markers 8192 x 1024 101.5 /
-    // 106.0).  With the two population buffers a little above L2 (129 MB) the
-    // two come within 2 % with markers (2048 x 1024 33.95 / 34.2), and the
-    // persistent form stays there, and for lattices taller than two rows a
-    // block can cover.
+    // 106.0).  The persistent form is left where the two population buffers are a
+    // little above L2 (129 MB) and for lattices taller than two rows a block can
+    // cover.  Just above L2 it is no better: with markers even (2048 x 880 29.0 /
+    // 29.7, 2000 x 1000 33.2 / 33.2, 3072 x 640 31.9 / 31.6, 2048 x 1080 35.4 /
+    // 35.9), without them behind (19.9 / 21.3, 22.4 / 24.0, 21.7 / 22.6, 24.6 /
+    // 25.5), far behind where short rows leave its segments half empty (520 x
+    // 3800 24.2 / 42.7).
     // 16-bit storage moves half the bytes per instruction and needs the
     // persistent form's bulk copies beyond L2 (4096 x 2048 52 us at 4,0, 79-82
     // with row tiles) and from 2^21 nodes on (2048 x 1400 18.8 / 26.1; below,

@@ -64,7 +64,7 @@ __device__ __forceinline__ void lb_tile(const LbArgs& a, int bx, int by) {
     // (FP64, and one node a thread with markers: every node's own element of the
     // shifted directions is read straight away.  The off-vector elements and
     // their shuffles cost FP64 the registers that hide its pipe's latency,
-    // 60-member ensemble 1720 -> 1650 us per step, and the latency-bound small
+    // 60-member ensemble 1720 -> 1590 to 1620 us per step, and the latency-bound small
     // lattices their issue slots, capillary 12.1 -> 11.0 us; a 1501 x 333 lattice
     // without markers is faster with the aligned loads, 7.6 against 8.1 us)
     constexpr bool kDirect = (VEC == 1 && HAS_IB) || sizeof(S) == 8;

@@ -2,8 +2,9 @@
 //
 // The row-tile kernel (lb_kernels.cu) keeps its nine pulled populations in
 // registers, so the bytes it has in flight per SM are bounded by how many
-// warps fit: on large lattices it waits on DRAM latency.  This form decouples
-// the two: each CTA (one to three per SM, for the whole lattice) walks a strided
+// warps fit.  In FP32 that is enough at any size (default_tiling in api.cu);
+// 16-bit storage moves half the bytes with as many registers and waits on DRAM
+// latency on large lattices.  This form decouples the two: each CTA (one to three per SM, for the whole lattice) walks a strided
 // list of row segments of W = 256 * NPT nodes and streams, for every segment,
 // the nine source rows it pulls from into a 4-stage shared-memory ring with
 // cp.async.bulk copies that complete on an mbarrier.  While the threads

@@ -119,14 +119,16 @@ __device__ __forceinline__ EdgeProducts<C> edge_products(E xL, E yL, E xv, E yv,
 }
 
 // Enclosed area of a ring by the shoelace formula, summed in a fixed order, so
-// that every caller gets the same bits (the rest shape then has exactly its
-// rest area).
+// that every caller gets the same bits at the same state (the rest shape of a
+// ring of up to kDirectArea vertices then has exactly its rest area; a longer
+// ring's while X^{n-1} of its vertex 0 is the set-up's too).
 //
 // Rings of up to kDirectArea vertices: about vertex 0, by the 64 lanes of two
 // consecutive warps starting at `w0`: four sums, of the terms k with k / 32 mod
 // 4 = 0 .. 3 (lane l of sum s takes terms 32 s + l + 128 i in order, the lanes
-// are reduced by a fixed tree), added in order.  `red` holds 4 values; the result is valid in the first warp's lanes after
-// the named barrier `bar` (64 threads).
+// are reduced by a fixed tree), added in order.  `red` holds 4 values; the
+// result is valid in the first warp's lanes after the named barrier `bar` (64
+// threads).
 //
 // Longer rings: every block of the force kernel would walk the whole ring (27
 // blocks of 1700 vertices on the fine capillary, 9800 of their 18900 cycles).
