@@ -312,8 +312,15 @@ __device__ __forceinline__ void advance_unit(const MarkerArgs& a, int u) {
     }
 }
 
+// (Up to 128 registers, 100 in FP32.  Left to itself ptxas stops at 80, three
+// blocks of 256 threads, which a single run's few blocks never are on one SM;
+// what it then keeps in flight turned on unrelated edits: 640 x 160 capillary,
+// 100 steps from three starts, 1255 / 1095 / 1190 us in one build, 1440 / 1220 /
+// 1250 with eight bytes fewer in MarkerArgs, 1116 / 1136 / 1126 now.  Thousands
+// of units lose a little by the fewer blocks that fit: 2500 rings, a step 206.5
+// -> 207.1 us.)
 template <typename C, bool DYN>
-__global__ void __launch_bounds__(kAdvThreads) k_advance(const MarkerArgs a) {
+__global__ void __launch_bounds__(kAdvThreads, 2) k_advance(const MarkerArgs a) {
     advance_unit<C, DYN>(a, blockIdx.x);
 }
 
